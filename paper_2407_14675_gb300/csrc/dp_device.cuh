@@ -333,6 +333,20 @@ __device__ __forceinline__ unsigned long long sub2(unsigned long long a, unsigne
     return d;
 }
 
+__device__ __forceinline__ unsigned long long add2(unsigned long long a, unsigned long long b)
+{
+    unsigned long long d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+
+__device__ __forceinline__ unsigned long long mul2(unsigned long long a, unsigned long long b)
+{
+    unsigned long long d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+
 // The 16 corner values of a cell as differences to the node's value, ready
 // for the blend.  Corner x = 4 r + 2 v_r + v_t (bits of the cell corner) has
 // e0[x] at the lower mass node and de[x] = step to the upper mass node.

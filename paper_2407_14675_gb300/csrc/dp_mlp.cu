@@ -485,6 +485,351 @@ mlp_persistent_kernel(const bf16* __restrict__ A, int lda, const bf16* __restric
     if (warp == 0) tmem_dealloc(tmem, kTileN);
 }
 
+// The network's inference in one kernel: a CTA takes 128 rows at a time
+// through all four layers, so that no activation leaves the SM.  The 128 x 256
+// activations sit in shared memory (64 KB, the MMAs' core-matrix layout), the
+// accumulators in TMEM (256 columns), and the 256 x 256 weights of the two
+// hidden layers pass through a ring of four 8 KB slots, one K step of 16 each,
+// by bulk copies that one thread issues three steps ahead (128 KB a layer and
+// tile from L2, about 2.5 TB/s over the chip).  109 KB a CTA, so that two share
+// an SM and one's activations cover the other's MMAs.
+//
+// What bounds it: the exact-erf GELU, 768 a row and 33 instructions each with
+// its bias, rounding and store (9.4 ms of issue slots over the 13.8M nodes of
+// 61^4); 62 % of the issue slots are busy, the rest is both CTAs waiting for
+// MMAs at once.  14.9 ms over 61^4, where separate kernels for the inputs, the
+// first layer, each hidden layer, the output layer and the write, passing the
+// activations through memory, took 28.0 ms.  With a 32 KB slice of 64 columns
+// at a time copied by every thread and a block barrier per slice 17.9 ms; with
+// the ring's addresses formed in the issuing thread's loop 16.3 ms.
+//
+// Same arithmetic as the training step's kernels, in the same order: the
+// first layer's FMA chain, K accumulated in steps of 16 from 0, the output
+// layer's sums over groups of eight features combined by the tree a warp
+// shuffle gives (features 8 g .. 8 g + 7 are group g; groups g and g + 16, then
+// g and g + 8, ... are added).
+//
+// GRID: rows are the stored nodes of a grid, whose normalised coordinates
+// come from the table coord (4 x kCoordMax, per dimension), and the outputs
+// become the node's value M clamp(y_0, 0, 1) (0 on target nodes) and the code
+// of atan2(y_2, y_1); otherwise rows are x (rows x 4) and the outputs go to y
+// (rows x 3).
+constexpr int kInferThreads = 512;
+constexpr int kInferSlots = 4;                                     // ring of weight K steps
+constexpr int kInferStep = kH * 16 * 2;                            // bytes of one: 256 rows x 16 columns
+constexpr int kInferSteps = kH / 16;                               // per layer
+constexpr int kCoordMax = 1024;                                    // largest grid dimension
+constexpr int kInferSmemA = kTileM * kKC * 2, kInferSmemW = kInferSlots * kInferStep;
+constexpr int kInferSmemF = 4 * kH + kH + kH + kH + 3 * kH + 4;    // W1 (by input), b1, b2, b3, W4, b4
+constexpr int kInferSmem = kInferSmemA + kInferSmemW + (kInferSmemF + 9 * kTileM) * 4;
+
+struct InferGrid {
+    const float* coord;
+    double M;
+    void* V;
+    uint16_t* code;
+    int fp32;
+};
+
+// Weights of both hidden layers as the ring's steps: step s of a layer holds
+// columns 16 s .. 16 s + 15 as core matrices (8 rows x 16 bytes), row block rb
+// and K block kb at (rb * 2 + kb) * 128.  One thread per 16 bytes.
+__global__ void infer_weights_kernel(const bf16* __restrict__ W2, const bf16* __restrict__ W3,
+                                     uint4* __restrict__ out)
+{
+    const int v = blockIdx.x * blockDim.x + threadIdx.x;           // 2 x 16 x 512
+    const int layer = v >> 13, s = (v >> 9) & 15, rb = (v >> 4) & 31, kb = (v >> 3) & 1, row = rb * 8 + (v & 7);
+    out[v] = *reinterpret_cast<const uint4*>((layer ? W3 : W2) + (size_t)row * kH + s * 16 + kb * 8);
+}
+
+__global__ void coord_table_kernel(const Geo<double> g, Box4 nlo, Box4 nhi, float* __restrict__ coord)
+{
+    const int d = blockIdx.x, i = threadIdx.x;
+    if (i >= g.n[d]) return;
+    const double lo[4] = {nlo.x, nlo.y, nlo.z, nlo.w}, hi[4] = {nhi.x, nhi.y, nhi.z, nhi.w};
+    const double xd = g.lo[d] + (double)i * g.h[d];
+    coord[d * kCoordMax + i] = (float)(2.0 * (xd - lo[d]) / (hi[d] - lo[d]) - 1.0);
+}
+
+// GELU of a pair: gelu() of each, the plain multiplications and the addition
+// two at a time.
+__device__ __forceinline__ unsigned long long gelu2(unsigned long long z)
+{
+    float a, b;
+    unpack2(mul2(z, pack2(kInvSqrt2, kInvSqrt2)), a, b);
+    return mul2(mul2(z, pack2(0.5f, 0.5f)), add2(pack2(1.0f, 1.0f), pack2(erff(a), erff(b))));
+}
+
+// Eight consecutive floats of shared memory (16-byte aligned) as four pairs.
+__device__ __forceinline__ void lds8(const float* p, unsigned long long q[4])
+{
+    const ulonglong2 a = *reinterpret_cast<const ulonglong2*>(p), b = *reinterpret_cast<const ulonglong2*>(p + 4);
+    q[0] = a.x; q[1] = a.y; q[2] = b.x; q[3] = b.y;
+}
+
+template <bool GRID>
+__global__ void __launch_bounds__(kInferThreads, 2)
+mlp_infer_kernel(const __grid_constant__ Geo<double> g, const __grid_constant__ InferGrid ig,
+                 const float* __restrict__ x, const float* __restrict__ P, const unsigned char* __restrict__ Wsteps,
+                 int count, float* __restrict__ y, int* __restrict__ err, int polls)
+{
+    extern __shared__ __align__(1024) unsigned char smem[];
+    unsigned char* sA = smem;
+    unsigned char* sW = smem + kInferSmemA;
+    float* sW1 = reinterpret_cast<float*>(smem + kInferSmemA + kInferSmemW);     // 4 x 256, by input
+    float* sB1 = sW1 + 4 * kH;
+    float* sB2 = sB1 + kH;
+    float* sB3 = sB2 + kH;
+    float* sW4 = sB3 + kH;                                                       // 3 x 256, then b4
+    float* sT = sW4 + 3 * kH + 4;                                                // 3 outputs x parts 1..3 x 128
+    __shared__ unsigned tmem_slot;
+    __shared__ int s_fail;
+    __shared__ __align__(8) unsigned long long mbar, full[kInferSlots], empty[kInferSlots];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int r = tid & (kTileM - 1), part = tid >> 7;             // row (TMEM lane), column part 0..3
+
+    for (int i = tid; i < 4 * kH; i += kInferThreads) sW1[(i & 3) * kH + (i >> 2)] = P[kOffW1 + i];
+    for (int i = tid; i < kH; i += kInferThreads) {
+        sB1[i] = P[kOffB1 + i];
+        sB2[i] = P[kOffB2 + i];
+        sB3[i] = P[kOffB3 + i];
+    }
+    for (int i = tid; i < 3 * kH + 3; i += kInferThreads) sW4[i] = P[kOffW4 + i];
+    if (warp == 0) tmem_alloc(&tmem_slot, kH);
+    if (tid == 0) {
+        s_fail = 0;
+        mbar_init(&mbar);
+        for (int b = 0; b < kInferSlots; ++b) {
+            mbar_init(&full[b]);
+            mbar_init(&empty[b]);
+        }
+    }
+    fence_before_sync();
+    __syncthreads();
+    fence_after_sync();
+    const unsigned tmem = tmem_slot;
+    constexpr unsigned idesc = umma_idesc_bf16(kTileM, kTileN);
+    const int tiles = (int)(((long long)count + kTileM - 1) / kTileM);
+
+    // The ring: step s of either layer sits in slot s mod 4 (a layer has 16
+    // steps, so slots and phase parities repeat layer by layer and are
+    // constants of the unrolled loop).  Thread 0 issues the copies and the
+    // MMAs; `left` counts the steps of this CTA not yet requested, `next` is
+    // the next one's address.
+    const int my_tiles = (tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
+    long long left = 2LL * kInferSteps * my_tiles;
+    const unsigned char* next = Wsteps;
+    auto load = [&](int b) {
+        mbar_expect_bytes(&full[b], kInferStep);
+        bulk_copy(sW + b * kInferStep, next, kInferStep, &full[b]);
+        next += kInferStep;
+        if (next == Wsteps + 2 * kInferSteps * kInferStep) next = Wsteps;
+        --left;
+    };
+    if (tid == 0) {
+#pragma unroll
+        for (int b = 0; b < kInferSlots; ++b) load(b);   // a layer has more steps than the ring
+    }
+    const unsigned long long adesc = umma_desc(smem_u32(sA), 128, kKC / 8 * 128);
+    const unsigned long long bdesc = umma_desc(smem_u32(sW), 128, 256);
+
+    int phase = 0;
+    bool first = true;
+    // One hidden layer: acc = sA W^T.  False after a wait that gave up.
+    auto layer = [&]() -> bool {
+        fence_async_smem();
+        fence_before_sync();
+        __syncthreads();
+        if (tid == 0) {
+            fence_after_sync();
+            bool fine = true;
+#pragma unroll
+            for (int s = 0; s < kInferSteps; ++s) {
+                const int b = s % kInferSlots, p = (s + kInferSteps - 1) % kInferSteps;   // p: the step before
+                fine = fine && mbar_wait(&full[b], (s / kInferSlots) & 1, kWaitPolls);
+                if (fine) {
+#pragma unroll
+                    for (int h = 0; h < kH / kTileN; ++h)
+                        umma_bf16(tmem + h * kTileN, adesc + s * (256 / 16),
+                                  bdesc + (b * kInferStep + h * kTileN * 32) / 16, idesc, s > 0 ? 1u : 0u);
+                    umma_commit(&empty[b]);
+                    // the slot before this one takes its next step once its MMAs are done
+                    if (!(first && s == 0) && left > 0) {
+                        fine = mbar_wait(&empty[p % kInferSlots], (p / kInferSlots) & 1, kWaitPolls);
+                        if (fine) load(p % kInferSlots);
+                    }
+                }
+            }
+            if (!fine) s_fail = 1;
+            umma_commit(&mbar);
+        }
+        first = false;
+        bool ok = true;
+        if (!mbar_wait(&mbar, phase, polls)) {
+            ok = false;
+            if (lane == 0) atomicOr(err, 1);
+            mbar_wait(&mbar, phase, kWaitPolls);   // the committed MMAs finish first
+        }
+        phase ^= 1;
+        fence_after_sync();
+        ok = __syncthreads_and(ok);
+        if (s_fail) {
+            if (tid == 0) atomicOr(err, 1);
+            ok = false;
+        }
+        return ok;
+    };
+    // 16 bytes (eight features from 8 kb) of this row's activations
+    auto store8 = [&](int kb, const unsigned long long h[4]) {
+        unsigned u[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            float a, b;
+            unpack2(h[q], a, b);
+            const __nv_bfloat162 h2 = __floats2bfloat162_rn(a, b);
+            u[q] = *reinterpret_cast<const unsigned*>(&h2);
+        }
+        *reinterpret_cast<uint4*>(sA + (size_t)((r >> 3) * (kKC / 8) + kb) * 128 + (r & 7) * 16) =
+            make_uint4(u[0], u[1], u[2], u[3]);
+    };
+    // pre-activations of eight features: accumulator plus bias
+    const unsigned trow = tmem + ((unsigned)((warp & 3) * 32) << 16);
+    auto pre8 = [&](int kb, const float* bias, unsigned long long z[4]) {
+        float v[8];
+        unsigned long long b[4];
+        tmem_ld8(trow + kb * 8, v);
+        lds8(bias + kb * 8, b);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) z[q] = add2(pack2(v[2 * q], v[2 * q + 1]), b[q]);
+    };
+#pragma unroll 1
+    for (int t = blockIdx.x; t < tiles; t += gridDim.x) {
+        const long long s = (long long)t * kTileM + r;
+        const bool live = s < count;
+        int id[4] = {0, 0, 0, 0};
+        float4 xs = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        if (live) {
+            if constexpr (GRID) {
+                decode_node(g, (int)s, id);
+                xs = make_float4(__ldg(ig.coord + id[0]), __ldg(ig.coord + kCoordMax + id[1]),
+                                 __ldg(ig.coord + 2 * kCoordMax + id[2]), __ldg(ig.coord + 3 * kCoordMax + id[3]));
+            } else {
+                xs = *reinterpret_cast<const float4*>(x + 4 * s);
+            }
+        }
+        {
+            const unsigned long long xx[4] = {pack2(xs.x, xs.x), pack2(xs.y, xs.y), pack2(xs.z, xs.z),
+                                              pack2(xs.w, xs.w)};
+#pragma unroll 1
+            for (int k = 0; k < kH / 32; ++k) {
+                const int kb = part * (kH / 32) + k;
+                unsigned long long z[4], w[4];
+                lds8(sB1 + kb * 8, z);
+#pragma unroll
+                for (int d = 0; d < 4; ++d) {
+                    lds8(sW1 + d * kH + kb * 8, w);
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) z[q] = fma2(w[q], xx[d], z[q]);
+                }
+#pragma unroll
+                for (int q = 0; q < 4; ++q) z[q] = gelu2(z[q]);
+                store8(kb, z);
+            }
+        }
+        if (!layer()) break;
+#pragma unroll 1
+        for (int k = 0; k < kH / 32; ++k) {
+            const int kb = part * (kH / 32) + k;
+            unsigned long long z[4];
+            pre8(kb, sB2, z);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) z[q] = gelu2(z[q]);
+            store8(kb, z);
+        }
+        if (!layer()) break;
+        // output layer: this thread's groups are part, part + 4, ..., taken in
+        // the order that leaves the tree's partial sums fewest
+        float T[3] = {0.0f, 0.0f, 0.0f};
+        {
+            float a4[3] = {}, a8[3] = {}, p16[3] = {};
+#pragma unroll 1
+            for (int k = 0; k < 8; ++k) {
+                const int i = ((k & 1) << 2) | (k & 2) | (k >> 2);
+                const int kb = part + 4 * i;
+                unsigned long long z[4], w[3][4];
+                pre8(kb, sB3, z);
+#pragma unroll
+                for (int o = 0; o < 3; ++o) lds8(sW4 + o * kH + kb * 8, w[o]);
+                float p[3] = {0.0f, 0.0f, 0.0f};
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    float h0, h1;
+                    unpack2(gelu2(z[q]), h0, h1);
+                    h0 = __bfloat162float(__float2bfloat16(h0));
+                    h1 = __bfloat162float(__float2bfloat16(h1));
+#pragma unroll
+                    for (int o = 0; o < 3; ++o) {
+                        float w0, w1;
+                        unpack2(w[o][q], w0, w1);
+                        p[o] = fmaf(w1, h1, fmaf(w0, h0, p[o]));
+                    }
+                }
+#pragma unroll
+                for (int o = 0; o < 3; ++o) {
+                    if (!(k & 1)) {
+                        p16[o] = p[o];
+                    } else {
+                        const float q16 = p16[o] + p[o];          // groups g, g + 16
+                        if (!(k & 2)) {
+                            a8[o] = q16;
+                        } else {
+                            const float q8 = a8[o] + q16;         // and g + 8, g + 24
+                            if (!(k & 4)) a4[o] = q8;
+                            else T[o] = a4[o] + q8;               // and g + 4, ...
+                        }
+                    }
+                }
+            }
+        }
+        // the four parts of a row meet in part 0; the others go on to the next tile
+        if (part > 0) {
+#pragma unroll
+            for (int o = 0; o < 3; ++o) sT[(o * 3 + part - 1) * kTileM + r] = T[o];
+        }
+        __syncthreads();
+        if (part == 0 && live) {
+            float out[3];
+#pragma unroll
+            for (int o = 0; o < 3; ++o) {
+                const float* q = sT + o * 3 * kTileM + r;
+                out[o] = ((T[o] + q[kTileM]) + (q[0] + q[2 * kTileM])) + sW4[3 * kH + o];
+            }
+            if constexpr (GRID) {
+                const double v = fmin(fmax((double)out[0], 0.0), 1.0) * ig.M;
+                const bool tgt = in_target(g, id);
+                if (ig.fp32) ((float*)ig.V)[s] = tgt ? 0.0f : (float)v;
+                else ((double*)ig.V)[s] = tgt ? 0.0 : v;
+                const double a = atan2((double)out[2], (double)out[1]);   // (-pi, pi]
+                const long long c = llrint(a * (65536.0 / 6.283185307179586476925286766559));
+                ig.code[s] = (uint16_t)(c & 65535);
+            } else {
+#pragma unroll
+                for (int o = 0; o < 3; ++o) y[3 * s + o] = out[o];
+            }
+        }
+    }
+    if (tid == 0 && left > 0) {
+        // a wait gave up: no copy may outlive the CTA.  The slots' last copies
+        // were those of the layer's last four steps, or of the next layer's
+        // first three and the last: every slot's copy of the current phase
+#pragma unroll
+        for (int b = 0; b < kInferSlots; ++b) mbar_wait(&full[b], b < kInferSlots - 1 ? 0 : 1, kWaitPolls);
+    }
+    fence_before_sync();
+    __syncthreads();
+    if (warp == 0) tmem_dealloc(tmem, kH);
+}
+
 // Inputs (normalised to [-1, 1]^4) and targets (V / M, cos, sin) of nodes
 // idx = (mult * (start + i) + offset) mod n of a grid (a seeded permutation).
 // Without V only the inputs are written.  Inputs are normalised to the
@@ -567,30 +912,6 @@ __global__ void l1_fwd_kernel(const float* __restrict__ x, const float* __restri
             h1[(size_t)s * kH + o] = __float2bfloat16(s < count ? gelu(z) : 0.0f);
             if (z1) z1[(size_t)s * kH + o] = z;
         }
-    }
-}
-
-// Output layer (256 -> 3): one warp per sample, each lane 8 consecutive
-// features (one 16-byte load), the three sums reduced across the warp.
-__global__ void out_kernel(const bf16* __restrict__ h3, const float* __restrict__ P, int count,
-                           float* __restrict__ y)
-{
-    __shared__ float sW[3 * kH + 3];
-    for (int i = threadIdx.x; i < 3 * kH + 3; i += blockDim.x) sW[i] = P[kOffW4 + i];   // W4 then b4
-    __syncthreads();
-    const int lane = threadIdx.x & 31;
-    const int s = (int)((blockIdx.x * (size_t)blockDim.x + threadIdx.x) >> 5);
-    if (s >= count) return;
-    float a[8];
-    load_row8(h3 + (size_t)s * kH + lane * 8, a);
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        float sum = 0.0f;
-#pragma unroll
-        for (int q = 0; q < 8; ++q) sum += sW[k * kH + lane * 8 + q] * a[q];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-        if (lane == 0) y[3 * (size_t)s + k] = sum + sW[3 * kH + k];
     }
 }
 
@@ -819,24 +1140,6 @@ __global__ void bf16_weights_kernel(const float* __restrict__ P, bf16* __restric
     W3T[i * kH + o] = __float2bfloat16(P[kOffW3 + e]);
 }
 
-// Warm start: V = M clamp(V/M-hat, 0, 1) (target nodes 0) and the code of
-// atan2(sin-hat, cos-hat), for compact nodes [start, start + count).
-template <typename S>
-__global__ void warm_write_kernel(Geo<double> g, const float* __restrict__ y, long long start, int count, double M,
-                                  S* __restrict__ V, uint16_t* __restrict__ code)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= count) return;
-    const long long j = start + i;
-    int id[4];
-    decode_node(g, (int)j, id);
-    const double v = fmin(fmax((double)y[3 * i], 0.0), 1.0) * M;
-    V[j] = in_target(g, id) ? (S)0 : (S)v;
-    const double a = atan2((double)y[3 * i + 2], (double)y[3 * i + 1]);   // (-pi, pi]
-    long long c = llrint(a * (65536.0 / 6.283185307179586476925286766559));
-    code[j] = (uint16_t)(c & 65535);
-}
-
 int fail_cuda(const char* what, cudaError_t e)
 {
     char buf[256];
@@ -864,6 +1167,8 @@ struct dp_mlp {
     float *x = nullptr, *t = nullptr, *z1 = nullptr, *z2 = nullptr, *z3 = nullptr, *y = nullptr;
     bf16 *h1 = nullptr, *h2 = nullptr, *h3 = nullptr, *dz1 = nullptr, *dz2 = nullptr, *dz3 = nullptr;
     double* states = nullptr;
+    unsigned char* Wsteps = nullptr;   // hidden weights as the inference kernel's K steps
+    float* coord = nullptr;            // normalised node coordinates per dimension (4 x kCoordMax)
     float* loss = nullptr;
     float* part = nullptr;             // partial sums of the backward pass (kPartFloats)
     float* red = nullptr;              // per-row-tile sums of the fused backward GEMMs (cap / 128 x 5 x 256)
@@ -886,7 +1191,7 @@ void free_mlp(dp_mlp* m)
     cudaSetDevice(m->device);
     if (m->st) cudaStreamSynchronize(m->st);
     void* ps[] = {m->P, m->G, m->Am, m->Av, m->W2b, m->W3b, m->W2T, m->W3T, m->x, m->t, m->z1, m->z2, m->z3, m->y,
-                  m->h1, m->h2, m->h3, m->dz1, m->dz2, m->dz3, m->states, m->loss, m->part, m->red, m->arrive, m->err};
+                  m->h1, m->h2, m->h3, m->dz1, m->dz2, m->dz3, m->states, m->Wsteps, m->coord, m->loss, m->part, m->red, m->arrive, m->err};
     for (void* p : ps)
         if (p) cudaFree(p);
     if (m->h_loss) cudaFreeHost(m->h_loss);
@@ -987,29 +1292,31 @@ cudaError_t gemm(dp_mlp* m, const bf16* A, int lda, const bf16* B, int ldb, int 
     return gemm_kc<EPI, kKC>(m, A, lda, B, ldb, rows, k_total, k_split, bias, zout, zin, hout, cacc);
 }
 
-// Hidden layers of the forward pass of `count` rows held in m->x (rows
-// padded to a multiple of 128), through h3.  save: keep z1..z3 for a
-// backward pass.
-int forward_hidden(dp_mlp* m, int count, bool save)
+// Hidden layers of a training step's forward pass of `rows` rows held in m->x
+// (a multiple of 512), through h3, keeping z1..z3 for the backward pass.
+int forward_hidden(dp_mlp* m, int rows)
 {
-    const int rows = (count + kTileM - 1) / kTileM * kTileM;
     const long long e8 = (long long)rows * 32;
     const unsigned b1 = (unsigned)std::min<long long>((e8 + 255) / 256, 8LL * m->sm_count);
-    l1_fwd_kernel<<<b1, 256, 0, m->st>>>(m->x, m->P, count, rows, save ? m->z1 : nullptr, m->h1);
+    l1_fwd_kernel<<<b1, 256, 0, m->st>>>(m->x, m->P, rows, rows, m->z1, m->h1);
     MCK(cudaGetLastError());
-    MCK(gemm<kEpiFwd>(m, m->h1, kH, m->W2b, kH, rows, kH, 1, m->P + kOffB2, save ? m->z2 : nullptr, nullptr, m->h2,
-                      nullptr));
-    MCK(gemm<kEpiFwd>(m, m->h2, kH, m->W3b, kH, rows, kH, 1, m->P + kOffB3, save ? m->z3 : nullptr, nullptr, m->h3,
-                      nullptr));
+    MCK(gemm<kEpiFwd>(m, m->h1, kH, m->W2b, kH, rows, kH, 1, m->P + kOffB2, m->z2, nullptr, m->h2, nullptr));
+    MCK(gemm<kEpiFwd>(m, m->h2, kH, m->W3b, kH, rows, kH, 1, m->P + kOffB3, m->z3, nullptr, m->h3, nullptr));
     return DP_OK;
 }
 
-// Forward of `count` rows into m->y.
-int forward(dp_mlp* m, int count)
+// Inference of `count` rows: of m->x into m->y, or (GRID) of a grid's stored
+// nodes into its value and policy.
+template <bool GRID>
+int infer(dp_mlp* m, int count, const Geo<double>& g, const InferGrid& ig)
 {
-    int rc;
-    if ((rc = forward_hidden(m, count, false))) return rc;
-    out_kernel<<<(count + 7) / 8, 256, 0, m->st>>>(m->h3, m->P, count, m->y);
+    static std::atomic<bool> attr[kMaxDevices];
+    MCK(raise_smem_limit(mlp_infer_kernel<GRID>, kInferSmem, attr));
+    infer_weights_kernel<<<2 * kInferSteps * kInferStep / 16 / 256, 256, 0, m->st>>>(m->W2b, m->W3b, (uint4*)m->Wsteps);
+    MCK(cudaGetLastError());
+    const int tiles = (int)(((long long)count + kTileM - 1) / kTileM);
+    mlp_infer_kernel<GRID><<<std::min(tiles, 2 * m->sm_count), kInferThreads, kInferSmem, m->st>>>(
+        g, ig, m->x, m->P, m->Wsteps, count, m->y, m->err, m->wait_polls);
     MCK(cudaGetLastError());
     return DP_OK;
 }
@@ -1021,7 +1328,7 @@ int forward_backward(dp_mlp* m, int count, float inv_n)
 {
     const int rows = count;
     int rc;
-    if ((rc = forward_hidden(m, count, true))) return rc;
+    if ((rc = forward_hidden(m, rows))) return rc;
     // every gradient sum goes through per-block partial sums and a reduction
     // in a fixed order, so that a training run is reproducible bit for bit
     auto seg = [](const float* part, int n_part, int stride, int len, float* out, int accumulate) {
@@ -1260,7 +1567,7 @@ int dp_mlp_create(const double* lo, const double* hi, int32_t batch_capacity, vo
     A(&m->x, C * 4); A(&m->t, C * 3); A(&m->y, C * 3);
     A(&m->z1, CH); A(&m->z2, CH); A(&m->z3, CH);
     A(&m->h1, CH); A(&m->h2, CH); A(&m->h3, CH); A(&m->dz1, CH); A(&m->dz2, CH); A(&m->dz3, CH);
-    A(&m->states, C * 4); A(&m->loss, 1); A(&m->err, 1); A(&m->part, kPartFloats);
+    A(&m->states, C * 4); A(&m->Wsteps, 2 * kInferSteps * kInferStep); A(&m->coord, 4 * kCoordMax); A(&m->loss, 1); A(&m->err, 1); A(&m->part, kPartFloats);
     A(&m->red, C / kTileM * 5 * kH); A(&m->arrive, 1);
     A(&m->ts, 1);
     if (e == cudaSuccess) e = cudaMallocHost(&m->h_loss, sizeof(float));
@@ -1323,7 +1630,7 @@ int dp_mlp_forward(dp_mlp* m, const double* states, int32_t n, float* out)
                             m->st));
         states_in_kernel<<<(cnt + 255) / 256, 256, 0, m->st>>>(m->states, cnt, lo, hi, m->x);
         MCK(cudaGetLastError());
-        int rc = forward(m, cnt);
+        int rc = infer<false>(m, cnt, Geo<double>(), InferGrid());
         if (rc) return rc;
         MCK(cudaMemcpyAsync(out + 3 * (size_t)s0, m->y, sizeof(float) * 3 * cnt, cudaMemcpyDeviceToHost, m->st));
     }
@@ -1407,23 +1714,12 @@ int dp_warm_start(dp_mlp* m, dp_grid* grid, double* ms_out)
     Geo<double> g = gv.g64;
     const Box4 nlo{m->lo[0], m->lo[1], m->lo[2], m->lo[3]};
     const Box4 nhi{m->hi[0], m->hi[1], m->hi[2], m->hi[3]};
-    for (long long s0 = 0; s0 < gv.n; s0 += m->cap) {
-        const int cnt = (int)std::min<long long>(m->cap, gv.n - s0);
-        batch_from_grid_kernel<double><<<(cnt + 255) / 256, 256, 0, m->st>>>(
-            g, (const double*)nullptr, gv.code, gv.tab_hi64, gv.tab_lo64, gv.n, 1, 0, s0, cnt, 0.0, nlo, nhi, m->x,
-            nullptr);
-        MCK(cudaGetLastError());
-        if ((rc = forward(m, cnt))) return rc;
-        // the value goes to the storage-precision buffer (an FP32 grid holding
-        // FP64 values after a polish returns to its FP32 values)
-        if (gv.fp32)
-            warm_write_kernel<float><<<(cnt + 255) / 256, 256, 0, m->st>>>(g, m->y, s0, cnt, gv.M, (float*)gv.V,
-                                                                         gv.code);
-        else
-            warm_write_kernel<double><<<(cnt + 255) / 256, 256, 0, m->st>>>(g, m->y, s0, cnt, gv.M, (double*)gv.V,
-                                                                          gv.code);
-        MCK(cudaGetLastError());
-    }
+    coord_table_kernel<<<4, kCoordMax, 0, m->st>>>(g, nlo, nhi, m->coord);
+    MCK(cudaGetLastError());
+    // the value goes to the storage-precision buffer (an FP32 grid holding
+    // FP64 values after a polish returns to its FP32 values)
+    const InferGrid ig{m->coord, gv.M, const_cast<void*>(gv.V), gv.code, gv.fp32};
+    if ((rc = infer<true>(m, (int)gv.n, g, ig))) return rc;
     MCK(cudaEventRecord(e1, m->st));
     if ((rc = check_err(m))) return rc;
     float ms = 0;

@@ -59,6 +59,19 @@ __device__ __forceinline__ void mbar_init(unsigned long long* bar)
     asm volatile("fence.mbarrier_init.release.cluster;");
 }
 
+// The phase's arrival of this thread, expecting `bytes` of bulk copies, and a
+// bulk copy global -> shared that completes them (16-byte aligned addresses,
+// a size that is a multiple of 16).
+__device__ __forceinline__ void mbar_expect_bytes(unsigned long long* bar, unsigned bytes)
+{
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" :: "r"(smem_u32(bar)), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void bulk_copy(void* dst, const void* src, unsigned bytes, unsigned long long* bar)
+{
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                 :: "r"(smem_u32(dst)), "l"(src), "r"(bytes), "r"(smem_u32(bar)) : "memory");
+}
+
 // D (TMEM) = (accumulate ? D : 0) + A * B^T for one K = 16 step.
 __device__ __forceinline__ void umma_bf16(unsigned tmem_d, unsigned long long adesc, unsigned long long bdesc,
                                           unsigned idesc, unsigned accumulate)
@@ -82,6 +95,18 @@ __device__ __forceinline__ bool mbar_wait(unsigned long long* bar, int parity, i
         asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}\n"
                      : "=r"(done) : "r"(smem_u32(bar)), "r"(parity));
     return done != 0;
+}
+
+// 8 consecutive FP32 accumulator columns of this thread's TMEM lane.
+__device__ __forceinline__ void tmem_ld8(unsigned taddr, float v[8])
+{
+    unsigned r[8];
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(taddr));
+    asm volatile("tcgen05.wait::ld.sync.aligned;");
+#pragma unroll
+    for (int q = 0; q < 8; ++q) v[q] = __uint_as_float(r[q]);
 }
 
 // 16 consecutive FP32 accumulator columns of this thread's TMEM lane.
