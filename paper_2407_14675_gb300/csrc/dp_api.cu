@@ -42,6 +42,8 @@ int fail(int code, const char* fmt, ...)
     } while (0)
 
 constexpr int kRing = 8192;        // residual slots (power of two)
+constexpr int kLoopDoubles = 10;    // per state of a feedback or closed-loop call
+constexpr int kLoopPinned = 65536;  // states of feedback / closed-loop calls through the pinned buffer (5 MB)
 constexpr int kMaxChunk = 2048;    // sweeps enqueued between host checks (< kRing / 2)
 constexpr double kStallZone = 64.0; // "near the FP32 floor": below this multiple of the switch tolerance
 constexpr int kStallFar = 30;       // improvements without gain that switch anywhere
@@ -112,6 +114,10 @@ struct dp_grid {
     int gm_blocks = 0;
     GmCtl* gm_ctl = nullptr;
     GmTail* h_gm = nullptr;              // pinned, one per cycle of a round
+    // states and results of feedback and closed loop (pinned, read and written
+    // by the kernel in place; grown up to kLoopPinned states)
+    double* h_loop = nullptr;
+    int loop_cap = 0;
 
     Geo<double> g64;
     Geo<float> g32;
@@ -148,6 +154,7 @@ void free_grid(dp_grid* g)
     if (g->h_ctl) cudaFreeHost(g->h_ctl);
     if (g->h_ring) cudaFreeHost(g->h_ring);
     if (g->h_gm) cudaFreeHost(g->h_gm);
+    if (g->h_loop) cudaFreeHost(g->h_loop);
     delete g;
 }
 
@@ -730,15 +737,42 @@ int loop_common(const dp_grid* cg, const double* states, int n, double tau, doub
     long long steps = 0;
     if (t_arrive) steps = (long long)std::ceil(t_max / h - 1e-9);
     if (t_arrive && steps < 1) steps = 1;
+    // n x {state 4, angle or arrival 1, q 1, final state 4} doubles.  Up to
+    // kLoopPinned states they sit in pinned memory of the grid (few states: the
+    // residual ring's mirror, which only a solve uses), which the kernel reads
+    // once and writes once over the host link: a call is one launch and one
+    // synchronisation.  With a device buffer allocated and freed around the call
+    // (the synchronisation hands its pages back) and a copy each way a decision
+    // for 8 states took 194 us, of which the kernel is 11; larger calls keep
+    // that form.
     double* d_buf = nullptr;
-    size_t nb = (size_t)n * (4 + 1 + 1 + 4);
-    CK(cudaMallocAsync(&d_buf, nb * sizeof(double), g->st));
+    const size_t nb = (size_t)n * kLoopDoubles;
+    const bool pinned = n <= kLoopPinned;
+    if (pinned) {
+        static_assert(sizeof(double) == sizeof(*g->h_ring), "ring entries");
+        if (nb <= (size_t)kRing) {
+            d_buf = (double*)g->h_ring;
+        } else {
+            if (n > g->loop_cap) {
+                const int cap = std::min(kLoopPinned, 2 * n);
+                double* p = nullptr;
+                CK(cudaMallocHost((void**)&p, (size_t)cap * kLoopDoubles * sizeof(double)));
+                if (g->h_loop) cudaFreeHost(g->h_loop);   // no call is in flight: each one synchronises
+                g->h_loop = p;
+                g->loop_cap = cap;
+            }
+            d_buf = g->h_loop;
+        }
+        memcpy(d_buf, states, sizeof(double) * 4 * n);
+    } else
+        CK(cudaMallocAsync(&d_buf, nb * sizeof(double), g->st));
     double* d_x0 = d_buf;
     double* d_a = d_buf + 4 * (size_t)n;
     double* d_q = d_a + n;
     double* d_xf = d_q + n;
     int rc = DP_OK;
-    cudaError_t e = cudaMemcpyAsync(d_x0, states, sizeof(double) * 4 * n, cudaMemcpyHostToDevice, g->st);
+    cudaError_t e = cudaSuccess;
+    if (!pinned) e = cudaMemcpyAsync(d_x0, states, sizeof(double) * 4 * n, cudaMemcpyHostToDevice, g->st);
     if (e == cudaSuccess) {
         switch (store_of(g)) {
         case kStoreF64:
@@ -753,7 +787,7 @@ int loop_common(const dp_grid* cg, const double* states, int n, double tau, doub
             rc = run_loop<float, double>(g, g->g32, g->V64[g->cur64], d_x0, n, tau, h, steps, drag, d_a, d_q, d_a,
                                          d_xf);
         }
-        if (rc == DP_OK) {
+        if (rc == DP_OK && !pinned) {
             if (t_arrive) {
                 e = cudaMemcpyAsync(t_arrive, d_a, sizeof(double) * n, cudaMemcpyDeviceToHost, g->st);
                 if (e == cudaSuccess)
@@ -765,12 +799,21 @@ int loop_common(const dp_grid* cg, const double* states, int n, double tau, doub
             }
         }
     }
-    cudaError_t e2 = cudaFreeAsync(d_buf, g->st);
+    cudaError_t e2 = pinned ? cudaSuccess : cudaFreeAsync(d_buf, g->st);
     cudaError_t e3 = cudaStreamSynchronize(g->st);
     if (rc) return rc;
     if (e != cudaSuccess) return fail(DP_ECUDA, "closed loop: %s", cudaGetErrorString(e));
     if (e2 != cudaSuccess || e3 != cudaSuccess)
         return fail(DP_ECUDA, "closed loop: %s", cudaGetErrorString(e2 != cudaSuccess ? e2 : e3));
+    if (pinned) {
+        if (t_arrive) {
+            memcpy(t_arrive, d_a, sizeof(double) * n);
+            memcpy(x_final, d_xf, sizeof(double) * 4 * n);
+        } else {
+            memcpy(alpha_out, d_a, sizeof(double) * n);
+            if (q_out) memcpy(q_out, d_q, sizeof(double) * n);
+        }
+    }
     return DP_OK;
 }
 
