@@ -95,6 +95,7 @@ struct dp_grid {
     int foot_format = DP_FOOT_AUTO;         // dp_set_foot_format
     Feet64 f64;                             // frozen feet of FP64 grids
     bool feet64_valid = false;
+    bool diag64_valid = false;              // f64.r holds the factors of these feet
     float* acc = nullptr;                   // FP64-value polish: running sum of increments
     int* wave_sync = nullptr;               // FP32 grids: counters of the multi-level evaluation
     Ctl* ctl = nullptr;
@@ -147,7 +148,7 @@ void free_grid(dp_grid* g)
     if (g->st) cudaStreamSynchronize(g->st);
     void* ps[] = {g->rows, g->row_org, g->lines, g->hi64, g->lo64, g->hi32, g->lo32, g->V[0], g->V[1], g->V64[0],
                   g->V64[1], g->code, g->feet_lo, g->feet_hi, g->acc, g->ctl, g->ring, g->staging,
-                  g->scratch64, g->gm_Q, g->gm_partial, g->gm_ctl, g->f64.w, g->f64.t, g->f64.c,
+                  g->scratch64, g->gm_Q, g->gm_partial, g->gm_ctl, g->f64.w, g->f64.t, g->f64.c, g->f64.r,
                   g->wave_sync};
     for (void* p : ps)
         if (p) cudaFree(p);
@@ -354,14 +355,23 @@ cudaError_t enqueue_sweep(dp_grid* g, int pmode, long long t, int check_prev, do
             g->feet_valid = g->feet_lo != nullptr;
             g->feet8 = g->store_feet8;
         }
-        if (store_of(g) == kStoreF64) g->feet64_valid = g->f64.w != nullptr;
+        if (store_of(g) == kStoreF64) {
+            g->feet64_valid = g->f64.w != nullptr;
+            g->diag64_valid = false;
+        }
     }
     const int mode = internal_mode(g, pmode);
     switch (store_of(g)) {
     case kStoreF64: {
         const double* in = (const double*)g->V[(g->cur + a) & 1];
         double* out = (double*)g->V[(g->cur + a + 1) & 1];
-        return launch_sweep(sweep_launch<double, double>(g, g->g64, in, out, mode, t, check_prev, tol));
+        SweepLaunch<double, double> L = sweep_launch<double, double>(g, g->g64, in, out, mode, t, check_prev, tol);
+        if (mode == kEvalFeet64Diag) {
+            // the first such sweep of these feet stores their diagonal factors
+            L.incr_flags = g->diag64_valid ? 0 : 1;
+            g->diag64_valid = true;
+        }
+        return launch_sweep(L);
     }
     case kStoreF32: {
         const float* in = (const float*)g->V[(g->cur + a) & 1];
@@ -1149,7 +1159,7 @@ int dp_grid_create(const dp_grid_desc* desc, dp_grid** out)
                     (rc = dalloc(g, &g->wave_sync, wave_sync_ints(kWaveMaxLevels, g->n_active)))))
         return bail(rc);
     if (!g->fp32 && ((rc = dalloc(g, &g->f64.w, g->n_active)) || (rc = dalloc(g, &g->f64.t, 2 * g->n_active)) ||
-                     (rc = dalloc(g, &g->f64.c, g->n_active))))
+                     (rc = dalloc(g, &g->f64.c, g->n_active)) || (rc = dalloc(g, &g->f64.r, g->n_active))))
         return bail(rc);
     if ((rc = dalloc(g, &g->ctl, 1))) return bail(rc);
     if ((rc = dalloc(g, &g->ring, kRing))) return bail(rc);
@@ -1540,6 +1550,7 @@ int dp_policy_iterate(dp_grid* g, const dp_solve_opts* o, dp_solve_stats* stats)
             }
         }
     }
+    g->diag64_valid = false;   // the sweep that was to store the factors may have returned at a passed stopping test
     if (store_of(g) != kStoreMix) advance(g, t);
     S.history_count = std::min<long long>(hist_n, o->history ? o->history_capacity : 0);
     S.residual = res;

@@ -588,10 +588,14 @@ struct FootWord {
 // thrust cost included).  Evaluation from them gives the recomputing sweep's
 // results bit for bit for the minimum-time dynamics; with the running cost of
 // Eq. (11), computed in another kernel, to an ulp of the constant.
+// The first diagonal-solved sweep after an improvement also stores the node's
+// factor 1 / (1 - beta w_jj) in r, which the later ones read (8 bytes instead
+// of 16 of the 59 FP64 operations a node took).
 struct Feet64 {
     unsigned long long* w = nullptr;
     double2* t = nullptr;
     double* c = nullptr;
+    double* r = nullptr;
 };
 
 __device__ __forceinline__ FootWord foot_word_kind(int kind)

@@ -275,9 +275,16 @@ __device__ __forceinline__ void sweep_nodes(const Geo<G>& g, const Table<G>& T, 
     (void)T;
     (void)kSearch;
     if constexpr (MODE == kEvalFeet64 || MODE == kEvalFeet64Diag) {
-        // FP64 evaluation from the FP64 frozen feet
+        // FP64 evaluation from the FP64 frozen feet: bound by the FP64 pipe (two
+        // lanes a clock and SM), 43 operations a node.  The residual and the
+        // finiteness test run on the bits (non-negative doubles order like them).
+        // Example 1 (2.97M nodes): 0.25 ms diagonal-solved, 0.32 ms with the
+        // diagonal factor formed in every sweep and FP64 comparisons.
         constexpr bool kDiag = MODE == kEvalFeet64Diag;
         constexpr bool kPer = DYN == kDynPolar;
+        const bool first = incr_flags & 1;   // diagonal-solved: store the factors
+        constexpr unsigned long long kInf = 0x7ff0000000000000ull;
+        unsigned long long rbits = 0;
         for (int j = j0; j < end; j += stride) {
             const S vj = Vin[j];
             const unsigned long long w = __ldcs(&f64.w[j]);
@@ -285,7 +292,8 @@ __device__ __forceinline__ void sweep_nodes(const Geo<G>& g, const Table<G>& T, 
             S vnew = (S)0;
             if (kind != kFootTarget) {
                 const double cj = __ldcs(&f64.c[j]);
-                double D, ws = 0.0;
+                double D, ws = 0.0, rd = 0.0;
+                if (kDiag && !first) rd = __ldcs(&f64.r[j]);
                 if (kind == kFootOut) {
                     D = g.M64 - (double)vj;
                 } else if (kind == kFootInside) {
@@ -299,7 +307,7 @@ __device__ __forceinline__ void sweep_nodes(const Geo<G>& g, const Table<G>& T, 
                     Corners<double> K;
                     load_corners<double, G, S, REDUCED, kPer>(g, Vin, cl, vj, K);   // membership checked when stored
                     D = K.blend(t);
-                    if constexpr (kDiag) ws = self_weight<G, kPer>(g, i, cl, t);
+                    if (kDiag && first) ws = self_weight<G, kPer>(g, i, cl, t);
                 } else {
                     NodeEval<G, S, REDUCED, DYN> ev;
                     decode_node(g, j, ev.i);
@@ -313,13 +321,21 @@ __device__ __forceinline__ void sweep_nodes(const Geo<G>& g, const Table<G>& T, 
                     ws = wr;
                 }
                 double q = cj + g.beta64 * ((double)vj + D);
-                if constexpr (kDiag) q = diag_step(g, (double)vj, q, ws);
+                if constexpr (kDiag) {
+                    if (first) {
+                        rd = recip_newton(1.0 - g.beta64 * ws);
+                        __stcs(&f64.r[j], rd);
+                    }
+                    q = (double)vj + (q - (double)vj) * rd;   // diag_step()
+                }
                 vnew = (S)q;
             }
             Vout[j] = vnew;
-            resid = fmax(resid, (S)fabs(vnew - vj));
-            bad = bad || !isfinite(vnew);
+            const unsigned long long b = (unsigned long long)__double_as_longlong(vnew - vj) & ~(1ull << 63);
+            if (b > rbits && b <= kInf) rbits = b;   // a NaN raises `bad` instead, as fmax would pass it over
+            bad = bad || ((unsigned long long)__double_as_longlong(vnew) & kInf) == kInf;
         }
+        resid = fmax(resid, (S)__longlong_as_double((long long)rbits));
     } else if constexpr (MODE == kEvalFeet || MODE == kEvalFeet8 || MODE == kIncr || MODE == kEvalFeetDiag ||
                          MODE == kIncrDiag) {
         constexpr bool kDiag = MODE == kEvalFeetDiag || MODE == kIncrDiag;
