@@ -22,6 +22,7 @@
 
 #include "dp_device.cuh"
 #include "dp_host.h"
+#include "dp_search64.cuh"
 
 namespace dpk {
 
@@ -272,6 +273,8 @@ __device__ __forceinline__ void sweep_nodes(const Geo<G>& g, const Table<G>& T, 
     constexpr bool kImprove = MODE == kImproveFull || MODE == kImproveWalk;
     constexpr bool kGeo32 = std::is_same<G, float>::value;
     constexpr bool kPolish = kGeo32 && std::is_same<S, double>::value;   // FP32 geometry, FP64 values
+    // FP64 grids decide their searches by an FP32 model (dp_search64.cuh)
+    constexpr bool kModel = !kGeo32 && DYN != kDynUnitSpeed && MODE != kVIDiag;
     (void)T;
     (void)kSearch;
     if constexpr (MODE == kEvalFeet64 || MODE == kEvalFeet64Diag) {
@@ -459,15 +462,15 @@ __device__ __forceinline__ void sweep_nodes(const Geo<G>& g, const Table<G>& T, 
                     } else {
                         ev.reset();
                         typename Eval::R D;
-                        int k;
-                        const int c_old = MODE == kImproveWalk ? (int)code[j] : 0;
-                        // a node whose previous control was off has no angle to walk from
-                        if (MODE == kImproveWalk && !(g.off && c_old == kCodeOff))
-                            k = walk_table(ev, T, nearest_index(g.K, c_old), D);
-                        else
-                            k = enumerate_table(ev, T, D);
-                        int c = T.code[k] & (kCodes - 1);
-                        if (!kIsVI && g.refine) c = fibonacci_refine(ev, T, g.fib_n0, g.fib_stop, k, D, D);
+                        int c;
+                        if constexpr (!kGeo32) {   // polar grids are FP64
+                            const int c_old = MODE == kImproveWalk ? (int)code[j] : 0;
+                            // a node whose previous control was off has no angle to walk from
+                            if (MODE == kImproveWalk && !(g.off && c_old == kCodeOff))
+                                c = search64<REDUCED, DYN, true>(ev, T, g, nearest_index(g.K, c_old), g.refine != 0, D);
+                            else
+                                c = search64<REDUCED, DYN, false>(ev, T, g, 0, !kIsVI && g.refine, D);
+                        }
                         q = lrun + g.thrust_cost + g.beta64 * ((double)vj + (double)D);
                         if (g.off) {
                             const double q_off = lrun + g.beta64 * ((double)vj + (double)ev.at_sc((G)0, (G)0));
@@ -504,14 +507,22 @@ __device__ __forceinline__ void sweep_nodes(const Geo<G>& g, const Table<G>& T, 
                     D = ev.at_code_w(code[j], ws);
                 } else {
                     ev.reset();
-                    int k;
                     const int c_old = (MODE == kImproveWalk || kPolish) ? (int)code[j] : 0;
-                    if (MODE == kImproveWalk)
-                        k = walk_table(ev, T, nearest_index(g.K, c_old), D);
-                    else
-                        k = enumerate_table(ev, T, D);
-                    int c = T.code[k] & (kCodes - 1);
-                    if (!kIsVI && g.refine) c = fibonacci_refine(ev, T, g.fib_n0, g.fib_stop, k, D, D);
+                    int c;
+                    if constexpr (kModel) {
+                        if constexpr (MODE == kImproveWalk)
+                            c = search64<REDUCED, DYN, true>(ev, T, g, nearest_index(g.K, c_old), g.refine != 0, D);
+                        else
+                            c = search64<REDUCED, DYN, false>(ev, T, g, 0, !kIsVI && g.refine, D);
+                    } else {
+                        int k;
+                        if (MODE == kImproveWalk)
+                            k = walk_table(ev, T, nearest_index(g.K, c_old), D);
+                        else
+                            k = enumerate_table(ev, T, D);
+                        c = T.code[k] & (kCodes - 1);
+                        if (!kIsVI && g.refine) c = fibonacci_refine(ev, T, g.fib_n0, g.fib_stop, k, D, D);
+                    }
                     if constexpr (kImprove && kPolish) {
                         // FP64 blend of the chosen code.  Both the walk and the
                         // full tabulation keep the node's current code unless the
@@ -657,10 +668,23 @@ __host__ __device__ constexpr int big_block()
                                                                                         : kBlock;
 }
 
-template <int MODE, bool REDUCED, bool BIG>
+// FP64 searches run many small blocks, one round each (no grid-stride): the
+// FP64 pipe of an SM is the bound, so what counts is an even share per SM, and
+// nodes differ in how much FP64 they need.  The 17^4 box in 256-thread blocks,
+// two resident per SM, took two rounds for 1.07 of nodes.
+constexpr int kSearch64Block = 64;
+
+template <typename G, typename S, int MODE>
+__host__ __device__ constexpr bool search64_blocks()
+{
+    return std::is_same<G, double>::value && std::is_same<S, double>::value &&
+           (MODE == kVI || MODE == kVIDiag || MODE == kImproveFull || MODE == kImproveWalk);
+}
+
+template <typename G, typename S, int MODE, bool REDUCED, bool BIG>
 __host__ __device__ constexpr int sweep_block()
 {
-    return BIG ? big_block<MODE, REDUCED>() : kBlock;
+    return BIG ? big_block<MODE, REDUCED>() : search64_blocks<G, S, MODE>() ? kSearch64Block : kBlock;
 }
 
 template <typename G, typename S, int MODE, bool REDUCED, bool BIG>
@@ -668,6 +692,7 @@ constexpr int min_blocks()
 {
     constexpr bool feet64 = MODE == kEvalFeet64 || MODE == kEvalFeet64Diag;
     if (BIG) return feet64 ? 1 : 2;
+    if (search64_blocks<G, S, MODE>()) return MODE == kVI ? 10 : 8;   // 96 and 128 registers
     // FP32 angle searches: 3 blocks of 256 per SM (80 registers).  Left to
     // itself the compiler gives the reduced-grid walk 96 registers (2 blocks):
     // 4.84 against 4.36 ms per sweep on the 121^4 band
@@ -681,7 +706,7 @@ constexpr int min_blocks()
 }
 
 template <typename G, typename S, int MODE, bool REDUCED, int DYN, bool BIG>
-__global__ void __launch_bounds__(sweep_block<MODE, REDUCED, BIG>(), min_blocks<G, S, MODE, REDUCED, BIG>())
+__global__ void __launch_bounds__(sweep_block<G, S, MODE, REDUCED, BIG>(), min_blocks<G, S, MODE, REDUCED, BIG>())
 sweep_kernel(const __grid_constant__ Geo<G> g, const S* __restrict__ Vin, S* __restrict__ Vout,
              uint16_t* __restrict__ code, unsigned long long* __restrict__ feet_lo, unsigned* __restrict__ feet_hi,
              float* __restrict__ inc, float* __restrict__ acc, double* __restrict__ V64, int incr_flags,
@@ -702,8 +727,10 @@ sweep_kernel(const __grid_constant__ Geo<G> g, const S* __restrict__ Vin, S* __r
     }
 
     // angle searches read the tabulated codes and (sin, cos) from shared memory
-    __shared__ int s_code[kSearch ? kMaxAngles + 1 : 1];
-    __shared__ typename V2<G>::type s_sc[kSearch ? kMaxAngles : 1];
+    // (sized by the table, so that the rest of it stays L1)
+    extern __shared__ __align__(16) unsigned char s_table[];
+    typename V2<G>::type* s_sc = reinterpret_cast<typename V2<G>::type*>(s_table);
+    int* s_code = reinterpret_cast<int*>(s_sc + (kSearch ? g.K : 0));
     if constexpr (kSearch) {
         build_table(g, s_code, s_sc);
         __syncthreads();
@@ -712,7 +739,7 @@ sweep_kernel(const __grid_constant__ Geo<G> g, const S* __restrict__ Vin, S* __r
 
     S resid = (S)0;
     bool bad = false;
-    constexpr int B = sweep_block<MODE, REDUCED, BIG>();
+    constexpr int B = sweep_block<G, S, MODE, REDUCED, BIG>();
     const int j0 = blockIdx.x * B + threadIdx.x, end = g.n_nodes, stride = gridDim.x * B;
     constexpr bool kReach = std::is_same<G, float>::value && (MODE == kImproveFull || MODE == kImproveWalk);
     int reach = 0;
@@ -731,18 +758,21 @@ template <typename G, typename S, int MODE, bool REDUCED, int DYN, bool BIG>
 cudaError_t launch_sized(const SweepLaunch<G, S>& L)
 {
     auto kern = sweep_kernel<G, S, MODE, REDUCED, DYN, BIG>;
-    constexpr int B = sweep_block<MODE, REDUCED, BIG>();
+    constexpr int B = sweep_block<G, S, MODE, REDUCED, BIG>();
+    constexpr bool kSearch = MODE == kVI || MODE == kVIDiag || MODE == kImproveFull || MODE == kImproveWalk;
+    const size_t smem = kSearch ? (size_t)L.g.K * sizeof(typename V2<G>::type) + (size_t)(L.g.K + 1) * sizeof(int) : 0;
     static int per_sm = 0;
     if (per_sm == 0) {
-        cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, B, 0);
+        cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, B, smem);
         if (e != cudaSuccess) return e;
         if (per_sm < 1) per_sm = 1;
     }
     long long need = ((long long)L.g.n_nodes + B - 1) / B;
     long long cap = (long long)per_sm * L.sm_count;
-    int blocks = (int)(need < cap ? need : cap);
+    // FP64 searches: as many blocks as nodes need, handed out as SMs come free
+    int blocks = (int)(need < cap || search64_blocks<G, S, MODE>() ? need : cap);
     if (blocks < 1) blocks = 1;
-    kern<<<blocks, B, 0, L.stream>>>(L.g, L.Vin, L.Vout, L.code, L.feet_lo, L.feet_hi, L.inc, L.acc, L.V64,
+    kern<<<blocks, B, smem, L.stream>>>(L.g, L.Vin, L.Vout, L.code, L.feet_lo, L.feet_hi, L.inc, L.acc, L.V64,
                                       L.incr_flags, L.ctl, L.ring, L.ring_mask, L.sweep, L.check_prev, L.tol, L.f64,
                                       L.feet8);
     return cudaGetLastError();
