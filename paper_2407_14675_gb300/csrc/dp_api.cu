@@ -93,6 +93,9 @@ struct dp_grid {
     bool feet8 = false;                     // they are 8-byte words (stored with FP32 values)
     bool store_feet8 = true;                // what the next FP32-value improvements store
     int foot_format = DP_FOOT_AUTO;         // dp_set_foot_format
+    double2* dyn_tables = nullptr;          // FP64 grids: tables of the one-step map, one allocation:
+    double2 *row_dyn = nullptr, *mass_dyn = nullptr;   //   rows, mass nodes, coordinates, running cost
+    double *coord = nullptr, *run_cost = nullptr;
     Feet64 f64;                             // frozen feet of FP64 grids
     bool feet64_valid = false;
     bool diag64_valid = false;              // f64.r holds the factors of these feet
@@ -148,8 +151,8 @@ void free_grid(dp_grid* g)
     if (g->st) cudaStreamSynchronize(g->st);
     void* ps[] = {g->rows, g->row_org, g->lines, g->hi64, g->lo64, g->hi32, g->lo32, g->V[0], g->V[1], g->V64[0],
                   g->V64[1], g->code, g->feet_lo, g->feet_hi, g->acc, g->ctl, g->ring, g->staging,
-                  g->scratch64, g->gm_Q, g->gm_partial, g->gm_ctl, g->f64.w, g->f64.t, g->f64.c, g->f64.r,
-                  g->wave_sync};
+                  g->scratch64, g->gm_Q, g->gm_partial, g->gm_ctl, g->f64.t,
+                  g->wave_sync, g->dyn_tables};
     for (void* p : ps)
         if (p) cudaFree(p);
     if (g->h_ctl) cudaFreeHost(g->h_ctl);
@@ -247,6 +250,16 @@ void fill_geo(const dp_grid* gr, Geo<G>& g)
         g.foot_dm = (int)fl;
         g.foot_tm = um - fl;
     }
+    {
+        G fl = std::floor(g.um);
+        g.um_c = (int)fl;
+        g.um_t = g.um - fl;
+    }
+    g.row_dyn = gr->row_dyn;
+    g.mass_dyn = gr->mass_dyn;
+    g.coord = gr->coord;
+    g.run_cost = gr->run_cost;
+    for (int k = 0; k < 3; ++k) g.hh[k] = 0.5 * d.dt * (1.0 / gr->h[k]);
     g.dyn = d.dynamics;
     const bool polar = d.dynamics == DP_DYN_POLAR;
     g.off = polar && d.off_control;
@@ -1158,9 +1171,15 @@ int dp_grid_create(const dp_grid_desc* desc, dp_grid** out)
     if (g->fp32 && ((rc = dalloc(g, &g->feet_lo, g->n_active)) || (rc = dalloc(g, &g->feet_hi, g->n_active)) ||
                     (rc = dalloc(g, &g->wave_sync, wave_sync_ints(kWaveMaxLevels, g->n_active)))))
         return bail(rc);
-    if (!g->fp32 && ((rc = dalloc(g, &g->f64.w, g->n_active)) || (rc = dalloc(g, &g->f64.t, 2 * g->n_active)) ||
-                     (rc = dalloc(g, &g->f64.c, g->n_active)) || (rc = dalloc(g, &g->f64.r, g->n_active))))
-        return bail(rc);
+    if (!g->fp32) {
+        // FP64 frozen feet, one allocation: fractions (32 bytes a node), then
+        // words, constants and diagonal factors
+        const size_t n = (size_t)g->n_active;
+        if ((rc = dalloc(g, &g->f64.t, n * 7 / 2 + 1))) return bail(rc);
+        g->f64.w = (unsigned long long*)(g->f64.t + 2 * n);
+        g->f64.c = (double*)(g->f64.w + n);
+        g->f64.r = g->f64.c + n;
+    }
     if ((rc = dalloc(g, &g->ctl, 1))) return bail(rc);
     if ((rc = dalloc(g, &g->ring, kRing))) return bail(rc);
     if (cudaMemsetAsync(g->code, 0, sizeof(uint16_t) * g->n_active, g->st) != cudaSuccess ||
@@ -1172,6 +1191,18 @@ int dp_grid_create(const dp_grid_desc* desc, dp_grid** out)
         return bail(fail(DP_ENOMEM, "pinned host allocation failed"));
     }
 
+    if (!g->fp32 && d.dynamics != DP_DYN_UNIT_SPEED) {
+        const bool polar = d.dynamics == DP_DYN_POLAR;
+        const size_t nr = 2 * (size_t)g->n_rows, nm = 2 * (size_t)(polar ? 1 : d.n[3]), nc = 2 * (size_t)kCoordStride;
+        if ((rc = dalloc(g, &g->dyn_tables, nr + nm + nc + (polar ? ((size_t)g->n_active + 1) / 2 : 0)))) return bail(rc);
+        g->row_dyn = g->dyn_tables;
+        g->mass_dyn = g->row_dyn + nr;
+        g->coord = (double*)(g->mass_dyn + nm);
+        if (polar) g->run_cost = g->coord + 2 * nc;
+        fill_geo(g, g->g64);
+        if ((e = launch_dyn_tables(g->g64, g->row_dyn, g->mass_dyn, g->coord, g->run_cost, g->st)) != cudaSuccess)
+            return bail(fail(DP_ECUDA, "one-step map tables: %s", cudaGetErrorString(e)));
+    }
     fill_geo(g, g->g64);
     fill_geo(g, g->g32);
     g->g64.tab_hi = g->hi64;

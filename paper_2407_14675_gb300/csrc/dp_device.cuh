@@ -76,6 +76,8 @@ struct Geo {
     G um;                      // mass displacement in cells, identical at every node
     int foot_dm;               // its cell offset floor(um) and fraction um - floor(um)
     float foot_tm;             //   (grid constants of every frozen foot)
+    int um_c;                  // the same in G (the geometry's own um): offset and fraction
+    G um_t;
     int dyn;
     int K, refine, fib_stop;   // refinement stops once the bracket is <= fib_stop codes
     int fib_n0;                // Fibonacci index of the shortest refinement bracket
@@ -94,7 +96,15 @@ struct Geo {
     double cost_b, cost_g;     // weights of (a - a_bar)^2 and of the eccentricity term
     double a_bar, ex_bar, ey_bar;
     double thrust_cost;        // dt alpha |u| of every thrust control
+    // FP64 grids: what the one-step map needs of a node per row and per mass
+    // node (NULL: computed at the node), and polar grids the running cost
+    const double2* row_dyn;    // per (i_r, i_vr): {1 / r, mu / r^2}, {1 / r_2, mu / r_2^2}, r_2 = r + dt v_r
+    const double2* mass_dyn;   // per i_m (polar: one entry): {dt a/m, a/m + a/m_2}, {b0, b1} of NodeDyn
+    const double* coord;       // node coordinates of dimension d at kCoordStride d
+    const double* run_cost;    // dt l(x_j) per stored node
+    double hh[3];              // half a step over the spacing
 };
+constexpr int kCoordStride = 1024;   // the largest grid dimension
 
 template <typename G> __device__ __forceinline__ G ginf();
 template <> __device__ __forceinline__ float ginf<float>() { return CUDART_INF_F; }
@@ -232,6 +242,43 @@ __device__ __forceinline__ NodeDyn<G> node_dyn(const Geo<G>& g, const StepP<G>& 
             n.a3 = xmul(h3, xfma(n.vt, ir, q));
             n.g3 = xmul(h3, p1r);
         }
+    }
+    return n;
+}
+
+// node_dyn() of a node of an FP64 grid with the parts that a row or a mass
+// node shares read from the grid's tables, the same operations otherwise: 25
+// FP64 operations instead of about 95 (four reciprocals, the coordinates).
+template <int DYN>
+__device__ __forceinline__ NodeDyn<double> node_dyn_table(const Geo<double>& g, const StepP<double>& sp, const int i[4])
+{
+    const int row = i[0] * g.n[1] + i[1];
+    const double2 ra = __ldg(&g.row_dyn[2 * row]), rb = __ldg(&g.row_dyn[2 * row + 1]);
+    const int m = DYN == kDynOrbit ? i[3] : 0;
+    const double2 ma = __ldg(&g.mass_dyn[2 * m]), mb = __ldg(&g.mass_dyn[2 * m + 1]);
+    const double ir = ra.x, ir2 = rb.x, R1 = ma.x, P1 = ma.x, amm = ma.y;
+    NodeDyn<double> n;
+    n.vr = __ldg(&g.coord[kCoordStride + i[1]]);
+    n.vt = __ldg(&g.coord[2 * kCoordStride + i[2]]);
+    const double d1vr = xfma(xmul(n.vt, n.vt), ir, -ra.y);
+    const double d1vt = -xmul(xmul(n.vr, n.vt), ir);
+    const double R0 = xfma(sp.dt, d1vr, n.vr), P0 = xfma(sp.dt, d1vt, n.vt);
+    const double h0 = g.hh[0], h1 = g.hh[1], h2 = g.hh[2];
+    const double q = xmul(P0, ir2), p1r = xmul(P1, ir2);
+    n.a0 = xmul(h0, xadd(n.vr, R0));
+    n.b0 = mb.x;
+    n.a1 = xmul(h1, xadd(d1vr, xfma(P0, q, -rb.y)));
+    n.b1 = mb.y;
+    n.g1 = xmul(h1, xmul(xadd(P1, P1), q));
+    n.d1 = xmul(h1, xmul(P1, p1r));
+    n.a2 = xmul(h2, xfma(-R0, q, d1vt));
+    n.b2 = -xmul(h2, xmul(R1, q));
+    n.g2 = xmul(h2, xfma(-R0, p1r, amm));
+    n.e2 = -xmul(h2, xmul(R1, p1r));
+    if (DYN == kDynPolar) {
+        const double h3 = xmul(sp.hdt, g.ih[3]);
+        n.a3 = xmul(h3, xfma(n.vt, ir, q));
+        n.g3 = xmul(h3, p1r);
     }
     return n;
 }
@@ -769,8 +816,21 @@ struct CachedEval {
     {
         cc[0] = -1;
         pen = (R)((S)g->M64 - vj);
-        if (DYN != kDynPolar) outm = foot_dim(g->n[3], i[3], OFF ? sp.um + u0[3] : sp.um, cm, tm);
-        else outm = false;
+        if (DYN == kDynPolar) {
+            outm = false;
+        } else if (OFF) {
+            outm = foot_dim(g->n[3], i[3], sp.um + u0[3], cm, tm);
+        } else {
+            // foot_dim() of the grid's constant displacement
+            cm = i[3] + g->um_c;
+            tm = g->um_t;
+            outm = false;
+            if ((unsigned)cm > (unsigned)(g->n[3] - 2)) {
+                outm = cm != g->n[3] - 1 || tm > (G)0;
+                cm = g->n[3] - 2;
+                tm = (G)1;
+            }
+        }
     }
 
     // 0 <= t < 1 (false for NaN and -0)
@@ -939,10 +999,12 @@ struct Table {
     const typename V2<G>::type* sc;
     int K;
     int off = 0;     // the lattice code kCodeOff stands for thrust off
+    const float2* scf = nullptr;   // FP64 searches: sc rounded to FP32
 };
 
 template <typename G>
-__device__ __forceinline__ void build_table(const Geo<G>& g, int* code, typename V2<G>::type* sc)
+__device__ __forceinline__ void build_table(const Geo<G>& g, int* code, typename V2<G>::type* sc,
+                                            float2* scf = nullptr)
 {
     for (int k = threadIdx.x; k <= g.K; k += blockDim.x) {
         int c = table_code(g.K, k);
@@ -952,6 +1014,7 @@ __device__ __forceinline__ void build_table(const Geo<G>& g, int* code, typename
             code_sincos(g, c, s, cs);
             sc[k].x = s;
             sc[k].y = cs;
+            if (scf) scf[k] = make_float2((float)s, (float)cs);
         }
     }
 }

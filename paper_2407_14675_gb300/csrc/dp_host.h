@@ -115,6 +115,10 @@ cudaError_t launch_rows(int4* rows, int* err, int n0, int n1, int n2, int n3, co
                         cudaStream_t st);
 cudaError_t launch_row_offsets(int4* rows, int n_rows, int n_m, long long* total, cudaStream_t st,
                                int* org = nullptr);
+// Tables of an FP64 grid's one-step map (Geo::row_dyn, mass_dyn, coord) and,
+// for the polar dynamics, the running cost of every stored node.
+cudaError_t launch_dyn_tables(const Geo<double>& g, double2* rows, double2* mass, double* coord, double* cost,
+                              cudaStream_t st);
 cudaError_t launch_lines(const int4* rows, unsigned* lines, int n0, int n1, int n2, int n_m,
                          cudaStream_t st);
 cudaError_t launch_store_value(const double* src, void* dst, int fp32, int n, const Geo<double>& g, int* bad,

@@ -31,10 +31,11 @@
 // the FP64 evaluations, which at the end of a refinement is what limits it.
 // A point counts only where its fractions are clear of the cell's faces.
 //
-// Measured (GB300, with one-round blocks of 64): a walk sweep of a 31x41x25x17
-// box 0.48 ms, evaluating every angle 1.17; of the paper's 110x30^3 6.1 against
-// 9.9 ms; a value-iteration sweep of 17^4, 16 angles, 78 against 166 us.  FP64
-// instructions a warp of the first: 388 against 864.
+// Measured (GB300, with one-round blocks of 64): a value-iteration sweep of
+// 17^4, 16 angles, 50 us, evaluating every angle 166; a walk sweep of a
+// 31x41x25x17 box 0.34 against 1.17 ms, of the paper's 110x30^3 2.3 against 9.9
+// ms.  Before the one-step map's shared parts came from tables
+// (node_dyn_table()) 78 us, 0.48 and 6.1 ms.
 #pragma once
 
 #include "dp_device.cuh"
@@ -92,47 +93,61 @@ struct Search64 {
 
     __device__ __forceinline__ Search64(E& e) : ev(e) {}
 
+    // A bound of the largest magnitude, from the exponents and leading bits.
+    static __device__ __forceinline__ float top(const double* v, int n)
+    {
+        unsigned b = 0;
+#pragma unroll
+        for (int x = 0; x < n; ++x) b = max(b, (unsigned)__double2hiint(v[x]) & 0x7fffffffu);
+        return (float)__hiloint2double((int)(b + 1u), 0);
+    }
+
     // Evaluates the angle (s0, c0).  kSearchConst: for every angle within
     // `reach` radians of it.
     __device__ __forceinline__ int start(double sd, double cd, float reach)
     {
         const Geo<double>& g = *ev.g;
         const NodeDyn<double>& nd = ev.nd;
-        double u[4], t[4];
+        double u[4], t[4], fl[4];
         int cl[4];
+        float tf[4], uf[4];
         heun_cells<double, DYN>(g, ev.sp, nd, sd, cd, u);
-        bool out = ev.outm;
-#pragma unroll
-        for (int d = 0; d < 3; ++d) out = foot_dim(g.n[d], ev.i[d], u[d], cl[d], t[d]) || out;
-        if (kPolar) out = foot_dim_periodic(g.n[3], ev.i[3], u[3], cl[3], t[3]) || out;
-        else {
-            cl[3] = ev.cm;
-            t[3] = ev.tm;
-        }
         b0 = (float)nd.b0, b1 = (float)nd.b1, g1 = (float)nd.g1, d1 = (float)nd.d1;
         b2 = (float)nd.b2, g2 = (float)nd.g2, e2 = (float)nd.e2, g3 = kPolar ? (float)nd.g3 : 0.0f;
         const float L[4] = {fabsf(b0), fabsf(b1) + fabsf(g1) + fabsf(d1), fabsf(b2) + fabsf(g2) + fabsf(e2), fabsf(g3)};
-        if (out) {
-            bool far = ev.outm;
-#pragma unroll
-            for (int d = 0; d < 3; ++d) {
-                const float pos = (float)ev.i[d] + (float)u[d], r = fmaf(1.001f * reach, L[d], 1e-3f);
-                far = far || pos < -r || pos > (float)(g.n[d] - 1) + r;
-            }
-            return far ? kSearchConst : kSearchOpen;
-        }
-        s0 = (float)sd;
-        c0 = (float)cd;
         face = 4e-6f * (1.0f + L[0] + L[1] + L[2] + L[3]);
-        const float tf[4] = {(float)t[0], (float)t[1], (float)t[2], kPolar ? (float)t[3] : 0.5f};
-        bool in = true, in_all = true;
+        // cell and fractions: the cell from the FP32 displacement, which decides
+        // it wherever the fraction is clear of a face (the displacement's FP32
+        // rounding is part of that margin)
+        bool in = true, in_all = true, box = !ev.outm, far = ev.outm;
 #pragma unroll
         for (int d = 0; d < kDims; ++d) {
-            const float r = fmaf(1.001f * reach, L[d], face);
-            in = in && tf[d] > face && tf[d] < 1.0f - face;
+            uf[d] = (float)u[d];
+            const float fi = floorf(uf[d]), margin = face + 3e-7f * fabsf(uf[d]), r = fmaf(1.001f * reach, L[d], margin);
+            fl[d] = (double)fi;
+            t[d] = u[d] - fl[d];
+            tf[d] = uf[d] - fi;
+            cl[d] = ev.i[d] + (int)fi;
+            in = in && tf[d] > margin && tf[d] < 1.0f - margin;
             in_all = in_all && tf[d] > r && tf[d] < 1.0f - r;
+            if (d < 3) {
+                box = box && (unsigned)cl[d] <= (unsigned)(g.n[d] - 2);
+                const float pos = (float)ev.i[d] + uf[d], rp = r + 1e-3f;
+                far = far || pos < -rp || pos > (float)(g.n[d] - 1) + rp;
+            } else {
+                cl[d] = cl[d] % g.n[d];   // the periodic angle
+                if (cl[d] < 0) cl[d] += g.n[d];
+            }
         }
-        if (!in) return kSearchOpen;
+        if (!kPolar) {
+            cl[3] = ev.cm;
+            t[3] = ev.tm;
+            tf[3] = 0.5f;
+        }
+        if (far) return kSearchConst;
+        if (!in || !box) return kSearchOpen;
+        s0 = (float)sd;
+        c0 = (float)cd;
         mid[0] = tf[0] - b0 * s0;
         mid[1] = tf[1] - fmaf(b1, s0, c0 * fmaf(d1, c0, g1));
         mid[2] = tf[2] - fmaf(b2, s0, c0 * fmaf(e2, s0, g2));
@@ -141,11 +156,11 @@ struct Search64 {
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
             ev.cc[d] = cl[d];
-            ev.co[d] = (double)(cl[d] - ev.i[d]);
+            ev.co[d] = fl[d];
         }
         if (kPolar) {
             ev.cm = cl[3];
-            co3 = floor(u[3]);
+            co3 = fl[3];
         } else {
             ev.K.fold_m(ev.tm);
         }
@@ -167,6 +182,7 @@ struct Search64 {
         const double wa = w[1] - w[0], wb = w[3] - w[2];
         const double x0 = w[0] + t[1] * wa, x1 = w[2] + t[1] * wb, H02 = x1 - x0, G2 = x0 + t[0] * H02;
         const double H012 = wb - wa, H12 = wa + t[0] * H012;
+        float E3 = 0.0f;
         Sd = G0 * nd.b0 + G1 * nd.b1 + G2 * nd.b2;
         Cd = G1 * nd.g1 + G2 * nd.g2;
         if (kPolar) {
@@ -177,6 +193,11 @@ struct Search64 {
                 df[y] = ev.K.de[2 * y] + t[2] * (ev.K.de[2 * y + 1] - ev.K.de[2 * y]);
             const double a0 = df[0] + t[1] * (df[1] - df[0]), a1 = df[2] + t[1] * (df[3] - df[2]);
             Cd += (a0 + t[0] * (a1 - a0)) * nd.g3;
+            // and what is left out: how that derivative varies over the cell
+            double de[8];
+#pragma unroll
+            for (int x = 0; x < 8; ++x) de[x] = ev.K.de[x] - ev.K.de[0];
+            E3 = top(de, 8);
         }
         S = (float)Sd;
         C = (float)Cd;
@@ -187,13 +208,7 @@ struct Search64 {
         asc = h01 * b0 * g1 + h02 * b0 * g2 + h12 * (b1 * g2 + g1 * b2);
         acc = h12 * g1 * g2;
         // largest corner difference, from the exponents and leading bits
-        unsigned eb = 0;
-#pragma unroll
-        for (int x = 0; x < 8; ++x) {
-            eb = max(eb, (unsigned)__double2hiint(ev.K.e0[x]) & 0x7fffffffu);
-            if (kPolar) eb = max(eb, ((unsigned)__double2hiint(ev.K.de[x]) & 0x7fffffffu));
-        }
-        const float E0 = (float)__hiloint2double((int)(eb + 1u), 0) * (kPolar ? 2.0f : 1.0f);
+        const float E0 = top(e, 8);
         float um = 2.0f;
 #pragma unroll
         for (int d = 0; d < 3; ++d) um = fmaxf(um, (float)abs(cl[d] - ev.i[d]) + 1.0f);
@@ -202,9 +217,9 @@ struct Search64 {
         if (!(E0 * Ls > 1e-20f)) return kSearchOpen;
         const float hh = Hs * Ls;
         // slopes, per radian from theta_0: the H terms' rounding and F, Q parts, the angle coordinate's cross terms
-        eh = fmaf(8e-6f * hh, Ls, 6.0f * hh * X) + 32.0f * E0 * L[3] * Ls;
+        eh = fmaf(8e-6f * hh, Ls, 6.0f * hh * X) + 16.0f * E3 * L[3] * Ls;
         et = 3.0f * h012 * L[0] * L[1] * L[2];   // and H_012, per radian squared
-        noise = 2.5e-15f * E0 * (um + 3.0f);
+        noise = 2.5e-15f * E0 * (um + 3.0f);   // half the rounding of a difference: slopes are at most 2 E0
         eps = fmaf(1e-6f, fabsf(S) + fabsf(C), 4e-6f * (fabsf(F) + fabsf(Q))) + 2.0f * eh + 3.0f * et + 2.0f * noise;
         return kSearchCell;
     }
@@ -236,7 +251,23 @@ struct Search64 {
     {
         double t[4];
         fractions(s, c, t);
+        return blend(t);
+    }
+    __device__ __forceinline__ double blend(const double t[4]) const
+    {
         return kPolar ? ev.K.blend(t) : ev.K.blend_m_folded(t);
+    }
+    // Word of a frozen foot in this cell, as CachedEval::foot64_of() forms it.
+    __device__ __forceinline__ unsigned long long foot_word() const
+    {
+        unsigned long long w = (unsigned long long)kFootInside << 32;
+#pragma unroll
+        for (int d = 0; d < 4; ++d) {
+            const int off = (d < 3 ? ev.cc[d] : ev.cm) - ev.i[d];
+            if (off < -128 || off > 127) return (unsigned long long)kFootRecompute << 32;
+            w |= (unsigned long long)(unsigned char)(signed char)off << (8 * d);
+        }
+        return w;
     }
     __device__ __forceinline__ double at_code(int code) const
     {
@@ -260,7 +291,7 @@ struct Search64 {
         float lo = 0.0f;                 // around(angle 0)
         bool in = isfinite(eps);
         for (int k = 1; k < T.K; ++k) {
-            const float s = (float)T.sc[k].x, c = (float)T.sc[k].y;
+            const float s = T.scf[k].x, c = T.scf[k].y;
             in = in && inside(s, c);
             lo = fminf(lo, around(s, c));
         }
@@ -269,7 +300,7 @@ struct Search64 {
         double Db = CUDART_INF;
         kb = 0;
         for (int k = 0; k < T.K; ++k) {
-            while (k < T.K && !((k == 0 ? 0.0f : around((float)T.sc[k].x, (float)T.sc[k].y)) <= lim)) ++k;
+            while (k < T.K && !((k == 0 ? 0.0f : around(T.scf[k].x, T.scf[k].y)) <= lim)) ++k;
             if (k >= T.K) break;
             const double Dk = at_sc(T.sc[k].x, T.sc[k].y);
             if (Dk < Db) { Db = Dk; kb = k; }
@@ -284,7 +315,7 @@ struct Search64 {
     {
         const int K = T.K;
         auto value = [&](int kk, bool& in) {
-            const float s = (float)T.sc[kk].x, c = (float)T.sc[kk].y;
+            const float s = T.scf[kk].x, c = T.scf[kk].y;
             in = in && inside(s, c);
             return around(s, c);
         };
@@ -332,8 +363,8 @@ struct Search64 {
         SlopeModel M;
         {
             const double sd = T.sc[k].x, cd = T.sc[k].y;
-            M.sk = (float)sd;
-            M.ck = (float)cd;
+            M.sk = T.scf[k].x;
+            M.ck = T.scf[k].y;
             if (!inside(M.sk, M.ck, kCodeAngle * (float)max(hi, -a0) * 1.001f)) return false;
             M.p = (float)(Sd * cd - Cd * sd);
             M.q = (float)(Sd * sd + Cd * cd);
@@ -393,12 +424,19 @@ struct Search64 {
     }
 };
 
+// The frozen foot of the chosen code, where the search has it.
+struct FootHint {
+    bool known = false;
+    unsigned long long w;
+    double t[4];
+};
+
 // The search of a node of an FP64 grid: the chosen code and D at it, as
 // walk_table() from k0 (WALK) or enumerate_table() and then, with refine,
 // fibonacci_refine() give them.
 template <bool REDUCED, int DYN, bool WALK, class E>
 __device__ __forceinline__ int search64(E& ev, const Table<double>& T, const Geo<double>& g, int k0, bool refine,
-                                        double& D)
+                                        double& D, FootHint& fh)
 {
     int k = WALK ? k0 : 0;
     const bool fine = !refine || T.K >= kModelMinAngles;
@@ -409,6 +447,9 @@ __device__ __forceinline__ int search64(E& ev, const Table<double>& T, const Geo
         const int how = S.start(T.sc[k].x, T.sc[k].y, WALK ? step : 2.0f);
         if (how == kSearchConst) {
             D = ev.pen;   // nothing is lower than anything
+            fh.known = true;
+            fh.w = (unsigned long long)kFootOut << 32;
+            fh.t[0] = fh.t[1] = fh.t[2] = fh.t[3] = 0.0;
             return T.code[k] & (kCodes - 1);
         }
         if (how == kSearchCell) {
@@ -421,7 +462,12 @@ __device__ __forceinline__ int search64(E& ev, const Table<double>& T, const Geo
                 return T.code[k] & (kCodes - 1);
             }
             if (ok && S.refine(T, g.fib_n0, g.fib_stop, k, code)) {
-                D = S.at_code(code);
+                double s, c;
+                code_sincos(g, code, s, c);
+                S.fractions(s, c, fh.t);
+                D = S.blend(fh.t);
+                fh.known = true;
+                fh.w = S.foot_word();
                 return code;
             }
         }

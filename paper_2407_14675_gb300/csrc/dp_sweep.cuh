@@ -90,9 +90,6 @@ __device__ __forceinline__ S warp_max(S v)
 template <typename G, typename S, int DYN, class E>
 __device__ __forceinline__ void setup_node(E& ev, const Geo<G>& g, const S* __restrict__ V, S vj)
 {
-    G x[4];
-#pragma unroll
-    for (int d = 0; d < 4; ++d) x[d] = g.lo[d] + (G)ev.i[d] * g.h[d];
     ev.g = &g;
     ev.V = V;
     ev.vj = vj;
@@ -101,6 +98,15 @@ __device__ __forceinline__ void setup_node(E& ev, const Geo<G>& g, const S* __re
     ev.sp.um = g.um;
 #pragma unroll
     for (int d = 0; d < 4; ++d) ev.u0[d] = (G)0;
+    if constexpr (std::is_same<G, double>::value && DYN != kDynUnitSpeed) {
+        if (g.row_dyn) {
+            ev.nd = node_dyn_table<DYN>(g, ev.sp, ev.i);
+            return;
+        }
+    }
+    G x[4];
+#pragma unroll
+    for (int d = 0; d < 4; ++d) x[d] = g.lo[d] + (G)ev.i[d] * g.h[d];
     ev.nd = node_dyn<G, DYN>(g, ev.sp, x);
 }
 
@@ -445,7 +451,8 @@ __device__ __forceinline__ void sweep_nodes(const Geo<G>& g, const Table<G>& T, 
                 // thrust-off control, which wins a tie (FP64 grids only)
                 if (!in_target(g, ev.i)) {
                     setup_node<G, S, DYN>(ev, g, Vin, vj);
-                    const double lrun = __dmul_rn(g.dt64, state_cost(g, ev.i));   // rounded on its own: no contraction with the sums below
+                    // rounded on its own: no contraction with the sums below
+                    const double lrun = g.run_cost ? __ldg(&g.run_cost[j]) : __dmul_rn(g.dt64, state_cost(g, ev.i));
                     double q;
                     if constexpr (MODE == kEval) {
                         const int c0 = code[j];
@@ -463,13 +470,14 @@ __device__ __forceinline__ void sweep_nodes(const Geo<G>& g, const Table<G>& T, 
                         ev.reset();
                         typename Eval::R D;
                         int c;
+                        FootHint fh;
                         if constexpr (!kGeo32) {   // polar grids are FP64
                             const int c_old = MODE == kImproveWalk ? (int)code[j] : 0;
                             // a node whose previous control was off has no angle to walk from
                             if (MODE == kImproveWalk && !(g.off && c_old == kCodeOff))
-                                c = search64<REDUCED, DYN, true>(ev, T, g, nearest_index(g.K, c_old), g.refine != 0, D);
+                                c = search64<REDUCED, DYN, true>(ev, T, g, nearest_index(g.K, c_old), g.refine != 0, D, fh);
                             else
-                                c = search64<REDUCED, DYN, false>(ev, T, g, 0, !kIsVI && g.refine, D);
+                                c = search64<REDUCED, DYN, false>(ev, T, g, 0, !kIsVI && g.refine, D, fh);
                         }
                         q = lrun + g.thrust_cost + g.beta64 * ((double)vj + (double)D);
                         if (g.off) {
@@ -483,11 +491,14 @@ __device__ __forceinline__ void sweep_nodes(const Geo<G>& g, const Table<G>& T, 
                         if constexpr (!kGeo32 && kImprove) {
                             if (f64.w) {
                                 const bool off = g.off && c == kCodeOff;
-                                G sn = (G)0, cs = (G)0, t[4];
-                                if (!off) code_sincos(g, c, sn, cs);
-                                f64.w[j] = ev.foot64_of(sn, cs, t);
-                                f64.t[2 * (size_t)j] = make_double2((double)t[0], (double)t[1]);
-                                f64.t[2 * (size_t)j + 1] = make_double2((double)t[2], (double)t[3]);
+                                if (off || !fh.known) {
+                                    G sn = (G)0, cs = (G)0;
+                                    if (!off) code_sincos(g, c, sn, cs);
+                                    fh.w = ev.foot64_of(sn, cs, fh.t);
+                                }
+                                f64.w[j] = fh.w;
+                                f64.t[2 * (size_t)j] = make_double2(fh.t[0], fh.t[1]);
+                                f64.t[2 * (size_t)j + 1] = make_double2(fh.t[2], fh.t[3]);
                                 f64.c[j] = off ? lrun : lrun + g.thrust_cost;
                             }
                         }
@@ -509,11 +520,13 @@ __device__ __forceinline__ void sweep_nodes(const Geo<G>& g, const Table<G>& T, 
                     ev.reset();
                     const int c_old = (MODE == kImproveWalk || kPolish) ? (int)code[j] : 0;
                     int c;
+                    FootHint fh;
+                    (void)fh;
                     if constexpr (kModel) {
                         if constexpr (MODE == kImproveWalk)
-                            c = search64<REDUCED, DYN, true>(ev, T, g, nearest_index(g.K, c_old), g.refine != 0, D);
+                            c = search64<REDUCED, DYN, true>(ev, T, g, nearest_index(g.K, c_old), g.refine != 0, D, fh);
                         else
-                            c = search64<REDUCED, DYN, false>(ev, T, g, 0, !kIsVI && g.refine, D);
+                            c = search64<REDUCED, DYN, false>(ev, T, g, 0, !kIsVI && g.refine, D, fh);
                     } else {
                         int k;
                         if (MODE == kImproveWalk)
@@ -575,11 +588,14 @@ __device__ __forceinline__ void sweep_nodes(const Geo<G>& g, const Table<G>& T, 
                     }
                     if constexpr (!kGeo32 && kImprove) {
                         if (f64.w) {
-                            G sn, cs, t[4];
-                            code_sincos(g, c, sn, cs);
-                            f64.w[j] = ev.foot64_of(sn, cs, t);
-                            f64.t[2 * (size_t)j] = make_double2((double)t[0], (double)t[1]);
-                            f64.t[2 * (size_t)j + 1] = make_double2((double)t[2], (double)t[3]);
+                            if (!fh.known) {
+                                G sn, cs;
+                                code_sincos(g, c, sn, cs);
+                                fh.w = ev.foot64_of(sn, cs, fh.t);
+                            }
+                            f64.w[j] = fh.w;
+                            f64.t[2 * (size_t)j] = make_double2(fh.t[0], fh.t[1]);
+                            f64.t[2 * (size_t)j + 1] = make_double2(fh.t[2], fh.t[3]);
                             f64.c[j] = g.dt64;
                         }
                     }
@@ -671,7 +687,10 @@ __host__ __device__ constexpr int big_block()
 // FP64 searches run many small blocks, one round each (no grid-stride): the
 // FP64 pipe of an SM is the bound, so what counts is an even share per SM, and
 // nodes differ in how much FP64 they need.  The 17^4 box in 256-thread blocks,
-// two resident per SM, took two rounds for 1.07 of nodes.
+// two resident per SM, took two rounds for 1.07 of nodes.  Resident blocks (the
+// registers they leave): 8 for value iteration (2.95 ms for 50 sweeps of 17^4;
+// 7: 2.93, 10: 3.30, 12: 4.25), 5 for the improvements (24.6 ms for two outer
+// steps of the paper's 110x30^3; 4: 25.0, 8 with spills: 25.5).
 constexpr int kSearch64Block = 64;
 
 template <typename G, typename S, int MODE>
@@ -692,7 +711,7 @@ constexpr int min_blocks()
 {
     constexpr bool feet64 = MODE == kEvalFeet64 || MODE == kEvalFeet64Diag;
     if (BIG) return feet64 ? 1 : 2;
-    if (search64_blocks<G, S, MODE>()) return MODE == kVI ? 10 : 8;   // 96 and 128 registers
+    if (search64_blocks<G, S, MODE>()) return MODE == kVI ? 8 : 5;
     // FP32 angle searches: 3 blocks of 256 per SM (80 registers).  Left to
     // itself the compiler gives the reduced-grid walk 96 registers (2 blocks):
     // 4.84 against 4.36 ms per sweep on the 121^4 band
@@ -730,12 +749,14 @@ sweep_kernel(const __grid_constant__ Geo<G> g, const S* __restrict__ Vin, S* __r
     // (sized by the table, so that the rest of it stays L1)
     extern __shared__ __align__(16) unsigned char s_table[];
     typename V2<G>::type* s_sc = reinterpret_cast<typename V2<G>::type*>(s_table);
-    int* s_code = reinterpret_cast<int*>(s_sc + (kSearch ? g.K : 0));
+    constexpr bool kTab32 = search64_blocks<G, S, MODE>();
+    float2* s_scf = kTab32 ? reinterpret_cast<float2*>(s_sc + g.K) : nullptr;
+    int* s_code = kTab32 ? reinterpret_cast<int*>(s_scf + g.K) : reinterpret_cast<int*>(s_sc + (kSearch ? g.K : 0));
     if constexpr (kSearch) {
-        build_table(g, s_code, s_sc);
+        build_table(g, s_code, s_sc, s_scf);
         __syncthreads();
     }
-    const Table<G> T{s_code, s_sc, g.K, g.off};
+    const Table<G> T{s_code, s_sc, g.K, g.off, s_scf};
 
     S resid = (S)0;
     bool bad = false;
@@ -760,7 +781,9 @@ cudaError_t launch_sized(const SweepLaunch<G, S>& L)
     auto kern = sweep_kernel<G, S, MODE, REDUCED, DYN, BIG>;
     constexpr int B = sweep_block<G, S, MODE, REDUCED, BIG>();
     constexpr bool kSearch = MODE == kVI || MODE == kVIDiag || MODE == kImproveFull || MODE == kImproveWalk;
-    const size_t smem = kSearch ? (size_t)L.g.K * sizeof(typename V2<G>::type) + (size_t)(L.g.K + 1) * sizeof(int) : 0;
+    const size_t smem = kSearch ? (size_t)L.g.K * (sizeof(typename V2<G>::type) + (search64_blocks<G, S, MODE>() ? 8 : 0)) +
+                                      (size_t)(L.g.K + 1) * sizeof(int)
+                                : 0;
     static int per_sm = 0;
     if (per_sm == 0) {
         cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, B, smem);
