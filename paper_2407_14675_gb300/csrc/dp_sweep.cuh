@@ -294,7 +294,15 @@ __device__ __forceinline__ void sweep_nodes(const Geo<G>& g, const Table<G>& T, 
         const bool first = incr_flags & 1;   // diagonal-solved: store the factors
         constexpr unsigned long long kInf = 0x7ff0000000000000ull;
         unsigned long long rbits = 0;
-        for (int j = j0; j < end; j += stride) {
+        // Whole rounds of the grid, then the remaining nodes in equal shares per
+        // block: handed out in blocks of 1024 they would keep some SMs for a
+        // whole round more (the 31x41x25x17 box is 3.5 rounds: 53 against 60 us)
+        const int rounds = end / stride, rest = end - rounds * stride;
+        const int share = (rest + 32 * (int)gridDim.x - 1) / (32 * (int)gridDim.x) * 32;
+        for (int it = 0; it <= rounds; ++it) {
+            const long long last = (long long)rounds * stride + (long long)blockIdx.x * share + threadIdx.x;
+            if (it == rounds && ((int)threadIdx.x >= share || last >= end)) break;
+            const int j = it < rounds ? j0 + it * stride : (int)last;
             const S vj = Vin[j];
             const unsigned long long w = __ldcs(&f64.w[j]);
             const int kind = (int)((w >> 32) & 3u);
