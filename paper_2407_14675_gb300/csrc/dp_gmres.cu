@@ -14,59 +14,80 @@
 //   optionally twice), y = argmin ||beta0 e1 - H y||, V <- V + Q y.
 // The basis vectors are stored unnormalised, with scale[i] = 1 / ||Q_i||.
 // An Arnoldi step is three launches: the product (gather-bound, one node per
-// thread at the evaluation sweep's occupancy), the projections, and the
-// update with the norm (both streaming, tiles of kGmTile nodes with 16-byte
-// loads).  A streaming launch sums its dot products per block into a partial
-// row, and the last block to finish adds the rows in a fixed order (the
-// result does not depend on block scheduling) and does the O(m) Hessenberg
-// and Givens work on one thread.  No block waits for another.
+// thread at the evaluation sweep's occupancy), the projections, and the update
+// with the norm.  The streaming launches give every block an equal contiguous
+// share of the vectors in 16-byte loads, eight vectors at a time.  A launch
+// sums its dot products per block into a partial row, and the last block to
+// finish adds the rows in a fixed order (the result does not depend on block
+// scheduling) and does the Hessenberg and Givens work from shared memory.  No
+// block waits for another.
 //
-// Element-wise work and the warp reductions run in the basis precision VT
-// (FP32 on FP32 grids: the FP64 pipe of this GPU is a small fraction of its
-// FP32 pipe, and FP64 adds in every lane of the warp trees made the
-// orthogonalisation FP64-bound).  Each warp's total over 128 products is
-// widened to FP64 for the block and grid sums and the Hessenberg problem.
+// Element-wise work runs in the basis precision VT (FP32 on FP32 grids: the
+// FP64 pipe of this GPU is a small fraction of its FP32 pipe).  A thread sums
+// its share of a dot product as a pair of floats (TwoSum, so that long shares
+// lose nothing) and the warp's lanes are combined the same way; the warps'
+// totals are widened to FP64 for the block and grid sums and the Hessenberg
+// problem.
+#include <algorithm>
+
 #include "dp_sweep.cuh"
 
 namespace dpk {
 namespace {
 
 constexpr int kGmBlock = 256;
-constexpr int kGmS = 4;                     // nodes per thread and tile (four consecutive
-                                            // nodes per thread in the streaming loops)
-constexpr int kGmTile = kGmBlock * kGmS;
 constexpr int kGmWarps = kGmBlock / 32;
+constexpr int kGmCols = 8;                  // vectors read at a time by the streaming kernels
+constexpr int kGmStreamBlocks = 4;          // blocks per SM of the streaming kernels, at most
 
-template <typename T>
-__device__ __forceinline__ T warp_sum(T v)
-{
+// A running sum: FP32 terms as an unevaluated pair of floats (Knuth's TwoSum
+// keeps what each addition rounds off), FP64 terms plainly.
+template <typename T> struct Acc;
+template <> struct Acc<float> {
+    float hi = 0.0f, lo = 0.0f;
+    __device__ __forceinline__ void add(float x)
+    {
+        const float s = __fadd_rn(hi, x), b = __fadd_rn(s, -hi);
+        lo = __fadd_rn(lo, __fadd_rn(__fadd_rn(hi, -__fadd_rn(s, -b)), __fadd_rn(x, -b)));
+        hi = s;
+    }
+    __device__ __forceinline__ double warp_total()
+    {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
+        for (int o = 16; o > 0; o >>= 1) {
+            const float h = __shfl_xor_sync(0xffffffffu, hi, o), l = __shfl_xor_sync(0xffffffffu, lo, o);
+            add(h);
+            lo = __fadd_rn(lo, l);
+        }
+        return (double)hi + (double)lo;
+    }
+};
+template <> struct Acc<double> {
+    double v = 0.0;
+    __device__ __forceinline__ void add(double x) { v += x; }
+    __device__ __forceinline__ double warp_total()
+    {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        return v;
+    }
+};
 
-// Per-block sums: every warp adds into its own row.
+// Per-block sums: a row per warp.
 struct BlockSums {
     double acc[kGmWarps][kGmLd];
 };
 
-__device__ __forceinline__ void sums_zero(BlockSums& S)
-{
-    for (int c = threadIdx.x; c < kGmWarps * kGmLd; c += kGmBlock) (&S.acc[0][0])[c] = 0.0;
-    __syncthreads();
-}
-
-// Adds the warp's total of v to column c.  Every lane of the warp calls it.
-// The warp tree runs in v's precision (a pairwise sum of 32 per-thread
-// partials); only its total is widened to FP64.
+// The warp's total of a thread's sum into its row's column c.  Every lane of
+// the warp calls it, once per column.
 template <typename T>
-__device__ __forceinline__ void sums_add(BlockSums& S, int c, T v)
+__device__ __forceinline__ void sums_put(BlockSums& S, int c, Acc<T> a)
 {
-    v = warp_sum(v);
-    if ((threadIdx.x & 31) == 0) S.acc[threadIdx.x >> 5][c] += (double)v;
+    const double v = a.warp_total();
+    if ((threadIdx.x & 31) == 0) S.acc[threadIdx.x >> 5][c] = v;
 }
 
-// Stores the block's columns [0, ncol) in its partial row.  Returns true in
+// Stores the block's columns [0, ncol) among the partial sums (column by column).  Returns true in
 // every thread of the last block to finish, with red[c] = the sum over all
 // blocks (lane-strided over blocks, then a fixed shuffle tree).
 __device__ bool sums_finish(BlockSums& S, int ncol, double* __restrict__ partial, GmCtl* gc, double* red)
@@ -77,7 +98,7 @@ __device__ bool sums_finish(BlockSums& S, int ncol, double* __restrict__ partial
         double v = 0.0;
 #pragma unroll
         for (int w = 0; w < kGmWarps; ++w) v += S.acc[w][c];
-        partial[(size_t)blockIdx.x * kGmLd + c] = v;
+        partial[(size_t)c * gridDim.x + blockIdx.x] = v;
     }
     __threadfence();
     __syncthreads();
@@ -87,14 +108,23 @@ __device__ bool sums_finish(BlockSums& S, int ncol, double* __restrict__ partial
     __threadfence();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     for (int c = warp; c < ncol; c += kGmWarps) {
-        double v = 0.0;
-        for (int b = lane; b < (int)gridDim.x; b += 32) v += __ldcg(&partial[(size_t)b * kGmLd + c]);
-        v = warp_sum(v);
+        Acc<double> a;
+#pragma unroll 8
+        for (int b = lane; b < (int)gridDim.x; b += 32) a.add(__ldcg(&partial[(size_t)c * gridDim.x + b]));
+        const double v = a.warp_total();
         if (lane == 0) red[c] = v;
     }
     __syncthreads();
     if (threadIdx.x == 0) gc->counter = 0;
     return true;
+}
+
+// This block's share [first, last) of the vectors' 4-entry groups.
+__device__ __forceinline__ void share(int n, int& first, int& last)
+{
+    const int n4 = (n >> 2) + ((n & 3) != 0), per = n4 / (int)gridDim.x, more = n4 % (int)gridDim.x;
+    first = (int)blockIdx.x * per + min((int)blockIdx.x, more);
+    last = first + per + ((int)blockIdx.x < more ? 1 : 0);
 }
 
 // Four consecutive entries j4..j4+3 of a vector (j4 a multiple of 4 and the
@@ -207,23 +237,26 @@ gm_start_kernel(const VV* __restrict__ Vin, const VV* __restrict__ Vnext, VT* __
 {
     __shared__ BlockSums S;
     __shared__ double red[kGmLd];
-    sums_zero(S);
-    const int tiles = (n + kGmTile - 1) / kGmTile;
-    for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
-        const int j4 = tile * kGmTile + kGmS * threadIdx.x;
-        VV a[kGmS], b[kGmS];
-        VT r[kGmS];
+    Acc<VT> nrm;
+    int first, last;
+    share(n, first, last);
+#pragma unroll 2
+    for (int e = first + (int)threadIdx.x; e < last; e += kGmBlock) {
+        const int j4 = 4 * e;
+        VV a[4], b[4];
+        VT r[4];
         load4(Vin, j4, n, a);
         load4(Vnext, j4, n, b);
-        VT nrm = (VT)0;
+        VT d = (VT)0;
 #pragma unroll
-        for (int s = 0; s < kGmS; ++s) {
+        for (int s = 0; s < 4; ++s) {
             r[s] = (VT)(b[s] - a[s]);
-            nrm += r[s] * r[s];
+            d += r[s] * r[s];
         }
         store4(q0, j4, n, r);
-        sums_add(S, 0, nrm);
+        nrm.add(d);
     }
+    sums_put(S, 0, nrm);
     if (!sums_finish(S, 1, partial, gc, red)) return;
     if (threadIdx.x == 0) {
         const double b = sqrt(red[0]);
@@ -288,108 +321,216 @@ gm_matvec_kernel(const __grid_constant__ Geo<G> g, VT* __restrict__ Q, long long
 
 // Closes column k once ||Q_{k+1}||^2 is known: rotations, residual estimate,
 // and, when the cycle ends, the back substitution R y = g into coef (as
-// coefficients of the raw Q_i).  One thread.
-__device__ void finalize_column(GmCtl* gc, int k, int m, double rtol, double nrm2)
+// coefficients of the raw Q_i).  A whole block: what the recurrences read is
+// copied to shared memory first, in parallel (read from memory step by step by
+// one thread, the column's loads alone took several microseconds, and the
+// k^2 / 2 of the substitution tens of them).
+__device__ void finalize_column(GmCtl* gc, int k, int m, double rtol, double nrm2, double* sR, double* sh)
 {
-    const double nu = sqrt(fmax(nrm2, 0.0));
-    for (int i = 0; i < k; ++i) {
-        const double a = gc->H[i][k], b = gc->H[i + 1][k];
-        gc->H[i][k] = gc->cs[i] * a + gc->sn[i] * b;
-        gc->H[i + 1][k] = -gc->sn[i] * a + gc->cs[i] * b;
+    double* hc = sh;                               // column k
+    double* cs = sh + kGmMaxRestart + 1;
+    double* sn = cs + kGmMaxRestart;
+    __shared__ int s_kk, s_stop;
+    const int tid = threadIdx.x;
+    for (int i = tid; i <= k; i += kGmBlock) hc[i] = gc->H[i][k];
+    for (int i = tid; i < k; i += kGmBlock) {
+        cs[i] = gc->cs[i];
+        sn[i] = gc->sn[i];
     }
-    const double a = gc->H[k][k];
-    const double r = hypot(a, nu);
-    int kk = k + 1;
-    bool stop = kk >= m;
-    if (!(r > 0.0) || !isfinite(r)) {
-        kk = k;             // no usable column: solve with the previous ones
-        stop = true;
-    } else {
-        const double c = a / r, s = nu / r;
-        gc->cs[k] = c;
-        gc->sn[k] = s;
-        gc->H[k][k] = r;
-        gc->H[k + 1][k] = 0.0;
-        gc->gv[k + 1] = -s * gc->gv[k];
-        gc->gv[k] = c * gc->gv[k];
-        gc->scale[k + 1] = nu > 0.0 ? 1.0 / nu : 0.0;
-        gc->rel = fabs(gc->gv[k + 1]) / gc->beta0;
-        // converged, or the Krylov space is (numerically) invariant
-        if (gc->rel <= rtol || !(nu > 1e-14 * r)) stop = true;
-    }
-    gc->k = kk;
-    if (stop) {
-        for (int i = kk - 1; i >= 0; --i) {
-            double v = gc->gv[i];
-            for (int l = i + 1; l < kk; ++l) v -= gc->H[i][l] * gc->coef[l];
-            gc->coef[i] = v / gc->H[i][i];
+    __syncthreads();
+    if (tid == 0) {
+        const double nu = sqrt(fmax(nrm2, 0.0));
+        for (int i = 0; i < k; ++i) {
+            const double a = hc[i], b = hc[i + 1];
+            hc[i] = cs[i] * a + sn[i] * b;
+            hc[i + 1] = -sn[i] * a + cs[i] * b;
         }
-        for (int i = 0; i < kk; ++i) gc->coef[i] *= gc->scale[i];
-        gc->done = 1;
+        const double a = hc[k];
+        const double r = hypot(a, nu);
+        int kk = k + 1;
+        bool stop = kk >= m;
+        if (!(r > 0.0) || !isfinite(r)) {
+            kk = k;             // no usable column: solve with the previous ones
+            stop = true;
+        } else {
+            const double c = a / r, s = nu / r;
+            gc->cs[k] = c;
+            gc->sn[k] = s;
+            hc[k] = r;
+            gc->H[k + 1][k] = 0.0;
+            const double g = gc->gv[k], g1 = -s * g;
+            gc->gv[k + 1] = g1;
+            gc->gv[k] = c * g;
+            gc->scale[k + 1] = nu > 0.0 ? 1.0 / nu : 0.0;
+            gc->rel = fabs(g1) / gc->beta0;
+            // converged, or the Krylov space is (numerically) invariant
+            if (fabs(g1) / gc->beta0 <= rtol || !(nu > 1e-14 * r)) stop = true;
+        }
+        gc->k = kk;
+        s_kk = kk;
+        s_stop = stop;
+    }
+    __syncthreads();
+    for (int i = tid; i <= k; i += kGmBlock) gc->H[i][k] = hc[i];
+    if (!s_stop) return;
+    // R (upper triangle, kk x kk) and g to shared memory, then column by column
+    const int kk = s_kk;
+    __syncthreads();
+    for (int e = tid; e < kk * kk; e += kGmBlock) {
+        const int i = e / kk, l = e % kk;
+        if (l >= i) sR[i * kGmMaxRestart + l] = l == k ? hc[i] : gc->H[i][l];
+    }
+    double* y = hc;   // hc is stored
+    __syncthreads();
+    for (int i = tid; i < kk; i += kGmBlock) y[i] = gc->gv[i];
+    __syncthreads();
+    if (tid < 32) {
+        for (int i = kk - 1; i >= 0; --i) {
+            const double c = y[i] / sR[i * kGmMaxRestart + i];
+            __syncwarp();
+            if (tid == 0) y[i] = c;
+            for (int l = tid; l < i; l += 32) y[l] -= sR[l * kGmMaxRestart + i] * c;
+            __syncwarp();
+        }
+        for (int i = tid; i < kk; i += 32) gc->coef[i] = y[i] * gc->scale[i];
+        if (tid == 0) gc->done = 1;
     }
 }
 
-// Arnoldi step k, Gram-Schmidt on Q_{k+1}.  SUB: Q_{k+1} -= sum_i coef_i Q_i.
-// DOTS: the projections h_ik = <q_i, Q_{k+1}> of the result, which set column
-// k of H (first pass, !SUB) or correct it (second pass) and become the next
-// coefficients; otherwise the norm that closes the column.
-template <typename VT, bool SUB, bool DOTS>
-__global__ void __launch_bounds__(kGmBlock)
-gm_update_kernel(VT* __restrict__ Q, long long ldq, int n, int k, int m, double rtol, double* __restrict__ partial,
-                 GmCtl* __restrict__ gc)
+// Vectors are read in equal groups of at most kGmCols: 9 as 5 and 4, not 8 and
+// 1, so that every pass keeps enough loads in flight.
+__host__ __device__ constexpr int group_width(int count)
+{
+    const int groups = (count + kGmCols - 1) / kGmCols;
+    return (count + groups - 1) / groups;
+}
+
+// Runs f with a compile-time width.
+template <int N> struct Width { static constexpr int n = N; };
+template <class F>
+__device__ __forceinline__ void with_width(int w, F f)
+{
+    switch (w) {
+    case 1: f(Width<1>()); break;
+    case 2: f(Width<2>()); break;
+    case 3: f(Width<3>()); break;
+    case 4: f(Width<4>()); break;
+    case 5: f(Width<5>()); break;
+    case 6: f(Width<6>()); break;
+    case 7: f(Width<7>()); break;
+    default: f(Width<8>()); break;
+    }
+}
+
+// Arnoldi step k, the projections h_ik = <q_i, Q_{k+1}>: they set column k of
+// H (SECOND: correct it, the second pass of Gram-Schmidt) and become the next
+// coefficients.  A thread reads up to eight vectors at a time and keeps their
+// sums in registers; the vector itself is read again for the next group.  41^4
+// in FP32 (11.3 MB a vector), ten vectors on average: 33 us cold; one tile of
+// 1,024 nodes at a time with a widened shared-memory addition per warp, vector
+// and tile, which the FP64 pipe bounded at 45 %, 55 us; groups of eight and a
+// remainder read one vector after another 40.
+template <typename VT, bool SECOND>
+__global__ void __launch_bounds__(kGmBlock, sizeof(VT) == 4 ? kGmStreamBlocks : 2)
+gm_dots_kernel(const VT* __restrict__ Q, long long ldq, int n, int k, double* __restrict__ partial,
+               GmCtl* __restrict__ gc)
 {
     if (*(volatile int*)&gc->done) return;
     __shared__ BlockSums S;
     __shared__ double red[kGmLd];
-    __shared__ VT s_coef[kGmMaxRestart + 1];
-    if (SUB)
-        for (int i = threadIdx.x; i <= k; i += kGmBlock) s_coef[i] = (VT)gc->coef[i];
-    sums_zero(S);
-    VT* w = Q + (size_t)(k + 1) * ldq;
-    const int tiles = (n + kGmTile - 1) / kGmTile;
-    for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
-        const int j4 = tile * kGmTile + kGmS * threadIdx.x;
-        VT wv[kGmS];
-        load4(w, j4, n, wv);
-        if constexpr (SUB) {
-#pragma unroll 4
-            for (int i = 0; i <= k; ++i) {
-                VT q[kGmS];
-                load4(Q + (size_t)i * ldq, j4, n, q);
-                const VT c = s_coef[i];
+    const VT* w = Q + (size_t)(k + 1) * ldq;
+    int first, last;
+    share(n, first, last);
+    const int width = group_width(k + 1);
+    for (int i0 = 0; i0 <= k; i0 += width) {
+        const VT* q0 = Q + (size_t)i0 * ldq;
+        with_width(min(width, k + 1 - i0), [&](auto wt) {
+            constexpr int W = decltype(wt)::n;
+            Acc<VT> acc[W];
+            for (int e = first + (int)threadIdx.x; e < last; e += kGmBlock) {
+                VT wv[4], q[W][4];
+                load4(w, 4 * e, n, wv);
 #pragma unroll
-                for (int s = 0; s < kGmS; ++s) wv[s] -= c * q[s];
+                for (int c = 0; c < W; ++c) load4(q0 + (size_t)c * ldq, 4 * e, n, q[c]);
+#pragma unroll
+                for (int c = 0; c < W; ++c) {
+                    VT d = (VT)0;
+#pragma unroll
+                    for (int s = 0; s < 4; ++s) d += q[c][s] * wv[s];
+                    acc[c].add(d);
+                }
             }
-            store4(w, j4, n, wv);
-        }
-        VT nrm = (VT)0;
 #pragma unroll
-        for (int s = 0; s < kGmS; ++s) nrm += wv[s] * wv[s];
-        if constexpr (DOTS) {
-#pragma unroll 4
-            for (int i = 0; i <= k; ++i) {
-                VT q[kGmS];
-                load4(Q + (size_t)i * ldq, j4, n, q);
-                VT d = (VT)0;
+            for (int c = 0; c < W; ++c) sums_put(S, i0 + c, acc[c]);
+        });
+    }
+    if (!sums_finish(S, k + 1, partial, gc, red)) return;
+    for (int i = threadIdx.x; i <= k; i += kGmBlock) {
+        const double h = gc->scale[i] * red[i];
+        gc->H[i][k] = SECOND ? gc->H[i][k] + h : h;
+        gc->coef[i] = h * gc->scale[i];
+    }
+}
+
+// v += sum over i < count of coef_i Q_i at the 4-entry group e, the vectors in
+// groups of W; coefficients past the last are 0 (their loads repeat it).
+template <int W, typename VT>
+__device__ __forceinline__ void combine(const VT* __restrict__ Q, long long ldq, int n, int e, int count,
+                                        const VT* coef, VT v[4])
+{
+    for (int i = 0; i < count; i += W) {
+        VT q[W][4];
 #pragma unroll
-                for (int s = 0; s < kGmS; ++s) d += q[s] * wv[s];
-                sums_add(S, i, d);
-            }
-        } else {
-            sums_add(S, 0, nrm);
+        for (int c = 0; c < W; ++c) load4(Q + (size_t)min(i + c, count - 1) * ldq, 4 * e, n, q[c]);
+#pragma unroll
+        for (int c = 0; c < W; ++c) {
+            const VT x = coef[i + c];
+#pragma unroll
+            for (int s = 0; s < 4; ++s) v[s] += x * q[c][s];
         }
     }
-    if (!sums_finish(S, DOTS ? k + 1 : 1, partial, gc, red)) return;
-    if (threadIdx.x == 0) {
-        if constexpr (DOTS) {
-            for (int i = 0; i <= k; ++i) {
-                const double h = gc->scale[i] * red[i];
-                gc->H[i][k] = SUB ? gc->H[i][k] + h : h;
-                gc->coef[i] = h * gc->scale[i];
+}
+
+// Q_{k+1} -= sum_i coef_i Q_i, and (NORM) the norm that closes the column.
+// Groups of vectors as the projections read them; each block walks its share
+// backwards, from the end that the projections read last and L2 still holds.
+// 34 us cold at ten vectors of 41^4; 47 with tiles of 1,024 nodes, four loads
+// in flight and the column closed by one thread from memory.
+template <typename VT, bool NORM>
+__global__ void __launch_bounds__(kGmBlock, sizeof(VT) == 4 ? kGmStreamBlocks : 2)
+gm_update_kernel(VT* __restrict__ Q, long long ldq, int n, int k, int m, double rtol, double* __restrict__ partial,
+                 GmCtl* __restrict__ gc)
+{
+    if (*(volatile int*)&gc->done) return;
+    // the sums of the norm, then the last block's copy of R
+    __shared__ union { BlockSums S; double R[kGmMaxRestart * kGmMaxRestart]; } U;
+    __shared__ double red[kGmLd], sh[3 * kGmMaxRestart + 1];
+    __shared__ VT s_coef[kGmMaxRestart + 1 + kGmCols];
+    for (int i = threadIdx.x; i <= k + kGmCols; i += kGmBlock) s_coef[i] = i <= k ? -(VT)gc->coef[i] : (VT)0;
+    __syncthreads();
+    VT* w = Q + (size_t)(k + 1) * ldq;
+    Acc<VT> nrm;
+    int first, last;
+    share(n, first, last);
+    with_width(group_width(k + 1), [&](auto wt) {
+        constexpr int W = decltype(wt)::n;
+        for (int e = last - 1 - (int)threadIdx.x; e >= first; e -= kGmBlock) {
+            VT wv[4];
+            load4(w, 4 * e, n, wv);
+            combine<W>(Q, ldq, n, e, k + 1, s_coef, wv);
+            store4(w, 4 * e, n, wv);
+            if constexpr (NORM) {
+                VT d = (VT)0;
+#pragma unroll
+                for (int s = 0; s < 4; ++s) d += wv[s] * wv[s];
+                nrm.add(d);
             }
-        } else {
-            finalize_column(gc, k, m, rtol, red[0]);
         }
+    });
+    if constexpr (NORM) {
+        sums_put(U.S, 0, nrm);
+        if (!sums_finish(U.S, 1, partial, gc, red)) return;
+        finalize_column(gc, k, m, rtol, red[0], U.R, sh);
     }
 }
 
@@ -400,34 +541,28 @@ __global__ void __launch_bounds__(kGmBlock)
 gm_apply_kernel(const VV* __restrict__ Vin, VV* __restrict__ Vnext, const VT* __restrict__ Q, long long ldq, int n,
                 const GmCtl* __restrict__ gc, Ctl* __restrict__ ctl)
 {
-    __shared__ VT s_coef[kGmMaxRestart + 1];
+    __shared__ VT s_coef[kGmMaxRestart + kGmCols];
     const int kk = gc->k;
-    for (int i = threadIdx.x; i < kk; i += kGmBlock) s_coef[i] = (VT)gc->coef[i];
+    for (int i = threadIdx.x; i < kk + kGmCols; i += kGmBlock) s_coef[i] = i < kk ? (VT)gc->coef[i] : (VT)0;
     __syncthreads();
     bool bad = false;
-    const int tiles = (n + kGmTile - 1) / kGmTile;
-    for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
-        const int j4 = tile * kGmTile + kGmS * threadIdx.x;
-        VT e[kGmS];
+    int first, last;
+    share(n, first, last);
+    with_width(kk > 0 ? group_width(kk) : 1, [&](auto wt) {
+        constexpr int W = decltype(wt)::n;
+        for (int e = first + (int)threadIdx.x; e < last; e += kGmBlock) {
+            VT x[4] = {(VT)0, (VT)0, (VT)0, (VT)0};
+            VV v[4];
+            load4(Vin, 4 * e, n, v);
+            combine<W>(Q, ldq, n, e, kk, s_coef, x);
 #pragma unroll
-        for (int s = 0; s < kGmS; ++s) e[s] = (VT)0;
-#pragma unroll 4
-        for (int i = 0; i < kk; ++i) {
-            VT q[kGmS];
-            load4(Q + (size_t)i * ldq, j4, n, q);
-            const VT c = s_coef[i];
-#pragma unroll
-            for (int s = 0; s < kGmS; ++s) e[s] += c * q[s];
+            for (int s = 0; s < 4; ++s) {
+                v[s] += (VV)x[s];
+                bad = bad || (4 * e + s < n && !isfinite(v[s]));
+            }
+            store4(Vnext, 4 * e, n, v);
         }
-        VV v[kGmS];
-        load4(Vin, j4, n, v);
-#pragma unroll
-        for (int s = 0; s < kGmS; ++s) {
-            v[s] += (VV)e[s];
-            bad = bad || (j4 + s < n && !isfinite(v[s]));
-        }
-        store4(Vnext, j4, n, v);
-    }
+    });
     if (__syncthreads_or(bad) && threadIdx.x == 0) atomicOr(&ctl->nonfinite, 1);
 }
 
@@ -454,19 +589,19 @@ feet_kernel(const __grid_constant__ Geo<float> g, const uint16_t* __restrict__ c
     }
 }
 
-// Blocks for a tiled launch: resident blocks on every SM, at most one per
-// tile and at most max_blocks (rows of the partial-sum buffer).
+// Blocks of a streaming launch: the resident ones of every SM, at most
+// max_blocks (rows of the partial-sum buffer) and one per 256 4-entry groups.
 template <typename K>
-int tiled_blocks(K kern, int n, int sm_count, int max_blocks, int& per_sm)
+int stream_blocks(K kern, int n, int sm_count, int max_blocks, int& per_sm)
 {
     if (per_sm == 0) {
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kGmBlock, 0) != cudaSuccess) per_sm = 1;
         if (per_sm < 1) per_sm = 1;
     }
-    long long tiles = ((long long)n + kGmTile - 1) / kGmTile;
-    long long b = (long long)per_sm * sm_count;
+    const long long groups = ((long long)n + 4 * kGmBlock - 1) / (4 * kGmBlock);
+    long long b = (long long)std::min(per_sm, kGmStreamBlocks) * sm_count;
     if (b > max_blocks) b = max_blocks;
-    if (b > tiles) b = tiles;
+    if (b > groups) b = groups;
     return b < 1 ? 1 : (int)b;
 }
 
@@ -486,21 +621,22 @@ cudaError_t launch_arnoldi(const GmArgs<G, VT>& a, int k)
     return cudaGetLastError();
 }
 
-template <typename VT, bool SUB, bool DOTS>
-cudaError_t launch_update(const GmArgs<float, VT>& a, int n, int k)
+template <bool SECOND, typename G, typename VT>
+cudaError_t launch_dots(const GmArgs<G, VT>& a, int n, int k)
 {
-    auto kern = gm_update_kernel<VT, SUB, DOTS>;
+    auto kern = gm_dots_kernel<VT, SECOND>;
     static int per_sm = 0;
-    const int b = tiled_blocks(kern, n, a.sm_count, a.max_blocks, per_sm);
-    kern<<<b, kGmBlock, 0, a.stream>>>(a.Q, a.ldq, n, k, a.m, a.rtol, a.partial, a.gctl);
+    const int b = stream_blocks(kern, n, a.sm_count, a.max_blocks, per_sm);
+    kern<<<b, kGmBlock, 0, a.stream>>>(a.Q, a.ldq, n, k, a.partial, a.gctl);
     return cudaGetLastError();
 }
-template <typename VT, bool SUB, bool DOTS>
-cudaError_t launch_update(const GmArgs<double, VT>& a, int n, int k)
+
+template <bool NORM, typename G, typename VT>
+cudaError_t launch_update(const GmArgs<G, VT>& a, int n, int k)
 {
-    auto kern = gm_update_kernel<VT, SUB, DOTS>;
+    auto kern = gm_update_kernel<VT, NORM>;
     static int per_sm = 0;
-    const int b = tiled_blocks(kern, n, a.sm_count, a.max_blocks, per_sm);
+    const int b = stream_blocks(kern, n, a.sm_count, a.max_blocks, per_sm);
     kern<<<b, kGmBlock, 0, a.stream>>>(a.Q, a.ldq, n, k, a.m, a.rtol, a.partial, a.gctl);
     return cudaGetLastError();
 }
@@ -536,19 +672,20 @@ cudaError_t cycle(const GmArgs<G, VT>& a, const VV* Vin, VV* Vnext)
     {
         auto kern = gm_start_kernel<VV, VT>;
         static int per_sm = 0;
-        const int b = tiled_blocks(kern, n, a.sm_count, a.max_blocks, per_sm);
+        const int b = stream_blocks(kern, n, a.sm_count, a.max_blocks, per_sm);
         kern<<<b, kGmBlock, 0, a.stream>>>(Vin, Vnext, a.Q, n, a.partial, a.gctl);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     for (int k = 0; k < a.m; ++k) {
         if ((e = dispatch_arnoldi(a, k)) != cudaSuccess) return e;
-        if ((e = launch_update<VT, false, true>(a, n, k)) != cudaSuccess) return e;      // projections
-        if (a.reorth && (e = launch_update<VT, true, true>(a, n, k)) != cudaSuccess) return e;
-        if ((e = launch_update<VT, true, false>(a, n, k)) != cudaSuccess) return e;      // update + norm
+        if ((e = launch_dots<false>(a, n, k)) != cudaSuccess) return e;
+        if (a.reorth && ((e = launch_update<false>(a, n, k)) != cudaSuccess || (e = launch_dots<true>(a, n, k)) != cudaSuccess))
+            return e;
+        if ((e = launch_update<true>(a, n, k)) != cudaSuccess) return e;
     }
     auto kern = gm_apply_kernel<VV, VT>;
     static int per_sm = 0;
-    const int b = tiled_blocks(kern, n, a.sm_count, a.max_blocks, per_sm);
+    const int b = stream_blocks(kern, n, a.sm_count, a.max_blocks, per_sm);
     kern<<<b, kGmBlock, 0, a.stream>>>(Vin, Vnext, a.Q, a.ldq, n, a.gctl, a.ctl);
     return cudaGetLastError();
 }
