@@ -168,6 +168,7 @@ __global__ void __launch_bounds__(kBlock, std::is_same<S, double>::value ? 2 : 3
                          : (MODE == kImproveFull ? kLImp32Full : kLImp32Walk);
     const int* pre = a.prefix + list * (a.count + 1);
     const int total = pre[a.count];
+    __shared__ float2 s_fine[512];
     int cur_t = -1;
     for (int it = blockIdx.x; it < total; it += gridDim.x) {
         const int t = item_transfer(pre, a.count, it);
@@ -176,6 +177,7 @@ __global__ void __launch_bounds__(kBlock, std::is_same<S, double>::value ? 2 : 3
             load_geo(s_g, &a.geo[t]);
             __syncthreads();
             build_table(s_g, s_code, s_sc);
+            if (cur_t < 0) build_fine(s_g, s_fine);   // one lattice for all transfers
             __syncthreads();
             cur_t = t;
         }
@@ -183,7 +185,8 @@ __global__ void __launch_bounds__(kBlock, std::is_same<S, double>::value ? 2 : 3
         const long long o = a.off[t];
         const int first = (it - pre[t]) * a.item_imp;
         const int end = min(first + a.item_imp, s_g.n_nodes);
-        const Table<float> T{s_code, s_sc, s_g.K};
+        Table<float> T{s_code, s_sc, s_g.K};
+        T.fine = s_fine;
         S resid = (S)0;
         bool bad = false;
         const S* Vin;

@@ -110,6 +110,10 @@ template <typename G> __device__ __forceinline__ G ginf();
 template <> __device__ __forceinline__ float ginf<float>() { return CUDART_INF_F; }
 template <> __device__ __forceinline__ double ginf<double>() { return CUDART_INF; }
 
+template <typename G> __device__ __forceinline__ G gnan();
+template <> __device__ __forceinline__ float gnan<float>() { return CUDART_NAN_F; }
+template <> __device__ __forceinline__ double gnan<double>() { return CUDART_NAN; }
+
 // Reciprocal for the geometry: FP32 uses the hardware approximation (about
 // 1 ulp); its error moves a foot by ~1e-9 cells, far below FP32 grid noise.
 __device__ __forceinline__ float grcp(float x) { return __fdividef(1.0f, x); }
@@ -146,13 +150,17 @@ __device__ __forceinline__ int wrap_code(int c) { return c & (kCodes - 1); }
 // (sin, cos) of a lattice code from two 256-entry tables:
 // alpha = a_hi + a_lo, sin = s_h c_l + c_h s_l, cos = c_h c_l - s_h s_l.
 template <typename G>
+__device__ __forceinline__ void angle_sum(const typename V2<G>::type& hi, const typename V2<G>::type& lo, G& s, G& c)
+{
+    s = hi.x * lo.y + hi.y * lo.x;
+    c = hi.y * lo.y - hi.x * lo.x;
+}
+
+template <typename G>
 __device__ __forceinline__ void code_sincos(const Geo<G>& g, int code, G& s, G& c)
 {
     code = wrap_code(code);
-    typename V2<G>::type hi = __ldg(&g.tab_hi[code >> 8]);
-    typename V2<G>::type lo = __ldg(&g.tab_lo[code & 255]);
-    s = hi.x * lo.y + hi.y * lo.x;
-    c = hi.y * lo.y - hi.x * lo.x;
+    angle_sum<G>(__ldg(&g.tab_hi[code >> 8]), __ldg(&g.tab_lo[code & 255]), s, c);
 }
 
 // Node decode: compact index -> (i_r, i_vr, i_vt, i_m).
@@ -460,17 +468,26 @@ template <> struct Corners<float> {
         unpack2(S, h0, h1);
         return h0 + t[0] * (h1 - h0);                                            // along r
     }
+    // qd[0] and qd[1] then hold the steps along v_t, which no angle changes
     __device__ __forceinline__ void fold_m(float t3)
     {
         const unsigned long long tt = pack2(t3, t3);
 #pragma unroll
         for (int x = 0; x < 4; ++x) q0[x] = fma2(qd[x], tt, q0[x]);
+        qd[0] = sub2(q0[1], q0[0]);
+        qd[1] = sub2(q0[3], q0[2]);
+    }
+    // every blend_m_folded() gives `v`
+    __device__ __forceinline__ void fold_constant(float v)
+    {
+        q0[0] = q0[2] = pack2(v, v);
+        qd[0] = qd[1] = 0;
     }
     __device__ __forceinline__ float blend_m_folded(const float t[4]) const
     {
         const unsigned long long t2 = pack2(t[2], t[2]), t1 = pack2(t[1], t[1]);
-        unsigned long long R0 = fma2(sub2(q0[1], q0[0]), t2, q0[0]);
-        unsigned long long R1 = fma2(sub2(q0[3], q0[2]), t2, q0[2]);
+        unsigned long long R0 = fma2(qd[0], t2, q0[0]);
+        unsigned long long R1 = fma2(qd[1], t2, q0[2]);
         unsigned long long S = fma2(sub2(R1, R0), t1, R0);
         float h0, h1;
         unpack2(S, h0, h1);
@@ -804,7 +821,7 @@ struct CachedEval {
     S vj;
     NodeDyn<G> nd;
     int cc[3];        // cached cell in (r, v_r, v_t); cc[0] = -1: none
-    G co[3];          // its offset from the node, cc - i
+    G co[3];          // its offset from the node, cc - i (none: NaN, which no foot lies in)
     bool cout;        // the cached cell has a corner outside the node set
     Corners<R> K;
     R pen;            // M - vj
@@ -815,6 +832,7 @@ struct CachedEval {
     __device__ __forceinline__ void reset()
     {
         cc[0] = -1;
+        co[0] = co[1] = co[2] = gnan<G>();
         pen = (R)((S)g->M64 - vj);
         if (DYN == kDynPolar) {
             outm = false;
@@ -833,8 +851,23 @@ struct CachedEval {
         }
     }
 
+    // the penalty of a cell with a corner outside sits in the corners, so that
+    // the angles need not ask for it
+    static constexpr bool kPenCorners = std::is_same<R, float>::value && DYN != kDynPolar && !DIAG;
+
+    // Fractions t of displacement u in the cached cell, true when it is there.
+    // FP32: one comparison of the largest fraction's bits.
+    __device__ __forceinline__ bool in_cached(const G u[4], G t[4]) const
+    {
+#pragma unroll
+        for (int d = 0; d < 3; ++d) t[d] = u[d] - co[d];
+        if constexpr (std::is_same<G, float>::value)
+            return max(max(__float_as_uint(t[0]), __float_as_uint(t[1])), __float_as_uint(t[2])) < 0x3f800000u;
+        else
+            return unit_fraction(t[0]) && unit_fraction(t[1]) && unit_fraction(t[2]);
+    }
+
     // 0 <= t < 1 (false for NaN and -0)
-    static __device__ __forceinline__ bool unit_fraction(float t) { return __float_as_uint(t) < 0x3f800000u; }
     static __device__ __forceinline__ bool unit_fraction(double t)
     {
         return (unsigned long long)__double_as_longlong(t) < 0x3ff0000000000000ull;
@@ -859,21 +892,13 @@ struct CachedEval {
         if constexpr (DYN != kDynPolar) {
             // the usual case: the foot lies in the cached cell, whose fractions
             // are u - (cell - node) in [0, 1), the same numbers foot_dim gives
-            if (cc[0] >= 0) {
-                bool in = true;
+            if (in_cached(u, t)) {
+                if (!kPenCorners && cout) return pen;
 #pragma unroll
-                for (int d = 0; d < 3; ++d) {
-                    t[d] = u[d] - co[d];
-                    in = in && unit_fraction(t[d]);
-                }
-                if (in) {
-                    if (cout) return pen;
-#pragma unroll
-                    for (int d = 0; d < 3; ++d) cl[d] = cc[d];
-                    cl[3] = cm;
-                    t[3] = tm;
-                    return blend_at(cl, t);
-                }
+                for (int d = 0; d < 3; ++d) cl[d] = cc[d];
+                cl[3] = cm;
+                t[3] = tm;
+                return blend_at(cl, t);
             }
         }
         bool out = outm;
@@ -897,6 +922,9 @@ struct CachedEval {
             }
             if (DYN == kDynPolar) cm = cl[3];
             else K.fold_m((R)tm);   // every foot of this state has the same mass fraction
+            if constexpr (kPenCorners) {
+                if (cout) K.fold_constant(pen);
+            }
         }
         if (cout) return pen;
         return blend_at(cl, t);
@@ -945,29 +973,35 @@ struct CachedEval {
         return w;
     }
 
-    // Cell cl and fractions t of this node's foot for a code (FP32 geometry
+    // Cell cl and fractions t of this node's foot for a control (FP32 geometry
     // only); false when the foot is outside the box or the node set.
-    __device__ __forceinline__ bool foot_at(int code, int cl[4], G t[4]) const
+    __device__ __forceinline__ bool foot_at(G s, G c, int cl[4], G t[4]) const
     {
-        G s, c, u[4];
+        G u[4];
         int base[4];
-        code_sincos(*g, code, s, c);
         heun_cells<G, DYN>(*g, sp, nd, s, c, u);
 #pragma unroll
         for (int d = 0; d < 4; ++d) u[d] += u0[d];
+        if (in_cached(u, t)) {   // where the search left off, nearly always
+#pragma unroll
+            for (int d = 0; d < 3; ++d) cl[d] = cc[d];
+            cl[3] = cm;
+            t[3] = tm;
+            return !cout;
+        }
         if (foot_cell(*g, i, u, cl, t)) return false;
         if (REDUCED && cell_rows<G, REDUCED>(*g, cl, base)) return false;
         return true;
     }
 
-    // Frozen-foot word pair of this node for a code (FP32 geometry only).
+    // Frozen-foot word pair of this node for a control (FP32 geometry only).
     // cell (nullable) receives the foot's cell when it has corners (kinds
     // inside and recompute).
-    __device__ __forceinline__ FootWord foot_of(int code, int* cell = nullptr) const
+    __device__ __forceinline__ FootWord foot_of(G s, G c, int* cell = nullptr) const
     {
         G t[4];
         int cl[4];
-        if (!foot_at(code, cl, t)) return foot_word_kind(kFootOut);
+        if (!foot_at(s, c, cl, t)) return foot_word_kind(kFootOut);
         if (cell) {
 #pragma unroll
             for (int d = 0; d < 4; ++d) cell[d] = cl[d];
@@ -976,11 +1010,11 @@ struct CachedEval {
     }
 
     // The same foot as one 8-byte word.
-    __device__ __forceinline__ unsigned long long foot8_of(int code, int* cell = nullptr) const
+    __device__ __forceinline__ unsigned long long foot8_of(G s, G c, int* cell = nullptr) const
     {
         G t[4];
         int cl[4];
-        if (!foot_at(code, cl, t)) return foot8_kind(kFootOut);
+        if (!foot_at(s, c, cl, t)) return foot8_kind(kFootOut);
         if (cell) {
 #pragma unroll
             for (int d = 0; d < 4; ++d) cell[d] = cl[d];
@@ -1000,7 +1034,28 @@ struct Table {
     int K;
     int off = 0;     // the lattice code kCodeOff stands for thrust off
     const float2* scf = nullptr;   // FP64 searches: sc rounded to FP32
+    const typename V2<G>::type* fine = nullptr;   // FP32 sweeps: the lattice tables tab_hi and tab_lo
+
+    // (sin, cos) of a lattice code that may lie a turn off
+    __device__ __forceinline__ void sincos(const Geo<G>& g, int c, G& s, G& cs) const
+    {
+        if constexpr (std::is_same<G, float>::value) {
+            if (fine) {
+                angle_sum<G>(fine[(c >> 8) & 255], fine[256 + (c & 255)], s, cs);
+                return;
+            }
+        }
+        code_sincos(g, c, s, cs);
+    }
 };
+
+// The lattice tables into shared memory (512 entries), for searches over
+// lattice codes: two shared loads an angle instead of two gathers with 64-bit
+// addresses.
+__device__ __forceinline__ void build_fine(const Geo<float>& g, float2* fine)
+{
+    for (int k = threadIdx.x; k < 512; k += blockDim.x) fine[k] = __ldg(k < 256 ? &g.tab_hi[k] : &g.tab_lo[k - 256]);
+}
 
 template <typename G>
 __device__ __forceinline__ void build_table(const Geo<G>& g, int* code, typename V2<G>::type* sc,
@@ -1081,45 +1136,46 @@ __device__ __forceinline__ int walk_table(E& ev, const Table<G>& T, int k0, type
 // to a Fibonacci length with +inf past the upper neighbour.  Returns the best
 // evaluated code (the tabulated minimiser included).  n0 is a lower bound of
 // the Fibonacci index of the bracket length.
+//
+// The bracket is [a, a + f] with f = F[n] and inner points a + F[n-2] and
+// a + F[n-1], whose values are f1 and f2: the state is a, the two values and
+// two Fibonacci numbers, stepped by subtraction (the search is bound by the
+// integer pipe, so the points themselves and table lookups would cost it).
 template <class E, typename G>
 __device__ __forceinline__ int fibonacci_refine(E& ev, const Table<G>& T, int n0, int fib_stop, int k,
                                                 typename E::R Dk, typename E::R& Dbest)
 {
     typedef typename E::R R;
-    const int ck = T.code[k];
     const int cl = (k == 0) ? T.code[T.K - 1] - kCodes : T.code[k - 1];
-    const int cr = T.code[k + 1];
-    const int lo_off = cl - ck, hi_off = cr - ck, L = hi_off - lo_off;
+    const int end = T.code[k + 1];
+    auto value = [&](int x) {
+        G s, c;
+        T.sincos(*ev.g, x, s, c);
+        const R f = ev.at_sc(s, c);
+        return (x >= end || (E::kMayOff && T.off && wrap_code(x) == kCodeOff)) ? ginf<R>() : f;
+    };
     int n = n0;
-    while (kFib[n] < L) ++n;
-    int best = ck;
+    while (kFib[n] < end - cl) ++n;
+    int best = T.code[k];
     R qb = Dk;
-    int a = lo_off;
-    int x1 = a + kFib[n - 2], x2 = a + kFib[n - 1];
-    R f1 = (x1 >= hi_off || (E::kMayOff && T.off && wrap_code(ck + x1) == kCodeOff)) ? ginf<R>() : ev.at_code(ck + x1);
-    R f2 = (x2 >= hi_off || (E::kMayOff && T.off && wrap_code(ck + x2) == kCodeOff)) ? ginf<R>() : ev.at_code(ck + x2);
-    if (f1 < qb) { qb = f1; best = ck + x1; }
-    if (f2 < qb) { qb = f2; best = ck + x2; }
-    for (int kk = n; kk > 4 && kFib[kk] > fib_stop; --kk) {
-        // keep [a, x2] (new point a + F[kk-3]) or [x1, a + F[kk]] (new point
-        // x1 + F[kk-2]); one evaluation per step, outside the branch
+    int a = cl, p = kFib[n - 2], r = kFib[n - 3];
+    R f1 = value(a + p), f2 = value(a + p + r);
+    if (f1 < qb) { qb = f1; best = a + p; }
+    if (f2 < qb) { qb = f2; best = a + p + r; }
+    const int stop = max(fib_stop, 3);
+    // a bracket of F[kk] = 2 p + r goes on while it is longer than the stop
+    while (2 * p + r > stop) {
         const bool left = f1 <= f2;
-        int xn;
-        if (left) {
-            x2 = x1; f2 = f1;
-            x1 = a + kFib[kk - 3];
-            xn = x1;
-        } else {
-            a = x1;
-            x1 = x2; f1 = f2;
-            x2 = a + kFib[kk - 2];
-            xn = x2;
-        }
-        const bool skip = xn >= hi_off || (E::kMayOff && T.off && wrap_code(ck + xn) == kCodeOff);
-        const R fn = skip ? ginf<R>() : ev.at_code(ck + xn);
-        if (left) f1 = fn;
-        else f2 = fn;
-        if (fn < qb) { qb = fn; best = ck + xn; }
+        if (!left) a += p;
+        const int x = a + (left ? r : p);
+        const R keep = left ? f1 : f2;
+        const R f = value(x);
+        f1 = left ? f : keep;
+        f2 = left ? keep : f;
+        if (f < qb) { qb = f; best = x; }
+        const int q = p - r;
+        p = r;
+        r = q;
     }
     Dbest = qb;
     return wrap_code(best);

@@ -578,13 +578,18 @@ feet_kernel(const __grid_constant__ Geo<float> g, const uint16_t* __restrict__ c
         CachedEval<float, float, REDUCED, DYN, float, false> ev;
         decode_node(g, j, ev.i);
         const bool target = in_target(g, ev.i);
-        if (!target) setup_node<float, float, DYN>(ev, g, (const float*)nullptr, 0.0f);
+        float sn = 0.0f, cs = 0.0f;
+        if (!target) {
+            setup_node<float, float, DYN>(ev, g, (const float*)nullptr, 0.0f);
+            ev.reset();
+            code_sincos(g, code[j], sn, cs);
+        }
         if (feet_hi) {
-            const FootWord w = target ? foot_word_kind(kFootTarget) : ev.foot_of(code[j]);
+            const FootWord w = target ? foot_word_kind(kFootTarget) : ev.foot_of(sn, cs);
             feet_lo[j] = w.lo;
             feet_hi[j] = w.hi;
         } else {
-            feet_lo[j] = target ? foot8_kind(kFootTarget) : ev.foot8_of(code[j]);
+            feet_lo[j] = target ? foot8_kind(kFootTarget) : ev.foot8_of(sn, cs);
         }
     }
 }

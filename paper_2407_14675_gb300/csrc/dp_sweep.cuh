@@ -581,12 +581,14 @@ __device__ __forceinline__ void sweep_nodes(const Geo<G>& g, const Table<G>& T, 
                             // values (feet8), else the 24-bit word pair
                             int cl[4];
                             int kind;
+                            G sn, cs;
+                            T.sincos(g, c, sn, cs);
                             if (!kPolish && feet8) {
-                                const unsigned long long w = ev.foot8_of(c, cl);
+                                const unsigned long long w = ev.foot8_of(sn, cs, cl);
                                 feet_lo[j] = w;
                                 kind = foot_kind(w);
                             } else {
-                                const FootWord w = ev.foot_of(c, cl);
+                                const FootWord w = ev.foot_of(sn, cs, cl);
                                 feet_lo[j] = w.lo;
                                 feet_hi[j] = w.hi;
                                 kind = foot_kind(w);
@@ -760,11 +762,15 @@ sweep_kernel(const __grid_constant__ Geo<G> g, const S* __restrict__ Vin, S* __r
     constexpr bool kTab32 = search64_blocks<G, S, MODE>();
     float2* s_scf = kTab32 ? reinterpret_cast<float2*>(s_sc + g.K) : nullptr;
     int* s_code = kTab32 ? reinterpret_cast<int*>(s_scf + g.K) : reinterpret_cast<int*>(s_sc + (kSearch ? g.K : 0));
+    constexpr bool kFine = std::is_same<G, float>::value && (MODE == kImproveFull || MODE == kImproveWalk);
+    __shared__ float2 s_fine[kFine ? 512 : 1];
     if constexpr (kSearch) {
         build_table(g, s_code, s_sc, s_scf);
+        if constexpr (kFine) build_fine(g, s_fine);
         __syncthreads();
     }
-    const Table<G> T{s_code, s_sc, g.K, g.off, s_scf};
+    Table<G> T{s_code, s_sc, g.K, g.off, s_scf};
+    if constexpr (kFine) T.fine = s_fine;
 
     S resid = (S)0;
     bool bad = false;
