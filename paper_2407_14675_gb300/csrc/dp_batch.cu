@@ -7,8 +7,9 @@
 // persistent launch over all transfers: a block walks a list of work items
 // (a transfer and a run of `item` consecutive nodes), loads that transfer's
 // geometry and angle table into shared memory when the transfer changes, and
-// runs the same per-node code as a single grid's sweep.  Item sizes are
-// picked by timing the candidates on the batch itself (dp_batch_autotune).
+// runs the same per-node code as a single grid's sweep.  Item sizes follow a
+// rule or are picked by timing the candidates on the batch itself
+// (dp_batch_autotune).
 //
 // Modified policy iteration (§3, Eq. (13)/(14), 1 improvement + n_eval
 // evaluation sweeps per outer step) runs per transfer as a small state
@@ -123,6 +124,26 @@ __device__ __forceinline__ void load_geo(Geo<float>& dst, const Geo<float>* src)
     for (int k = threadIdx.x; k < (int)(sizeof(Geo<float>) / 4); k += blockDim.x) d[k] = s[k];
 }
 
+// A block's share of a list's items, for the launches whose nodes cost the
+// same: equal runs of consecutive items, [lo, hi) of `total`.  run_of() takes
+// the part of it in one transfer, a run of consecutive nodes, off its front.
+// Handed out one by one, items of 8192 nodes left the last round of blocks
+// half empty, and smaller ones paid for each item's start and residual.
+// Evaluation sweeps one by one and by shares: 16 transfers (8.5M nodes) 62.9
+// and 50.7 us, 3 (476,187 nodes) 13.8 and 9.8, 200 (63M) 395 and 333.
+struct Share {
+    int lo, hi;
+    __device__ Share(int total)
+    {
+        lo = (int)((long long)total * blockIdx.x / gridDim.x);
+        hi = (int)((long long)total * (blockIdx.x + 1) / gridDim.x);
+    }
+};
+
+struct Run {
+    int t, first, end;   // transfer, nodes
+};
+
 // The transfer of work item `it` in list `pre`: pre[t] <= it < pre[t + 1].
 __device__ __forceinline__ int item_transfer(const int* pre, int count, int it)
 {
@@ -135,19 +156,30 @@ __device__ __forceinline__ int item_transfer(const int* pre, int count, int it)
     return lo;
 }
 
+// t: the transfer of the run before (-1: none yet).
+__device__ __forceinline__ Run run_of(Share& s, const int* pre, int count, int t, int item, const Geo<float>* geo)
+{
+    if (t < 0) t = item_transfer(pre, count, s.lo);
+    else while (__ldg(&pre[t + 1]) <= s.lo) ++t;
+    const int p0 = __ldg(&pre[t]), stop = min(s.hi, __ldg(&pre[t + 1]));
+    const long long end = (long long)(stop - p0) * item;
+    const Run r{t, (s.lo - p0) * item, (int)min(end, (long long)__ldg(&geo[t].n_nodes))};
+    s.lo = stop;
+    return r;
+}
+
 // FP32 values -> FP64 values at the switch.
 __global__ void __launch_bounds__(kBlock) batch_widen_kernel(const BArgs a)
 {
     const int* pre = a.prefix + kLWiden * (a.count + 1);
-    const int total = pre[a.count];
-    for (int it = blockIdx.x; it < total; it += gridDim.x) {
-        const int t = item_transfer(pre, a.count, it);
-        const int first = (it - pre[t]) * a.item_eval;
-        const int end = min(first + a.item_eval, a.geo[t].n_nodes);
+    Share share(pre[a.count]);
+    for (int t = -1; share.lo < share.hi;) {
+        const Run r = run_of(share, pre, a.count, t, a.item_eval, a.geo);
+        t = r.t;
         const BState& S = a.st[t];
         const float* src = pick(a.V32, S.cur) + a.off[t];
         double* dst = pick(a.V64, S.cur64) + a.off[t];
-        for (int j = first + threadIdx.x; j < end; j += kBlock) dst[j] = (double)src[j];
+        for (int j = r.first + threadIdx.x; j < r.end; j += kBlock) dst[j] = (double)src[j];
     }
 }
 
@@ -221,21 +253,17 @@ __global__ void __launch_bounds__(kBatchEvalBlock, 2) batch_eval_kernel(const BA
 {
     __shared__ Geo<float> s_g;
     const int* pre = a.prefix + kLEval * (a.count + 1);
-    const int total = pre[a.count];
+    Share share(pre[a.count]);
     const Table<float> T{nullptr, nullptr, 0};
-    int cur_t = -1;
-    for (int it = blockIdx.x; it < total; it += gridDim.x) {
-        const int t = item_transfer(pre, a.count, it);
+    for (int cur_t = -1; share.lo < share.hi;) {
+        const Run r = run_of(share, pre, a.count, cur_t, a.item_eval, a.geo);
+        const int t = r.t, first = r.first, end = r.end;
+        __syncthreads();   // the previous run is done with the geometry
+        load_geo(s_g, &a.geo[t]);
         __syncthreads();
-        if (t != cur_t) {
-            load_geo(s_g, &a.geo[t]);
-            __syncthreads();
-            cur_t = t;
-        }
+        cur_t = t;
         BState& st = a.st[t];
         const long long o = a.off[t];
-        const int first = (it - pre[t]) * a.item_eval;
-        const int end = min(first + a.item_eval, s_g.n_nodes);
         float resid = 0.0f;
         bool bad = false;
         if (st.phase == kPh32 || !FEET) {
@@ -522,7 +550,7 @@ struct dp_batch {
     int* d_bad = nullptr;
     BState* h_st = nullptr;        // pinned mirror of d_st
     BParams* h_par = nullptr;      // pinned
-    int item_eval = 8192, item_imp = 8192;
+    int item_eval = kBlock, item_imp = 8192;
     int blocks_widen = 0, blocks_imp32f = 0, blocks_imp32w = 0, blocks_imp64f = 0, blocks_imp64w = 0;
     int blocks_eval = 0, blocks_eval_nf = 0;
     cudaGraphExec_t exec = nullptr;
@@ -916,6 +944,16 @@ int dp_batch_create(const dp_grid_desc* descs, int32_t count, void* stream, dp_b
               occupancy_blocks(batch_eval_kernel<kDynUnitSpeed, false, false>, b->sm_count, &b->blocks_eval_nf, kBatchEvalBlock);
     }
     bad = bad || occupancy_blocks(batch_widen_kernel, b->sm_count, &b->blocks_widen);
+    // Improvement items: about eight per resident block.  Angle searches differ
+    // in how many angles they take, so items go round robin; fewer leave the
+    // last round half empty, more pay for their starts.  Walk sweeps with 8192
+    // nodes an item and by this rule: 16 transfers (8.5M nodes) 821 and 786 us,
+    // 24 (4.9M) 540 and 464, 3 (476,187) 182 and 57; 200 (63M) 5.89 ms at 4096
+    // and at 8192.
+    {
+        const long long per = b->total / (8LL * std::max(1, b->blocks_imp32w));
+        b->item_imp = (int)std::min(4096LL, std::max(512LL, (per + kBlock - 1) / kBlock * kBlock));
+    }
     if (bad) return bail(bfail(DP_ECUDA, "occupancy query failed"));
     *out = b;
     return DP_OK;

@@ -168,3 +168,20 @@ def test_batch_standalone_evaluation_after_a_solve(dp, solver, polish):
             v_o = o.sweep(V, mode=oracle.EVAL, codes=codes)[0]
             _check_values(b.get_value(i), v_o, TOL32, "transfer %d" % i, o=o, nodes=np.arange(p.nodes),
                           codes=codes)
+
+
+@pytest.mark.parametrize("sizes,count", [((2, 3, 4), 700), ((2, 9, 17), 40), ((17,), 1)])
+def test_equal_shares_of_uneven_transfers(dp, sizes, count):
+    # evaluation launches hand every block an equal run of items that may cross
+    # transfers: more transfers than blocks, runs that start inside a transfer,
+    # a single one.  The single grid's sweeps are the reference, bit for bit.
+    probs = W.batch_transfers(count=count, seed=3, sizes=sizes)
+    opts = dict(tol=0.0, max_sweeps=3, n_eval=4, polish=0)
+    with dp.Batch(probs) as b:
+        b.policy_iterate(**opts)
+        got = [(b.get_value(i), b.get_policy(i)) for i in range(count)]
+    for i in range(0, count, max(1, count // 12)):
+        with dp.Grid(probs[i]) as g:
+            g.policy_iterate(**opts)
+            np.testing.assert_array_equal(got[i][0], g.get_value())
+            np.testing.assert_array_equal(got[i][1], g.get_policy())
