@@ -56,17 +56,7 @@ constexpr int kOffW1 = 0, kOffB1 = kOffW1 + kH * 4, kOffW2 = kOffB1 + kH, kOffB2
 constexpr int kOffW3 = kOffB2 + kH, kOffB3 = kOffW3 + kH * kH, kOffW4 = kOffB3 + kH, kOffB4 = kOffW4 + 3 * kH;
 constexpr int kParams = kOffB4 + 3;           // 133,635
 constexpr int kTileM = 128, kTileN = 128, kKC = 256;
-// Shared memory of a K slice of A and B: 128 KB for a whole 256-wide slice
-// (one CTA per SM; small batches: every slice at once), 64 KB for 128-wide
-// slices (three CTAs per SM overlap one another's loads and epilogues).
-constexpr int gemm_smem(int kc) { return (kTileM + kTileN) * kc * 2; }
-// MN-major operands (kEpiSplitMN) get 32 KB more: the MMAs of a 256-wide
-// slice then read inside the allocation for either assignment of its
-// descriptors' two byte offsets (2048 along K, 128 along MN), at most
-// 92,416 bytes past an operand's start.
-constexpr int kMNPad = 32768;
-template <int EPI, int KC>
-constexpr int gemm_smem_of() { return gemm_smem(KC) + (EPI == 3 /* kEpiSplitMN */ ? kMNPad : 0); }
+constexpr int kGemmSmem = (kTileM + kTileN) * kKC * 2;   // A and B of a tile, 128 KB
 constexpr int kWaitPolls = 1 << 22;
 constexpr float kInvSqrt2 = 0.70710678118654752f, kInvSqrt2Pi = 0.39894228040143268f;
 
@@ -77,9 +67,8 @@ __device__ __forceinline__ float gelu_grad(float z)
 }
 
 // 8 consecutive BF16 values (one 16-byte load) as floats.
-__device__ __forceinline__ void load_row8(const bf16* p, float a[8])
+__device__ __forceinline__ void row8(const uint4& v, float a[8])
 {
-    const uint4 v = *reinterpret_cast<const uint4*>(p);
     const unsigned u[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
@@ -89,7 +78,7 @@ __device__ __forceinline__ void load_row8(const bf16* p, float a[8])
     }
 }
 
-enum { kEpiFwd = 0, kEpiBwd = 1, kEpiAtomic = 2, kEpiSplitMN = 3 };
+enum { kEpiFwd = 0, kEpiBwd = 1 };
 
 // Four doubles by value (the network's input box corners).
 struct Box4 {
@@ -102,39 +91,35 @@ __device__ __forceinline__ void cp_async16(void* dst, const void* src)
 {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(smem_u32(dst)), "l"(src) : "memory");
 }
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+// all but the N groups committed last
+template <int N>
+__device__ __forceinline__ void cp_async_wait_pending()
+{
+    asm volatile("cp.async.wait_group %0;" :: "n"(N) : "memory");
+}
 __device__ __forceinline__ void cp_async_wait_all()
 {
     asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;" ::: "memory");
 }
 
-// C[128 x 128 tile] = A[rows, K range] * B[256, K range]^T on tcgen05.
+// C[128 x 128 tile] = A[rows, 256] * B[256, 256]^T on tcgen05, for batches
+// below kManyRows rows.
 //   A: bf16 [*, lda] row-major (K contiguous); B: bf16 [256, ldb] row-major.
-//   Tile rows start at 128 blockIdx.x, columns at 128 blockIdx.y; K range
-//   [k_per_cta blockIdx.z, +k_per_cta), staged 256 at a time: every thread
-//   issues its 16-byte asynchronous copies of the whole slice at once, then
-//   one thread issues the 16 MMAs (K = 16 each) and commits them to an
-//   mbarrier.
+//   Tile rows start at 128 blockIdx.x, columns at 128 blockIdx.y: every thread
+//   issues its 16-byte asynchronous copies of both operands at once, then one
+//   thread issues the 16 MMAs (K = 16 each) and commits them to an mbarrier.
 //   kEpiFwd:    z = acc + bias -> zout (optional, FP32), h = GELU(z) -> hout (bf16)
 //   kEpiBwd:    dz = acc * GELU'(zin) -> hout (bf16)
-//   kEpiAtomic: cacc += acc (FP32, split-K weight gradients)
-//   kEpiSplitMN: both operands MN-major, A[K range, 128 blockIdx.x + i] and
-//     B[K range, 128 blockIdx.y + j] row-major with the tile's rows / columns
-//     contiguous (a weight gradient dz^T h straight from the activations, no
-//     transposed copies); the tile is stored, not added, at split blockIdx.z
-//     of cacc (256 x 256 floats per split), for a reduction in a fixed
-//     order.  Core matrix (K block kb,
-//     MN block mb) holds 8 K-rows of 8 contiguous MN elements at byte
-//     (kb * 16 + mb) * 128: 128 bytes to the next MN block, 2048 to the next
-//     K block.
-template <int EPI, int KC>
+template <int EPI>
 __global__ void __launch_bounds__(128)
-mlp_gemm_kernel(const bf16* __restrict__ A, int lda, const bf16* __restrict__ B, int ldb, int k_per_cta,
-                const float* __restrict__ bias, float* __restrict__ zout, const float* __restrict__ zin,
-                bf16* __restrict__ hout, float* __restrict__ cacc, int* __restrict__ err, int polls)
+mlp_gemm_kernel(const bf16* __restrict__ A, int lda, const bf16* __restrict__ B, int ldb, const float* __restrict__ bias,
+                float* __restrict__ zout, const float* __restrict__ zin, bf16* __restrict__ hout, int* __restrict__ err,
+                int polls)
 {
     extern __shared__ __align__(1024) unsigned char smem[];
-    unsigned char* sA = smem;                        // 128 x KC bf16
-    unsigned char* sB = smem + kTileM * KC * 2;      // 128 x KC bf16
+    unsigned char* sA = smem;                        // 128 x 256 bf16
+    unsigned char* sB = smem + kTileM * kKC * 2;     // 128 x 256 bf16
     __shared__ unsigned tmem_slot;
     __shared__ __align__(8) unsigned long long mbar;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -146,76 +131,49 @@ mlp_gemm_kernel(const bf16* __restrict__ A, int lda, const bf16* __restrict__ B,
     const unsigned tmem = tmem_slot;
     const size_t row0 = (size_t)blockIdx.x * kTileM;
     const int n0 = blockIdx.y * kTileN;
-    const int kbeg = blockIdx.z * k_per_cta;
-    constexpr bool kMN = EPI == kEpiSplitMN;
-    constexpr unsigned idesc = umma_idesc_bf16(kTileM, kTileN) | (kMN ? (1u << 15) | (1u << 16) : 0u);
-    constexpr int kGroups = KC / 8;                  // 16-byte groups per row of a slice
+    constexpr unsigned idesc = umma_idesc_bf16(kTileM, kTileN);
+    constexpr int kGroups = kKC / 8;                 // 16-byte groups per row
 
-    int phase = 0;
-    bool ok = true;
-    for (int k0 = kbeg; k0 < kbeg + k_per_cta; k0 += KC) {
-        // core-matrix staging: (row, kb) -> ((row / 8) * kGroups + kb) * 128 + (row % 8) * 16.
-        // A warp takes 8 rows x 4 consecutive 16-byte groups: 64 contiguous bytes
-        // of each row in global memory, 512 contiguous bytes (no bank conflict)
-        // in shared memory.
-        // the 16-byte groups go straight to shared memory (cp.async): every
-        // group of the slice is in flight at once, none through registers
-        if constexpr (kMN) {
-            // a warp takes 8 K-rows x 4 consecutive MN blocks: 64 contiguous
-            // bytes of each row in global memory, 512 in shared memory
+    // core-matrix staging: (row, kb) -> ((row / 8) * kGroups + kb) * 128 + (row % 8) * 16.
+    // A warp takes 8 rows x 4 consecutive 16-byte groups: 64 contiguous bytes
+    // of each row in global memory, 512 contiguous bytes (no bank conflict)
+    // in shared memory.  The groups go straight to shared memory (cp.async):
+    // every one is in flight at once, none through registers.
 #pragma unroll
-            for (int q = 0; q < kTileM * kGroups / 128; ++q) {
-                const int v = tid + 128 * q, grp = v >> 5, ln = v & 31;
-                const int kr = (grp >> 2) * 8 + (ln & 7), mb = (grp & 3) * 4 + (ln >> 3);
-                cp_async16(sA + (size_t)v * 16, A + (size_t)(k0 + kr) * lda + row0 + mb * 8);
-            }
-#pragma unroll
-            for (int q = 0; q < kTileN * kGroups / 128; ++q) {
-                const int v = tid + 128 * q, grp = v >> 5, ln = v & 31;
-                const int kr = (grp >> 2) * 8 + (ln & 7), mb = (grp & 3) * 4 + (ln >> 3);
-                cp_async16(sB + (size_t)v * 16, B + (size_t)(k0 + kr) * ldb + n0 + mb * 8);
-            }
-        } else {
-#pragma unroll
-            for (int q = 0; q < kTileM * kGroups / 128; ++q) {
-                const int v = tid + 128 * q, grp = v >> 5, ln = v & 31;
-                const int row = (grp / (kGroups / 4)) * 8 + (ln & 7), kb = (grp % (kGroups / 4)) * 4 + (ln >> 3);
-                cp_async16(sA + (size_t)v * 16, A + (row0 + row) * (size_t)lda + k0 + kb * 8);
-            }
-#pragma unroll
-            for (int q = 0; q < kTileN * kGroups / 128; ++q) {
-                const int v = tid + 128 * q, grp = v >> 5, ln = v & 31;
-                const int row = (grp / (kGroups / 4)) * 8 + (ln & 7), kb = (grp % (kGroups / 4)) * 4 + (ln >> 3);
-                cp_async16(sB + (size_t)v * 16, B + (size_t)(n0 + row) * ldb + k0 + kb * 8);
-            }
-        }
-        cp_async_wait_all();
-        fence_async_smem();
-        __syncthreads();
-        if (tid == 0) {
-            fence_after_sync();
-#pragma unroll
-            for (int s = 0; s < KC / 16; ++s) {
-                // K step s: two K blocks (K-major: 256 bytes on; MN-major: 4096)
-                const unsigned long long ad =
-                    kMN ? umma_desc(smem_u32(sA) + s * 4096, 2048, 128) : umma_desc(smem_u32(sA) + s * 256, 128, kGroups * 128);
-                const unsigned long long bd =
-                    kMN ? umma_desc(smem_u32(sB) + s * 4096, 2048, 128) : umma_desc(smem_u32(sB) + s * 256, 128, kGroups * 128);
-                umma_bf16(tmem, ad, bd, idesc, (k0 > kbeg || s > 0) ? 1u : 0u);
-            }
-            umma_commit(&mbar);
-        }
-        if (!mbar_wait(&mbar, phase, polls)) {
-            // give up (error flag), but let the committed MMAs finish before
-            // the accumulator is freed and the staging buffers are released
-            ok = false;
-            if (lane == 0) atomicOr(err, 1);
-            mbar_wait(&mbar, phase, kWaitPolls);
-        }
-        phase ^= 1;
-        __syncthreads();
-        if (!__syncthreads_and(ok)) break;
+    for (int q = 0; q < kTileM * kGroups / 128; ++q) {
+        const int v = tid + 128 * q, grp = v >> 5, ln = v & 31;
+        const int row = (grp / (kGroups / 4)) * 8 + (ln & 7), kb = (grp % (kGroups / 4)) * 4 + (ln >> 3);
+        cp_async16(sA + (size_t)v * 16, A + (row0 + row) * (size_t)lda + kb * 8);
     }
+#pragma unroll
+    for (int q = 0; q < kTileN * kGroups / 128; ++q) {
+        const int v = tid + 128 * q, grp = v >> 5, ln = v & 31;
+        const int row = (grp / (kGroups / 4)) * 8 + (ln & 7), kb = (grp % (kGroups / 4)) * 4 + (ln >> 3);
+        cp_async16(sB + (size_t)v * 16, B + (size_t)(n0 + row) * ldb + kb * 8);
+    }
+    cp_async_wait_all();
+    fence_async_smem();
+    __syncthreads();
+    if (tid == 0) {
+        fence_after_sync();
+#pragma unroll
+        for (int s = 0; s < kKC / 16; ++s) {
+            // K step s: two K blocks, 256 bytes on
+            const unsigned long long ad = umma_desc(smem_u32(sA) + s * 256, 128, kGroups * 128);
+            const unsigned long long bd = umma_desc(smem_u32(sB) + s * 256, 128, kGroups * 128);
+            umma_bf16(tmem, ad, bd, idesc, s > 0 ? 1u : 0u);
+        }
+        umma_commit(&mbar);
+    }
+    bool ok = true;
+    if (!mbar_wait(&mbar, 0, polls)) {
+        // give up (error flag), but let the committed MMAs finish before
+        // the accumulator is freed and the staging buffers are released
+        ok = false;
+        if (lane == 0) atomicOr(err, 1);
+        mbar_wait(&mbar, 0, kWaitPolls);
+    }
+    ok = __syncthreads_and(ok);
     fence_after_sync();
     if (ok) {
         const size_t r = row0 + warp * 32 + lane;   // TMEM lane = tile row
@@ -223,20 +181,6 @@ mlp_gemm_kernel(const bf16* __restrict__ A, int lda, const bf16* __restrict__ B,
             float v[16];
             tmem_ld16(tmem + ((unsigned)(warp * 32) << 16) + c0, v);
             const size_t off = r * kH + n0 + c0;     // 16 consecutive columns, 64-byte aligned
-            if (EPI == kEpiAtomic) {
-                // four 16-byte reductions (the row's 16 columns are 64-byte aligned)
-#pragma unroll
-                for (int q = 0; q < 16; q += 4)
-                    atomicAdd(reinterpret_cast<float4*>(cacc + off + q), make_float4(v[q], v[q + 1], v[q + 2], v[q + 3]));
-                continue;
-            }
-            if (EPI == kEpiSplitMN) {
-                float* dst = cacc + (size_t)blockIdx.z * kH * kH + off;
-#pragma unroll
-                for (int q = 0; q < 16; q += 4)
-                    *reinterpret_cast<float4*>(dst + q) = make_float4(v[q], v[q + 1], v[q + 2], v[q + 3]);
-                continue;
-            }
             float z[16];
             if (EPI == kEpiFwd) {
 #pragma unroll
@@ -263,6 +207,109 @@ mlp_gemm_kernel(const bf16* __restrict__ A, int lda, const bf16* __restrict__ B,
             }
             *(uint4*)(hout + off) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
             *(uint4*)(hout + off + 8) = make_uint4(pk[4], pk[5], pk[6], pk[7]);
+        }
+    }
+    fence_before_sync();
+    __syncthreads();
+    if (warp == 0) tmem_dealloc(tmem, kTileN);
+}
+
+// Weight gradient dz^T h of a hidden layer, split along the batch: the tile
+// C[128 blockIdx.x.., 128 blockIdx.y..] over the k_per_cta rows (a multiple of
+// kWgRows) from k_per_cta blockIdx.z of A = dz and B = h, both rows x 256, read
+// as they are (both operands MN-major, no transposed copies).  The tile is
+// stored at split blockIdx.z of out (256 x 256 floats per split), for a
+// reduction in a fixed order.  Core matrix (K block kb, MN block mb) holds 8
+// rows of 8 contiguous columns at byte (kb * 16 + mb) * 128: 128 bytes to the
+// next MN block, 2048 to the next K block.
+//
+// What bounds it: 256 KB of operands per CTA from L2 (two row slabs of 512 at a
+// batch of 16,384, 128 CTAs, about 2.1 us at 64 bytes a clock), and the latency
+// of the first and of the epilogue.  Rows pass through a ring of six 32 KB
+// chunks of 64 rows, five ahead of the MMAs; staged 256 rows at a time with
+// nothing in flight during their MMAs it took 15.3 us, now 14.0.
+constexpr int kWgRows = 64, kWgSlots = 6, kWgThreads = 256;
+constexpr int kWgChunk = kWgRows * kTileM * 2;                     // bytes of one operand's chunk
+constexpr int kWgSmem = kWgSlots * 2 * kWgChunk;                   // 192 KB
+
+__global__ void __launch_bounds__(kWgThreads)
+mlp_wgrad_kernel(const bf16* __restrict__ A, const bf16* __restrict__ B, int k_per_cta, float* __restrict__ out,
+                 int* __restrict__ err, int polls)
+{
+    extern __shared__ __align__(1024) unsigned char smem[];
+    __shared__ unsigned tmem_slot;
+    __shared__ __align__(8) unsigned long long done[kWgSlots];     // the slot's MMAs have completed
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int m0 = blockIdx.x * kTileM, n0 = blockIdx.y * kTileN, kbeg = blockIdx.z * k_per_cta;
+    const int chunks = k_per_cta / kWgRows;
+    // a warp takes 8 rows x 4 consecutive MN blocks: 64 contiguous bytes of
+    // each row in global memory, 512 in shared memory
+    auto stage = [&](int c) {
+        unsigned char* dst = smem + (c % kWgSlots) * 2 * kWgChunk;
+        const size_t k0 = (size_t)kbeg + (size_t)c * kWgRows;
+#pragma unroll
+        for (int q = 0; q < 2 * kWgChunk / 16 / kWgThreads; ++q) {
+            const int v = tid + kWgThreads * (q % (kWgChunk / 16 / kWgThreads)), grp = v >> 5;
+            const int kr = (grp >> 2) * 8 + (lane & 7), mb = (grp & 3) * 4 + (lane >> 3);
+            if (q < kWgChunk / 16 / kWgThreads) cp_async16(dst + (size_t)v * 16, A + (k0 + kr) * kH + m0 + mb * 8);
+            else cp_async16(dst + kWgChunk + (size_t)v * 16, B + (k0 + kr) * kH + n0 + mb * 8);
+        }
+    };
+    // one group of copies per chunk and turn, empty ones included, so that the
+    // groups left pending count the chunks
+#pragma unroll
+    for (int c = 0; c < kWgSlots - 1; ++c) {
+        if (c < chunks) stage(c);
+        cp_async_commit();
+    }
+    if (warp == 0) tmem_alloc(&tmem_slot, kTileN);
+    if (tid == 0) {
+        for (int b = 0; b < kWgSlots; ++b) mbar_init(&done[b]);
+    }
+    fence_before_sync();
+    __syncthreads();
+    fence_after_sync();
+    const unsigned tmem = tmem_slot;
+    constexpr unsigned idesc = umma_idesc_bf16(kTileM, kTileN) | (1u << 15) | (1u << 16);   // both MN-major
+    bool ok = true;
+    for (int c = 0; c < chunks; ++c) {
+        cp_async_wait_pending<kWgSlots - 2>();
+        fence_async_smem();
+        __syncthreads();
+        if (tid == 0) {
+            fence_after_sync();
+            const unsigned sa = smem_u32(smem + (c % kWgSlots) * 2 * kWgChunk);
+#pragma unroll
+            for (int s = 0; s < kWgRows / 16; ++s)   // K step s: two K blocks
+                umma_bf16(tmem, umma_desc(sa + s * 4096, 2048, 128), umma_desc(sa + kWgChunk + s * 4096, 2048, 128), idesc,
+                          c > 0 || s > 0 ? 1u : 0u);
+            umma_commit(&done[c % kWgSlots]);
+        }
+        // the slot of the chunk before takes the chunk five on once its MMAs are done
+        const int next = c + kWgSlots - 1;
+        if (next < chunks) {
+            if (c > 0 && !mbar_wait(&done[(c - 1) % kWgSlots], ((c - 1) / kWgSlots) & 1, kWaitPolls)) ok = false;
+            if (ok) stage(next);
+        }
+        cp_async_commit();
+    }
+    cp_async_wait_pending<0>();   // none is left after a full run; after a wait that gave up, no copy may outlive the CTA
+    if (!mbar_wait(&done[(chunks - 1) % kWgSlots], ((chunks - 1) / kWgSlots) & 1, polls)) {
+        ok = false;
+        mbar_wait(&done[(chunks - 1) % kWgSlots], ((chunks - 1) / kWgSlots) & 1, kWaitPolls);   // the committed MMAs finish first
+    }
+    if (!ok && lane == 0) atomicOr(err, 1);
+    ok = __syncthreads_and(ok);
+    fence_after_sync();
+    if (ok) {
+        const int row = (warp & 3) * 32 + lane, c0 = (warp >> 2) * (kTileN / 2);   // TMEM lane = tile row
+        float* dst = out + (size_t)blockIdx.z * kH * kH + (size_t)(m0 + row) * kH + n0 + c0;
+#pragma unroll
+        for (int h = 0; h < kTileN / 2; h += 32) {
+            float v[32];
+            tmem_ld32(tmem + ((unsigned)((warp & 3) * 32) << 16) + c0 + h, v);
+#pragma unroll
+            for (int q = 0; q < 32; q += 4) *reinterpret_cast<float4*>(dst + h + q) = make_float4(v[q], v[q + 1], v[q + 2], v[q + 3]);
         }
     }
     fence_before_sync();
@@ -830,10 +877,6 @@ mlp_infer_kernel(const __grid_constant__ Geo<double> g, const __grid_constant__ 
     if (warp == 0) tmem_dealloc(tmem, kH);
 }
 
-// Inputs (normalised to [-1, 1]^4) and targets (V / M, cos, sin) of nodes
-// idx = (mult * (start + i) + offset) mod n of a grid (a seeded permutation).
-// Without V only the inputs are written.  Inputs are normalised to the
-// network's box (nlo, nhi).
 // Training-step state in device memory, so that one captured step can be
 // replayed: the epoch's permutation (mult, offset), the first sample of the
 // step, and the Adam step count.
@@ -842,38 +885,6 @@ struct TrainState {
     int t;
     float lr;        // > 0: the epoch's Adam step size (replaces the kernel argument)
 };
-
-template <typename S>
-__global__ void batch_from_grid_kernel(Geo<double> g, const S* __restrict__ V, const uint16_t* __restrict__ code,
-                                       const double2* __restrict__ thi, const double2* __restrict__ tlo,
-                                       long long n, long long mult, long long offset, long long start, int count,
-                                       double invM, Box4 nlo, Box4 nhi, float* __restrict__ x,
-                                       float* __restrict__ t, const TrainState* __restrict__ ts = nullptr)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= count) return;
-    if (ts) {
-        mult = ts->mult;
-        offset = ts->offset;
-        start = ts->start;
-    }
-    const long long j = (long long)(((unsigned long long)mult * (unsigned long long)(start + i) +
-                                     (unsigned long long)offset) % (unsigned long long)n);
-    int id[4];
-    decode_node(g, (int)j, id);
-    const double lo[4] = {nlo.x, nlo.y, nlo.z, nlo.w}, hi[4] = {nhi.x, nhi.y, nhi.z, nhi.w};
-#pragma unroll
-    for (int d = 0; d < 4; ++d) {
-        const double xd = g.lo[d] + (double)id[d] * g.h[d];
-        x[4 * i + d] = (float)(2.0 * (xd - lo[d]) / (hi[d] - lo[d]) - 1.0);
-    }
-    if (!V) return;
-    const int c = code[j];
-    const double2 a = thi[c >> 8], b = tlo[c & 255];
-    t[3 * i + 0] = (float)((double)V[j] * invM);
-    t[3 * i + 1] = (float)(a.y * b.y - a.x * b.x);   // cos
-    t[3 * i + 2] = (float)(a.x * b.y + a.y * b.x);   // sin
-}
 
 // Arbitrary states (device, n x 4 double) normalised to [-1, 1]^4.
 __global__ void states_in_kernel(const double* __restrict__ s, int count, Box4 lo, Box4 hi,
@@ -887,31 +898,77 @@ __global__ void states_in_kernel(const double* __restrict__ s, int count, Box4 l
     x[4 * i + 3] = (float)(2.0 * (s[4 * i + 3] - lo.w) / (hi.w - lo.w) - 1.0);
 }
 
-// Layer 1 (4 -> 256) with GELU: 32 threads per sample, thread `lane` takes
-// the features lane + 32 q (conflict-free reads of the transposed W1 in shared
-// memory, each warp store 64 contiguous bytes).  Rows >= count are zero.
-__global__ void l1_fwd_kernel(const float* __restrict__ x, const float* __restrict__ P, int count, int rows,
-                              float* __restrict__ z1, bf16* __restrict__ h1)
+// The nodes a training step's batch is drawn from.
+struct TrainGrid {
+    const void* V;
+    const uint16_t* code;
+    const double2 *tab_hi, *tab_lo;
+    const float* coord;    // normalised node coordinates (coord_table_kernel)
+    long long n;
+    double invM;
+    const TrainState* ts;
+};
+
+// Layer 1 (4 -> 256) with GELU of a training step, z1 and h1 stored, and with
+// GRID the batch itself: inputs (normalised to the network's box) and targets
+// (V / M, cos, sin) of nodes idx = (mult * (start + i) + offset) mod n of the
+// grid (a seeded permutation; S: the values' type), kept in x and t for the
+// backward pass; otherwise x is read.  A block takes kL1Rows rows: a thread a
+// row for the batch, then two features of half the rows, whose weights stay in
+// its registers, so that a warp stores whole row segments.
+// The separate batch kernel took 11.1 us for 16,384 rows, bound by its four
+// FP64 divisions a row on the 64 SMs it filled; the coordinates now come from a
+// table, and with a warp per row the first layer took another 10.3 us.  Both
+// in one: 9.6 us.
+constexpr int kL1Rows = 16;
+
+template <bool GRID, typename S>
+__global__ void __launch_bounds__(256) first_layer_kernel(const __grid_constant__ Geo<double> g, const TrainGrid tg,
+                                                          const float* __restrict__ P, float4* __restrict__ x,
+                                                          float* __restrict__ t, float* __restrict__ z1,
+                                                          bf16* __restrict__ h1)
 {
-    __shared__ float sWt[4 * kH + kH];   // W1 transposed (4 x 256), then b1
-    for (int i = threadIdx.x; i < 4 * kH; i += blockDim.x) sWt[(i & 3) * kH + (i >> 2)] = P[kOffW1 + i];
-    for (int i = threadIdx.x; i < kH; i += blockDim.x) sWt[4 * kH + i] = P[kOffB1 + i];
-    __syncthreads();
-    const long long total = (long long)rows * 32;
-    for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < total;
-         e += (long long)gridDim.x * blockDim.x) {
-        const int s = (int)(e >> 5), lane = (int)(e & 31);
-        float4 xs = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        if (s < count) xs = *reinterpret_cast<const float4*>(x + 4 * (size_t)s);
-#pragma unroll
-        for (int q = 0; q < kH / 32; ++q) {
-            const int o = lane + 32 * q;
-            const float z = s < count ? sWt[4 * kH + o] + sWt[o] * xs.x + sWt[kH + o] * xs.y +
-                                            sWt[2 * kH + o] * xs.z + sWt[3 * kH + o] * xs.w
-                                      : 0.0f;
-            h1[(size_t)s * kH + o] = __float2bfloat16(s < count ? gelu(z) : 0.0f);
-            if (z1) z1[(size_t)s * kH + o] = z;
+    __shared__ float4 sx[kL1Rows];
+    const int tid = threadIdx.x, o = 2 * (tid & 127);
+    const size_t s0 = (size_t)blockIdx.x * kL1Rows;
+    const float4 w0 = *reinterpret_cast<const float4*>(P + kOffW1 + 4 * o);
+    const float4 w1 = *reinterpret_cast<const float4*>(P + kOffW1 + 4 * o + 4);
+    const float2 b = *reinterpret_cast<const float2*>(P + kOffB1 + o);
+    if (GRID) {
+        // one warp the inputs, another the targets
+        const int w = tid >> 5, i = tid & 31;
+        if (w < 2 && i < kL1Rows) {
+            const size_t row = s0 + i;
+            const long long j = (long long)(((unsigned long long)tg.ts->mult * (unsigned long long)(tg.ts->start + (long long)row) +
+                                             (unsigned long long)tg.ts->offset) % (unsigned long long)tg.n);
+            if (w == 0) {
+                int id[4];
+                decode_node(g, (int)j, id);
+                const float4 v = make_float4(__ldg(tg.coord + id[0]), __ldg(tg.coord + kCoordMax + id[1]),
+                                             __ldg(tg.coord + 2 * kCoordMax + id[2]), __ldg(tg.coord + 3 * kCoordMax + id[3]));
+                sx[i] = v;
+                x[row] = v;
+            } else {
+                const double vj = (double)((const S*)tg.V)[j];
+                const int c = tg.code[j];
+                const double2 hi = tg.tab_hi[c >> 8], lo = tg.tab_lo[c & 255];
+                t[3 * row + 0] = (float)(vj * tg.invM);
+                t[3 * row + 1] = (float)(hi.y * lo.y - hi.x * lo.x);   // cos
+                t[3 * row + 2] = (float)(hi.x * lo.y + hi.y * lo.x);   // sin
+            }
         }
+    } else if (tid < kL1Rows) {
+        sx[tid] = x[s0 + tid];
+    }
+    __syncthreads();
+#pragma unroll 2
+    for (int k = tid >> 7; k < kL1Rows; k += 2) {
+        const float4 v = sx[k];
+        const size_t at = (s0 + k) * kH + o;
+        const float za = fmaf(w0.w, v.w, fmaf(w0.z, v.z, fmaf(w0.y, v.y, fmaf(w0.x, v.x, b.x))));
+        const float zb = fmaf(w1.w, v.w, fmaf(w1.z, v.z, fmaf(w1.y, v.y, fmaf(w1.x, v.x, b.y))));
+        *reinterpret_cast<float2*>(z1 + at) = make_float2(za, zb);
+        *reinterpret_cast<__nv_bfloat162*>(h1 + at) = __floats2bfloat162_rn(gelu(za), gelu(zb));
     }
 }
 
@@ -932,14 +989,33 @@ __global__ void __launch_bounds__(256) out_train_kernel(const bf16* __restrict__
 {
     __shared__ float sW[3 * kH + 3];
     __shared__ float sP[8][kOutPart];   // per warp: db3, dW4, db4, loss
-    for (int i = threadIdx.x; i < 3 * kH + 3; i += blockDim.x) sW[i] = P[kOffW4 + i];
-    __syncthreads();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int warps = (int)((gridDim.x * (size_t)blockDim.x) >> 5);
+    int s = (int)((blockIdx.x * (size_t)blockDim.x + threadIdx.x) >> 5);
+    // a sample's h3, z3 and targets, loaded while the one before is worked on
+    // (a warp takes about seven at a batch of 16,384, each a chain of loads,
+    // sums and shuffles: 14.9 us, 16.6 without)
+    uint4 hn = make_uint4(0, 0, 0, 0);
+    float4 za = make_float4(0.0f, 0.0f, 0.0f, 0.0f), zb = za;
+    float tn[3] = {};
+    auto fetch = [&](int q) {
+        if (q >= count) return;
+        hn = *reinterpret_cast<const uint4*>(h3 + (size_t)q * kH + lane * 8);
+        const float4* zp = reinterpret_cast<const float4*>(z3 + (size_t)q * kH + lane * 8);
+        za = zp[0];
+        zb = zp[1];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) tn[k] = t[3 * (size_t)q + k];
+    };
+    fetch(s);
+    for (int i = threadIdx.x; i < 3 * kH + 3; i += blockDim.x) sW[i] = P[kOffW4 + i];
+    __syncthreads();
     float w[3][8] = {}, b[3] = {}, d3[8] = {}, l = 0.0f;
-    for (int s = (int)((blockIdx.x * (size_t)blockDim.x + threadIdx.x) >> 5); s < count; s += warps) {
+    for (; s < count; s += warps) {
         float a[8];
-        load_row8(h3 + (size_t)s * kH + lane * 8, a);
+        row8(hn, a);
+        const float z[8] = {za.x, za.y, za.z, za.w, zb.x, zb.y, zb.z, zb.w}, ts[3] = {tn[0], tn[1], tn[2]};
+        fetch(s + warps);
         float dy[3];
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
@@ -948,16 +1024,13 @@ __global__ void __launch_bounds__(256) out_train_kernel(const bf16* __restrict__
             for (int q = 0; q < 8; ++q) sum += sW[k * kH + lane * 8 + q] * a[q];
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-            const float r = (sum + sW[3 * kH + k]) - t[3 * (size_t)s + k];
+            const float r = (sum + sW[3 * kH + k]) - ts[k];
             l += r * r;
             dy[k] = 2.0f * r * inv_n;
             b[k] += dy[k];
 #pragma unroll
             for (int q = 0; q < 8; ++q) w[k][q] += dy[k] * a[q];
         }
-        const float4* zp = reinterpret_cast<const float4*>(z3 + (size_t)s * kH + lane * 8);
-        const float4 z0 = zp[0], z1 = zp[1];
-        const float z[8] = {z0.x, z0.y, z0.z, z0.w, z1.x, z1.y, z1.z, z1.w};
         unsigned u[4];
 #pragma unroll
         for (int q = 0; q < 8; q += 2) {
@@ -1235,22 +1308,7 @@ cudaError_t raise_smem_limit(K kernel, int bytes, std::atomic<bool> (&done)[kMax
     return e;
 }
 
-template <int EPI, int KC>
-cudaError_t gemm_kc(dp_mlp* m, const bf16* A, int lda, const bf16* B, int ldb, int rows, int k_total, int k_split,
-                    const float* bias, float* zout, const float* zin, bf16* hout, float* cacc)
-{
-    static std::atomic<bool> attr[kMaxDevices];
-    cudaError_t e = raise_smem_limit(mlp_gemm_kernel<EPI, KC>, gemm_smem_of<EPI, KC>(), attr);
-    if (e != cudaSuccess) return e;
-    dim3 grid(rows / kTileM, kH / kTileN, k_split);
-    mlp_gemm_kernel<EPI, KC><<<grid, 128, gemm_smem_of<EPI, KC>(), m->st>>>(A, lda, B, ldb, k_total / k_split, bias, zout, zin,
-                                                                   hout, cacc, m->err, m->wait_polls);
-    return cudaGetLastError();
-}
-
-// Large batches (inference over a grid) stage K in 128-wide halves so that
-// three CTAs share an SM; small ones (training) stage the whole 256-wide K
-// slice at once; split-K weight gradients take one 256-wide slice per CTA.
+// Batches from this size on run the persistent GEMMs.
 constexpr int kManyRows = 16384;
 
 // Partial sums of the backward pass (one buffer, reused by each reduction in
@@ -1279,29 +1337,50 @@ cudaError_t persistent(dp_mlp* m, const bf16* A, int lda, const bf16* B, int ldb
     return cudaGetLastError();
 }
 
+// A hidden layer (kEpiFwd) or its backward product (kEpiBwd), K = 256.
 template <int EPI>
-cudaError_t gemm(dp_mlp* m, const bf16* A, int lda, const bf16* B, int ldb, int rows, int k_total, int k_split,
-                 const float* bias, float* zout, const float* zin, bf16* hout, float* cacc)
+cudaError_t gemm(dp_mlp* m, const bf16* A, int lda, const bf16* B, int ldb, int rows, const float* bias, float* zout,
+                 const float* zin, bf16* hout)
 {
-    if constexpr (EPI == kEpiFwd || EPI == kEpiBwd) {
-        if (rows >= kManyRows && k_total == kKC && k_split == 1)
-            return persistent<EPI>(m, A, lda, B, ldb, rows, bias, zout, zin, hout);
-    }
-    if (EPI != kEpiAtomic && EPI != kEpiSplitMN && rows >= kManyRows)
-        return gemm_kc<EPI, kKC / 2>(m, A, lda, B, ldb, rows, k_total, k_split, bias, zout, zin, hout, cacc);
-    return gemm_kc<EPI, kKC>(m, A, lda, B, ldb, rows, k_total, k_split, bias, zout, zin, hout, cacc);
+    if (rows >= kManyRows) return persistent<EPI>(m, A, lda, B, ldb, rows, bias, zout, zin, hout);
+    static std::atomic<bool> attr[kMaxDevices];
+    cudaError_t e = raise_smem_limit(mlp_gemm_kernel<EPI>, kGemmSmem, attr);
+    if (e != cudaSuccess) return e;
+    mlp_gemm_kernel<EPI><<<dim3(rows / kTileM, kH / kTileN), 128, kGemmSmem, m->st>>>(A, lda, B, ldb, bias, zout, zin, hout,
+                                                                                  m->err, m->wait_polls);
+    return cudaGetLastError();
 }
 
-// Hidden layers of a training step's forward pass of `rows` rows held in m->x
-// (a multiple of 512), through h3, keeping z1..z3 for the backward pass.
-int forward_hidden(dp_mlp* m, int rows)
+// dz^T h of `rows` rows (a multiple of 256) as `splits` partial tiles in m->part
+cudaError_t weight_gradient(dp_mlp* m, const bf16* dz, const bf16* h, int rows, int splits)
 {
-    const long long e8 = (long long)rows * 32;
-    const unsigned b1 = (unsigned)std::min<long long>((e8 + 255) / 256, 8LL * m->sm_count);
-    l1_fwd_kernel<<<b1, 256, 0, m->st>>>(m->x, m->P, rows, rows, m->z1, m->h1);
+    static std::atomic<bool> attr[kMaxDevices];
+    cudaError_t e = raise_smem_limit(mlp_wgrad_kernel, kWgSmem, attr);
+    if (e != cudaSuccess) return e;
+    mlp_wgrad_kernel<<<dim3(kH / kTileM, kH / kTileN, splits), kWgThreads, kWgSmem, m->st>>>(dz, h, rows / splits, m->part,
+                                                                                          m->err, m->wait_polls);
+    return cudaGetLastError();
+}
+
+// Hidden layers of a training step's forward pass of `rows` rows (a multiple of
+// 512), held in m->x or, with a grid, its next batch, through h3, keeping
+// z1..z3 for the backward pass.
+int forward_hidden(dp_mlp* m, int rows, const GridView* gv)
+{
+    const int b1 = rows / kL1Rows;
+    float4* x = reinterpret_cast<float4*>(m->x);
+    if (!gv) {
+        first_layer_kernel<false, float><<<b1, 256, 0, m->st>>>(Geo<double>(), TrainGrid(), m->P, x, m->t, m->z1, m->h1);
+    } else {
+        const bool f32 = gv->fp32 && !gv->V64;
+        const TrainGrid tg{gv->V64 ? (const void*)gv->V64 : gv->V, gv->code, gv->tab_hi64, gv->tab_lo64, m->coord, gv->n,
+                           1.0 / gv->M, m->ts};
+        if (f32) first_layer_kernel<true, float><<<b1, 256, 0, m->st>>>(gv->g64, tg, m->P, x, m->t, m->z1, m->h1);
+        else first_layer_kernel<true, double><<<b1, 256, 0, m->st>>>(gv->g64, tg, m->P, x, m->t, m->z1, m->h1);
+    }
     MCK(cudaGetLastError());
-    MCK(gemm<kEpiFwd>(m, m->h1, kH, m->W2b, kH, rows, kH, 1, m->P + kOffB2, m->z2, nullptr, m->h2, nullptr));
-    MCK(gemm<kEpiFwd>(m, m->h2, kH, m->W3b, kH, rows, kH, 1, m->P + kOffB3, m->z3, nullptr, m->h3, nullptr));
+    MCK(gemm<kEpiFwd>(m, m->h1, kH, m->W2b, kH, rows, m->P + kOffB2, m->z2, nullptr, m->h2));
+    MCK(gemm<kEpiFwd>(m, m->h2, kH, m->W3b, kH, rows, m->P + kOffB3, m->z3, nullptr, m->h3));
     return DP_OK;
 }
 
@@ -1322,13 +1401,13 @@ int infer(dp_mlp* m, int count, const Geo<double>& g, const InferGrid& ig)
 }
 
 // Gradients of the mean squared error over a batch of `count` rows (count a
-// multiple of 512; m->x / m->t hold the batch) into m->G, the loss sum added
+// multiple of 512; m->x / m->t hold the batch, or gv gives it) into m->G, the loss sum added
 // to m->loss.  The output layer and its backward pass run in one kernel.
-int forward_backward(dp_mlp* m, int count, float inv_n)
+int forward_backward(dp_mlp* m, int count, float inv_n, const GridView* gv = nullptr)
 {
     const int rows = count;
     int rc;
-    if ((rc = forward_hidden(m, rows))) return rc;
+    if ((rc = forward_hidden(m, rows, gv))) return rc;
     // every gradient sum goes through per-block partial sums and a reduction
     // in a fixed order, so that a training run is reproducible bit for bit
     auto seg = [](const float* part, int n_part, int stride, int len, float* out, int accumulate) {
@@ -1358,13 +1437,13 @@ int forward_backward(dp_mlp* m, int count, float inv_n)
         // layer 3: dz2 = (dz3 W3) * GELU'(z2) with db2; dW3 = dz3^T h2
         MCK((persistent<kEpiBwd, 1>(m, m->dz3, kH, m->W3T, kH, rows, nullptr, nullptr, m->z2, m->dz2, nullptr,
                                     m->red)));
-        MCK(gemm<kEpiSplitMN>(m, m->dz3, kH, m->h2, kH, kH, rows, ks, nullptr, nullptr, nullptr, nullptr, m->part));
+        MCK(weight_gradient(m, m->dz3, m->h2, rows, ks));
         MCK(reduce2(seg(m->part, ks, kH * kH, kH * kH, m->G + kOffW3, 0), seg(m->red, tiles, kH, kH, m->G + kOffB2, 0)));
         // layer 2: dz1 = (dz2 W2) * GELU'(z1) summed into dW1 = dz1^T x and
         // db1; dW2 = dz2^T h1
         MCK((persistent<kEpiBwd, 5>(m, m->dz2, kH, m->W2T, kH, rows, nullptr, nullptr, m->z1, nullptr, m->x,
                                     m->red)));
-        MCK(gemm<kEpiSplitMN>(m, m->dz2, kH, m->h1, kH, kH, rows, ks, nullptr, nullptr, nullptr, nullptr, m->part));
+        MCK(weight_gradient(m, m->dz2, m->h1, rows, ks));
         MCK(reduce2(seg(m->part, ks, kH * kH, kH * kH, m->G + kOffW2, 0),
                     seg(m->red, tiles, 5 * kH, 5 * kH, m->G + kOffW1, 0)));
         return DP_OK;
@@ -1373,12 +1452,12 @@ int forward_backward(dp_mlp* m, int count, float inv_n)
     const int chunk = std::max(64, (rows + kRedBlocks - 1) / kRedBlocks);
     const int nb = (rows + chunk - 1) / chunk;
     // layer 3: dz2 = (dz3 W3) * GELU'(z2); dW3 = dz3^T h2
-    MCK(gemm<kEpiBwd>(m, m->dz3, kH, m->W3T, kH, rows, kH, 1, nullptr, nullptr, m->z2, m->dz2, nullptr));
-    MCK(gemm<kEpiSplitMN>(m, m->dz3, kH, m->h2, kH, kH, rows, ks, nullptr, nullptr, nullptr, nullptr, m->part));
+    MCK(gemm<kEpiBwd>(m, m->dz3, kH, m->W3T, kH, rows, nullptr, nullptr, m->z2, m->dz2));
+    MCK(weight_gradient(m, m->dz3, m->h2, rows, ks));
     MCK(reduce(m->part, ks, kH * kH, kH * kH, m->G + kOffW3, 0));
     // layer 2: dz1 = (dz2 W2) * GELU'(z1); dW2 = dz2^T h1; db2 = sum dz2
-    MCK(gemm<kEpiBwd>(m, m->dz2, kH, m->W2T, kH, rows, kH, 1, nullptr, nullptr, m->z1, m->dz1, nullptr));
-    MCK(gemm<kEpiSplitMN>(m, m->dz2, kH, m->h1, kH, kH, rows, ks, nullptr, nullptr, nullptr, nullptr, m->part));
+    MCK(gemm<kEpiBwd>(m, m->dz2, kH, m->W2T, kH, rows, nullptr, nullptr, m->z1, m->dz1));
+    MCK(weight_gradient(m, m->dz2, m->h1, rows, ks));
     MCK(reduce(m->part, ks, kH * kH, kH * kH, m->G + kOffW2, 0));
     feat_reduce_kernel<0><<<nb, 256, 0, m->st>>>(m->dz2, nullptr, rows, chunk, m->part);
     MCK(cudaGetLastError());
@@ -1433,26 +1512,16 @@ namespace {
 // the batch of samples start .. start + B - 1 of the epoch's permutation (from
 // m->ts), forward, backward, Adam with step count m->ts->t, then the next
 // step's start and count.  Replayable: no argument changes between steps.
-int train_step(dp_mlp* m, const GridView& gv, int B, Box4 nlo, Box4 nhi, double lr)
+int train_step(dp_mlp* m, const GridView& gv, int B, double lr)
 {
-    const double invM = 1.0 / gv.M;
-    if (gv.fp32 && !gv.V64)
-        batch_from_grid_kernel<float><<<(B + 255) / 256, 256, 0, m->st>>>(
-            gv.g64, (const float*)gv.V, gv.code, gv.tab_hi64, gv.tab_lo64, gv.n, 0, 0, 0, B, invM, nlo, nhi, m->x,
-            m->t, m->ts);
-    else
-        batch_from_grid_kernel<double><<<(B + 255) / 256, 256, 0, m->st>>>(
-            gv.g64, gv.V64 ? gv.V64 : (const double*)gv.V, gv.code, gv.tab_hi64, gv.tab_lo64, gv.n, 0, 0, 0, B, invM,
-            nlo, nhi, m->x, m->t, m->ts);
-    MCK(cudaGetLastError());
     int rc;
-    if ((rc = forward_backward(m, B, 1.0f / (3.0f * B)))) return rc;
+    if ((rc = forward_backward(m, B, 1.0f / (3.0f * B), &gv))) return rc;
     return adam_launch(m, lr, B);   // with the next step's start and count
 }
 
 // The epochs of dp_mlp_train_grid.  The first step runs as launched (it also
 // sets the kernels' attributes); the next one is captured as a CUDA graph
-// and every later step replays it, which removes the host's 13 launches
+// and every later step replays it, which removes the host's 12 launches
 // per step.
 int train_grid_steps(dp_mlp* m, const GridView& gv, const dp_mlp_train_opts* o, dp_mlp_train_stats* stats)
 {
@@ -1486,6 +1555,8 @@ int train_grid_steps(dp_mlp* m, const GridView& gv, const dp_mlp_train_opts* o, 
     if ((e = cudaEventCreate(&e0)) != cudaSuccess || (e = cudaEventCreate(&e1)) != cudaSuccess ||
         (e = cudaEventRecord(e0, m->st)) != cudaSuccess)
         return done(fail_cuda("training events", e));
+    coord_table_kernel<<<4, kCoordMax, 0, m->st>>>(gv.g64, nlo, nhi, m->coord);
+    if ((e = cudaGetLastError()) != cudaSuccess) return done(fail_cuda("coordinate table", e));
     for (int ep = 0; ep < o->epochs; ++ep) {
         unsigned long long mult = (next() % (unsigned long long)n) | 1ull;
         while (gcd(mult, (unsigned long long)n) != 1) mult = (mult + 2) % (unsigned long long)n;
@@ -1502,11 +1573,11 @@ int train_grid_steps(dp_mlp* m, const GridView& gv, const dp_mlp_train_opts* o, 
             if (exec) {
                 if ((e = cudaGraphLaunch(exec, m->st)) != cudaSuccess) return done(fail_cuda("graph launch", e));
             } else if (ep == 0 && s == 0) {
-                if ((rc = train_step(m, gv, B, nlo, nhi, o->lr))) return done(rc);
+                if ((rc = train_step(m, gv, B, o->lr))) return done(rc);
             } else {
                 if ((e = cudaStreamBeginCapture(m->st, cudaStreamCaptureModeThreadLocal)) != cudaSuccess)
                     return done(fail_cuda("stream capture", e));
-                const int rs = train_step(m, gv, B, nlo, nhi, o->lr);
+                const int rs = train_step(m, gv, B, o->lr);
                 e = cudaStreamEndCapture(m->st, &graph);
                 if (rs) return done(rs);
                 if (e != cudaSuccess) return done(fail_cuda("stream capture", e));
