@@ -103,6 +103,36 @@ __device__ __forceinline__ void cp_async_wait_all()
     asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;" ::: "memory");
 }
 
+// The 128 x 256 operand of 128 rows from r0 of a row-major matrix into shared
+// memory (64 KB): four blocks of 64 columns, 128-byte swizzled, K-major.  A warp
+// copies one whole row, every 16-byte piece straight to shared memory
+// (cp.async).  Taking 64 bytes of eight rows each, as the layout without a
+// swizzle wants, a warp's copy touched eight lines per eight lanes and fetched
+// every sector twice.
+constexpr int kOpBlock = kTileM * 128;    // bytes of a block of 64 columns
+
+template <int THREADS>
+__device__ __forceinline__ void stage_rows(unsigned char* dst, const bf16* src, size_t ld, size_t r0)
+{
+#pragma unroll 8
+    for (int q = 0; q < kTileM * kKC / 8 / THREADS; ++q) {
+        const int v = (int)threadIdx.x + THREADS * q, row = v >> 5, c = v & 31;
+        cp_async16(dst + (c >> 3) * kOpBlock + sw128(row, c & 7), src + (r0 + row) * ld + c * 8);
+    }
+}
+
+// The 16 MMAs of such a pair of operands; one thread.
+__device__ __forceinline__ void mma_rows(unsigned tmem, const unsigned char* sA, const unsigned char* sB)
+{
+    constexpr unsigned idesc = umma_idesc_bf16(kTileM, kTileN);
+#pragma unroll
+    for (int s = 0; s < kKC / 16; ++s) {
+        const unsigned at = (s >> 2) * kOpBlock + (s & 3) * 32;
+        umma_bf16(tmem, umma_desc_sw128(smem_u32(sA) + at, 16, 1024), umma_desc_sw128(smem_u32(sB) + at, 16, 1024), idesc,
+                  s > 0 ? 1u : 0u);
+    }
+}
+
 // C[128 x 128 tile] = A[rows, 256] * B[256, 256]^T on tcgen05, for batches
 // below kManyRows rows.
 //   A: bf16 [*, lda] row-major (K contiguous); B: bf16 [256, ldb] row-major.
@@ -131,38 +161,15 @@ mlp_gemm_kernel(const bf16* __restrict__ A, int lda, const bf16* __restrict__ B,
     const unsigned tmem = tmem_slot;
     const size_t row0 = (size_t)blockIdx.x * kTileM;
     const int n0 = blockIdx.y * kTileN;
-    constexpr unsigned idesc = umma_idesc_bf16(kTileM, kTileN);
-    constexpr int kGroups = kKC / 8;                 // 16-byte groups per row
 
-    // core-matrix staging: (row, kb) -> ((row / 8) * kGroups + kb) * 128 + (row % 8) * 16.
-    // A warp takes 8 rows x 4 consecutive 16-byte groups: 64 contiguous bytes
-    // of each row in global memory, 512 contiguous bytes (no bank conflict)
-    // in shared memory.  The groups go straight to shared memory (cp.async):
-    // every one is in flight at once, none through registers.
-#pragma unroll
-    for (int q = 0; q < kTileM * kGroups / 128; ++q) {
-        const int v = tid + 128 * q, grp = v >> 5, ln = v & 31;
-        const int row = (grp / (kGroups / 4)) * 8 + (ln & 7), kb = (grp % (kGroups / 4)) * 4 + (ln >> 3);
-        cp_async16(sA + (size_t)v * 16, A + (row0 + row) * (size_t)lda + kb * 8);
-    }
-#pragma unroll
-    for (int q = 0; q < kTileN * kGroups / 128; ++q) {
-        const int v = tid + 128 * q, grp = v >> 5, ln = v & 31;
-        const int row = (grp / (kGroups / 4)) * 8 + (ln & 7), kb = (grp % (kGroups / 4)) * 4 + (ln >> 3);
-        cp_async16(sB + (size_t)v * 16, B + (size_t)(n0 + row) * ldb + kb * 8);
-    }
+    stage_rows<128>(sA, A, (size_t)lda, row0);
+    stage_rows<128>(sB, B, (size_t)ldb, (size_t)n0);
     cp_async_wait_all();
     fence_async_smem();
     __syncthreads();
     if (tid == 0) {
         fence_after_sync();
-#pragma unroll
-        for (int s = 0; s < kKC / 16; ++s) {
-            // K step s: two K blocks, 256 bytes on
-            const unsigned long long ad = umma_desc(smem_u32(sA) + s * 256, 128, kGroups * 128);
-            const unsigned long long bd = umma_desc(smem_u32(sB) + s * 256, 128, kGroups * 128);
-            umma_bf16(tmem, ad, bd, idesc, s > 0 ? 1u : 0u);
-        }
+        mma_rows(tmem, sA, sB);
         umma_commit(&mbar);
     }
     bool ok = true;
@@ -219,15 +226,13 @@ mlp_gemm_kernel(const bf16* __restrict__ A, int lda, const bf16* __restrict__ B,
 // kWgRows) from k_per_cta blockIdx.z of A = dz and B = h, both rows x 256, read
 // as they are (both operands MN-major, no transposed copies).  The tile is
 // stored at split blockIdx.z of out (256 x 256 floats per split), for a
-// reduction in a fixed order.  Core matrix (K block kb, MN block mb) holds 8
-// rows of 8 contiguous columns at byte (kb * 16 + mb) * 128: 128 bytes to the
-// next MN block, 2048 to the next K block.
+// reduction in a fixed order.
 //
 // What bounds it: 256 KB of operands per CTA from L2 (two row slabs of 512 at a
 // batch of 16,384, 128 CTAs, about 2.1 us at 64 bytes a clock), and the latency
 // of the first and of the epilogue.  Rows pass through a ring of six 32 KB
 // chunks of 64 rows, five ahead of the MMAs; staged 256 rows at a time with
-// nothing in flight during their MMAs it took 15.3 us, now 14.0.
+// nothing in flight during their MMAs it took 15.3 us, now 8.2 (14.0 while its copies took 64 bytes of eight rows each).
 constexpr int kWgRows = 64, kWgSlots = 6, kWgThreads = 256;
 constexpr int kWgChunk = kWgRows * kTileM * 2;                     // bytes of one operand's chunk
 constexpr int kWgSmem = kWgSlots * 2 * kWgChunk;                   // 192 KB
@@ -242,17 +247,17 @@ mlp_wgrad_kernel(const bf16* __restrict__ A, const bf16* __restrict__ B, int k_p
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int m0 = blockIdx.x * kTileM, n0 = blockIdx.y * kTileN, kbeg = blockIdx.z * k_per_cta;
     const int chunks = k_per_cta / kWgRows;
-    // a warp takes 8 rows x 4 consecutive MN blocks: 64 contiguous bytes of
-    // each row in global memory, 512 in shared memory
+    // a chunk is two halves of 64 columns, 128-byte swizzled; a warp copies two
+    // rows of 128 columns
     auto stage = [&](int c) {
         unsigned char* dst = smem + (c % kWgSlots) * 2 * kWgChunk;
         const size_t k0 = (size_t)kbeg + (size_t)c * kWgRows;
 #pragma unroll
         for (int q = 0; q < 2 * kWgChunk / 16 / kWgThreads; ++q) {
-            const int v = tid + kWgThreads * (q % (kWgChunk / 16 / kWgThreads)), grp = v >> 5;
-            const int kr = (grp >> 2) * 8 + (lane & 7), mb = (grp & 3) * 4 + (lane >> 3);
-            if (q < kWgChunk / 16 / kWgThreads) cp_async16(dst + (size_t)v * 16, A + (k0 + kr) * kH + m0 + mb * 8);
-            else cp_async16(dst + kWgChunk + (size_t)v * 16, B + (k0 + kr) * kH + n0 + mb * 8);
+            const int v = tid + kWgThreads * (q % (kWgChunk / 16 / kWgThreads)), kr = v >> 4, c = v & 15;
+            const unsigned at = (c >> 3) * (kWgChunk / 2) + sw128(kr, c & 7);
+            if (q < kWgChunk / 16 / kWgThreads) cp_async16(dst + at, A + (k0 + kr) * kH + m0 + c * 8);
+            else cp_async16(dst + kWgChunk + at, B + (k0 + kr) * kH + n0 + c * 8);
         }
     };
     // one group of copies per chunk and turn, empty ones included, so that the
@@ -280,9 +285,9 @@ mlp_wgrad_kernel(const bf16* __restrict__ A, const bf16* __restrict__ B, int k_p
             fence_after_sync();
             const unsigned sa = smem_u32(smem + (c % kWgSlots) * 2 * kWgChunk);
 #pragma unroll
-            for (int s = 0; s < kWgRows / 16; ++s)   // K step s: two K blocks
-                umma_bf16(tmem, umma_desc(sa + s * 4096, 2048, 128), umma_desc(sa + kWgChunk + s * 4096, 2048, 128), idesc,
-                          c > 0 || s > 0 ? 1u : 0u);
+            for (int s = 0; s < kWgRows / 16; ++s)   // K step s: two atoms of 8 rows
+                umma_bf16(tmem, umma_desc_sw128(sa + s * 2048, kWgChunk / 2, 1024),
+                          umma_desc_sw128(sa + kWgChunk + s * 2048, kWgChunk / 2, 1024), idesc, c > 0 || s > 0 ? 1u : 0u);
             umma_commit(&done[c % kWgSlots]);
         }
         // the slot of the chunk before takes the chunk five on once its MMAs are done
@@ -367,22 +372,9 @@ mlp_persistent_kernel(const bf16* __restrict__ A, int lda, const bf16* __restric
     __syncthreads();
     fence_after_sync();
     const unsigned tmem = tmem_slot;
-    constexpr unsigned idesc = umma_idesc_bf16(kTileM, kTileN);
-    constexpr int kGroups = kKC / 8;
-
-    // (row, kb) -> ((row / 8) * kGroups + kb) * 128 + (row % 8) * 16, a warp
-    // taking 8 rows x 4 consecutive 16-byte groups
-    auto stage = [&](unsigned char* dst, const bf16* src, size_t ld, size_t r0) {
-#pragma unroll 4
-        for (int q = 0; q < kTileM * kGroups / kPersistThreads; ++q) {
-            const int v = tid + kPersistThreads * q, grp = v >> 5, ln = v & 31;
-            const int row = (grp / (kGroups / 4)) * 8 + (ln & 7), kb = (grp % (kGroups / 4)) * 4 + (ln >> 3);
-            cp_async16(dst + (size_t)v * 16, src + (r0 + row) * ld + kb * 8);
-        }
-    };
-    stage(sB, B, (size_t)ldb, (size_t)n0);
+    stage_rows<kPersistThreads>(sB, B, (size_t)ldb, (size_t)n0);
     int t = blockIdx.x;
-    if (t < tiles) stage(sA[0], A, (size_t)lda, (size_t)t * kTileM);
+    if (t < tiles) stage_rows<kPersistThreads>(sA[0], A, (size_t)lda, (size_t)t * kTileM);
     cp_async_wait_all();
     fence_async_smem();
     __syncthreads();
@@ -392,18 +384,13 @@ mlp_persistent_kernel(const bf16* __restrict__ A, int lda, const bf16* __restric
     for (; t < tiles; t += gridDim.x, buf ^= 1) {
         if (tid == 0) {
             fence_after_sync();
-#pragma unroll
-            for (int s = 0; s < kKC / 16; ++s) {
-                const unsigned long long ad = umma_desc(smem_u32(sA[buf]) + s * 256, 128, kGroups * 128);
-                const unsigned long long bd = umma_desc(smem_u32(sB) + s * 256, 128, kGroups * 128);
-                umma_bf16(tmem, ad, bd, idesc, s > 0 ? 1u : 0u);
-            }
+            mma_rows(tmem, sA[buf], sB);
             umma_commit(&mbar);
         }
         // the next tile's activations, into the other buffer (its last
         // reader, the previous tile's MMAs, has completed)
         const int tn = t + gridDim.x;
-        if (tn < tiles) stage(sA[buf ^ 1], A, (size_t)lda, (size_t)tn * kTileM);
+        if (tn < tiles) stage_rows<kPersistThreads>(sA[buf ^ 1], A, (size_t)lda, (size_t)tn * kTileM);
         if (!mbar_wait(&mbar, phase, polls)) {
             ok = false;
             if (lane == 0) atomicOr(err, 1);

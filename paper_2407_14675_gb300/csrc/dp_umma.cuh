@@ -31,6 +31,22 @@ __device__ __forceinline__ unsigned long long umma_desc(unsigned addr, unsigned 
     return d;
 }
 
+// The same with the 128-byte swizzle: the tile is made of atoms of 8 rows of 128
+// bytes (1024 bytes, aligned to 1024), the 16-byte piece c of row r kept at
+// piece c ^ (r mod 8).  A warp's copies can then take whole 128-byte pieces of
+// global rows and still write shared memory without bank conflicts (sw128()).
+//   K-major: a row is 64 elements of K; sbo to the next 8 rows; a K step of 16
+//     starts 32 bytes on (lbo is not used);
+//   MN-major: a row is 64 elements of MN at one K; lbo to the next 64 of MN, sbo
+//     to the next 8 of K.
+__device__ __forceinline__ unsigned long long umma_desc_sw128(unsigned addr, unsigned lbo, unsigned sbo)
+{
+    return umma_desc(addr, lbo, sbo) | (2ull << 61);
+}
+
+// Byte offset of piece c (0..7) of row r in such atoms.
+__device__ __forceinline__ unsigned sw128(int r, int c) { return (unsigned)(r * 128 + ((c ^ (r & 7)) << 4)); }
+
 // Instruction descriptor of kind::f16: FP32 accumulator, BF16 A and B, both
 // K-major, N / 8 and M / 16.
 __host__ __device__ constexpr unsigned umma_idesc_bf16(int M, int N)
