@@ -221,31 +221,42 @@ mlp_gemm_kernel(const bf16* __restrict__ A, int lda, const bf16* __restrict__ B,
     if (warp == 0) tmem_dealloc(tmem, kTileN);
 }
 
-// Weight gradient dz^T h of a hidden layer, split along the batch: the tile
+// Weight gradients dz^T h of both hidden layers, split along the batch: the tile
 // C[128 blockIdx.x.., 128 blockIdx.y..] over the k_per_cta rows (a multiple of
-// kWgRows) from k_per_cta blockIdx.z of A = dz and B = h, both rows x 256, read
-// as they are (both operands MN-major, no transposed copies).  The tile is
+// kWgRows) from k_per_cta (blockIdx.z mod splits) of A = dz and B = h, both rows
+// x 256, read as they are (both operands MN-major, no transposed copies); the
+// first `splits` z of the grid are one layer, the others the next.  The tile is
 // stored at split blockIdx.z of out (256 x 256 floats per split), for a
 // reduction in a fixed order.
 //
-// What bounds it: 256 KB of operands per CTA from L2 (two row slabs of 512 at a
-// batch of 16,384, 128 CTAs, about 2.1 us at 64 bytes a clock), and the latency
-// of the first and of the epilogue.  Rows pass through a ring of six 32 KB
-// chunks of 64 rows, five ahead of the MMAs; staged 256 rows at a time with
-// nothing in flight during their MMAs it took 15.3 us, now 8.2 (14.0 while its copies took 64 bytes of eight rows each).
-constexpr int kWgRows = 64, kWgSlots = 6, kWgThreads = 256;
+// What bounds it: 256 KB of operands per CTA from L2 (two slabs of 512 rows at a
+// batch of 16,384, 256 CTAs), and the latency of the first of them and of the
+// epilogue.  Rows pass through a ring of three 32 KB chunks of 64 rows, two
+// ahead of the MMAs, and two CTAs share an SM: 13.4 us for both layers.
+// A launch per layer (128 CTAs) with a ring of six took 8.2 us each, 14.0 while
+// a warp's copies took 64 bytes of eight rows, and 15.3 with 256 rows staged at a
+// time and nothing in flight during their MMAs.
+constexpr int kWgRows = 64, kWgSlots = 3, kWgThreads = 256;
 constexpr int kWgChunk = kWgRows * kTileM * 2;                     // bytes of one operand's chunk
-constexpr int kWgSmem = kWgSlots * 2 * kWgChunk;                   // 192 KB
+constexpr int kWgSmem = kWgSlots * 2 * kWgChunk;                   // 96 KB
 
-__global__ void __launch_bounds__(kWgThreads)
-mlp_wgrad_kernel(const bf16* __restrict__ A, const bf16* __restrict__ B, int k_per_cta, float* __restrict__ out,
+struct WgPair {
+    const bf16 *A[2], *B[2];
+};
+
+__global__ void __launch_bounds__(kWgThreads, 2)
+mlp_wgrad_kernel(const __grid_constant__ WgPair p, int splits, int k_per_cta, float* __restrict__ out,
                  int* __restrict__ err, int polls)
 {
+    const bool second = (int)blockIdx.z >= splits;
+    const bf16* __restrict__ A = second ? p.A[1] : p.A[0];
+    const bf16* __restrict__ B = second ? p.B[1] : p.B[0];
     extern __shared__ __align__(1024) unsigned char smem[];
     __shared__ unsigned tmem_slot;
     __shared__ __align__(8) unsigned long long done[kWgSlots];     // the slot's MMAs have completed
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int m0 = blockIdx.x * kTileM, n0 = blockIdx.y * kTileN, kbeg = blockIdx.z * k_per_cta;
+    const int m0 = blockIdx.x * kTileM, n0 = blockIdx.y * kTileN;
+    const int kbeg = ((int)blockIdx.z - (second ? splits : 0)) * k_per_cta;
     const int chunks = k_per_cta / kWgRows;
     // a chunk is two halves of 64 columns, 128-byte swizzled; a warp copies two
     // rows of 128 columns
@@ -290,7 +301,7 @@ mlp_wgrad_kernel(const bf16* __restrict__ A, const bf16* __restrict__ B, int k_p
                           umma_desc_sw128(sa + kWgChunk + s * 2048, kWgChunk / 2, 1024), idesc, c > 0 || s > 0 ? 1u : 0u);
             umma_commit(&done[c % kWgSlots]);
         }
-        // the slot of the chunk before takes the chunk five on once its MMAs are done
+        // the slot of the chunk before takes the next chunk to come once its MMAs are done
         const int next = c + kWgSlots - 1;
         if (next < chunks) {
             if (c > 0 && !mbar_wait(&done[(c - 1) % kWgSlots], ((c - 1) / kWgSlots) & 1, kWaitPolls)) ok = false;
@@ -1053,44 +1064,6 @@ __global__ void __launch_bounds__(256) out_train_kernel(const bf16* __restrict__
     }
 }
 
-// Fixed-order reductions of per-block partial sums: out[i] (+)= sum over k
-// of part[k * stride + i], i < len (accumulate: add to out instead of
-// storing).  Long outputs take a thread per output, which sums k in order;
-// short outputs with many partials a warp per output, lane l summing
-// partials l, l + 32, ... in order before a fixed shuffle tree combines the
-// lanes.  Two such reductions run in one launch: blocks [0, a.blocks) take
-// segment a, the rest segment b (b.blocks = 0: none).
-struct RedSeg {
-    const float* part;
-    int n_part, stride, len;
-    float* out;
-    int accumulate;
-    int warp;     // 1: a warp per output (8 per block), 0: a thread per output
-    int blocks;
-};
-
-__global__ void sum_segments_kernel(RedSeg a, RedSeg b)
-{
-    const bool first = (int)blockIdx.x < a.blocks;
-    const RedSeg& r = first ? a : b;
-    const int blk = first ? (int)blockIdx.x : (int)blockIdx.x - a.blocks;
-    if (r.warp) {
-        const int i = (int)((blk * (size_t)blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
-        if (i >= r.len) return;
-        float acc = 0.0f;
-        for (int k = lane; k < r.n_part; k += 32) acc += r.part[(size_t)k * r.stride + i];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-        if (lane == 0) r.out[i] = r.accumulate ? r.out[i] + acc : acc;
-    } else {
-        const int i = blk * blockDim.x + threadIdx.x;
-        if (i >= r.len) return;
-        float acc = 0.0f;
-        for (int k = 0; k < r.n_part; ++k) acc += r.part[(size_t)k * r.stride + i];
-        r.out[i] = r.accumulate ? r.out[i] + acc : acc;
-    }
-}
-
 // Per-feature reductions over a chunk of samples (thread = feature), for
 // batches below kManyRows rows (larger ones are summed per tile in the
 // persistent backward GEMM's epilogue), in
@@ -1136,49 +1109,116 @@ __global__ void feat_reduce_kernel(const bf16* __restrict__ dz, const float* __r
     pb[kH * X + o] = b;
 }
 
-// Adam on the FP32 master parameters, writing the BF16 copies of W2, W3 and
-// their transposes used by the tensor-core GEMMs as it goes.
-// The step count t (1 for the first step) comes from device memory; the
-// bias corrections are 1 - beta^t.  advance > 0 (a replayed training step):
-// the last block to finish moves the step on -- the next step's first
-// sample start += advance and t += 1 -- once every block has read t and the
-// step size; *arrive counts the finished blocks and is back at 0 afterwards.
-__global__ void adam_kernel(float* __restrict__ P, const float* __restrict__ G, float* __restrict__ m,
-                            float* __restrict__ v, int n, float lr, float b1, float b2, float eps,
-                            TrainState* __restrict__ ts, bf16* __restrict__ W2, bf16* __restrict__ W3,
-                            bf16* __restrict__ W2T, bf16* __restrict__ W3T, unsigned* __restrict__ arrive,
-                            int advance)
+// Adam (Kingma and Ba) on the FP32 master parameters, writing the BF16 copies of
+// W2, W3 and their transposes used by the tensor-core GEMMs as it goes.  The
+// step count t (1 for the first step) comes from device memory; the bias
+// corrections are 1 - beta^t.
+struct AdamArgs {
+    float *P, *m, *v;
+    float lr, b1, b2, eps;
+    TrainState* ts;
+    bf16 *W2, *W3, *W2T, *W3T;
+    unsigned* arrive;
+    int advance;
+};
+
+__device__ __forceinline__ void adam_update(const AdamArgs& a, int i, float g)
+{
+    const float tf = (float)a.ts->t;
+    const float lr = a.ts->lr > 0.0f ? a.ts->lr : a.lr;
+    const float bc1 = 1.0f - powf(a.b1, tf), bc2 = 1.0f - powf(a.b2, tf);
+    // rounded explicitly: the update is compiled into two kernels
+    const float mi = fmaf(1.0f - a.b1, g, __fmul_rn(a.b1, a.m[i]));
+    const float vi = fmaf(__fmul_rn(1.0f - a.b2, g), g, __fmul_rn(a.b2, a.v[i]));
+    a.m[i] = mi;
+    a.v[i] = vi;
+    const float p = a.P[i] - lr * (mi / bc1) / (sqrtf(vi / bc2) + a.eps);
+    a.P[i] = p;
+    const bool w2 = i >= kOffW2 && i < kOffW2 + kH * kH, w3 = i >= kOffW3 && i < kOffW3 + kH * kH;
+    if (w2 || w3) {
+        const int e = i - (w2 ? kOffW2 : kOffW3), o = e / kH, c = e % kH;
+        (w2 ? a.W2 : a.W3)[e] = __float2bfloat16(p);
+        (w2 ? a.W2T : a.W3T)[c * kH + o] = __float2bfloat16(p);
+    }
+}
+
+// A replayed training step: the last block to finish moves the step on -- the
+// next step's first sample start += advance and t += 1 -- once every block has
+// read t and the step size; *arrive counts the finished blocks and is back at 0
+// afterwards.  Every thread of the block calls it.
+__device__ __forceinline__ void adam_advance(const AdamArgs& a)
+{
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        if (atomicAdd(a.arrive, 1u) == gridDim.x - 1) {
+            a.ts->start += a.advance;
+            a.ts->t += 1;
+            *a.arrive = 0u;
+        }
+    }
+}
+
+__global__ void adam_kernel(const __grid_constant__ AdamArgs a, const float* __restrict__ G, int n)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) {
-        const float tf = (float)ts->t;
-        if (ts->lr > 0.0f) lr = ts->lr;
-        const float bc1 = 1.0f - powf(b1, tf), bc2 = 1.0f - powf(b2, tf);
-        const float g = G[i];
-        const float mi = b1 * m[i] + (1.0f - b1) * g;
-        const float vi = b2 * v[i] + (1.0f - b2) * g * g;
-        m[i] = mi;
-        v[i] = vi;
-        const float p = P[i] - lr * (mi / bc1) / (sqrtf(vi / bc2) + eps);
-        P[i] = p;
-        const bool w2 = i >= kOffW2 && i < kOffW2 + kH * kH, w3 = i >= kOffW3 && i < kOffW3 + kH * kH;
-        if (w2 || w3) {
-            const int e = i - (w2 ? kOffW2 : kOffW3), o = e / kH, c = e % kH;
-            (w2 ? W2 : W3)[e] = __float2bfloat16(p);
-            (w2 ? W2T : W3T)[c * kH + o] = __float2bfloat16(p);
+    if (i < n) adam_update(a, i, G[i]);
+}
+
+// Fixed-order reductions of per-block partial sums: the gradient of parameter
+// at + i, i < len, is the sum over k of part[k * stride + i] (at < 0: the loss,
+// which is added to *loss).  Long segments take a thread per output, which sums
+// k in order; short ones with many partials a warp per output, lane l summing
+// partials l, l + 32, ... in order before a fixed shuffle tree combines the
+// lanes.  All of a step's reductions run in one launch, each segment in blocks
+// of its own, and ADAM applies the gradients as they come (otherwise they go to
+// G): in three launches of their own and Adam after them the sums took 12.3 us
+// and Adam 6.1, all of it here 9.2.
+struct RedSeg {
+    const float* part;
+    int n_part, stride, len, at;
+    int end;      // blocks of this segment and the ones before it
+};
+constexpr int kRedSegs = 6, kRedLong = 8192;   // longer segments: a thread per output
+
+struct RedSegs {
+    RedSeg s[kRedSegs];
+};
+
+template <bool ADAM>
+__global__ void __launch_bounds__(256)
+reduce_kernel(const __grid_constant__ RedSegs segs, const __grid_constant__ AdamArgs a, float* __restrict__ G,
+              float* __restrict__ loss)
+{
+    int q = 0;
+#pragma unroll
+    for (int k = 0; k < kRedSegs - 1; ++k) q += (int)blockIdx.x >= segs.s[k].end;
+    const RedSeg r = segs.s[q];
+    const int blk = (int)blockIdx.x - (q > 0 ? segs.s[q - 1].end : 0);
+    auto put = [&](int i, float g) {
+        if (r.at < 0) *loss += g;
+        else if (ADAM) adam_update(a, r.at + i, g);
+        else G[r.at + i] = g;
+    };
+    if (r.len > kRedLong) {
+        const int i = blk * 256 + threadIdx.x;
+        if (i < r.len) {
+            float acc = 0.0f;
+#pragma unroll 8
+            for (int k = 0; k < r.n_part; ++k) acc += r.part[(size_t)k * r.stride + i];
+            put(i, acc);
+        }
+    } else {
+        const int i = (blk * 256 + (int)threadIdx.x) >> 5, lane = threadIdx.x & 31;
+        if (i < r.len) {
+            float acc = 0.0f;
+            for (int k = lane; k < r.n_part; k += 32) acc += r.part[(size_t)k * r.stride + i];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+            if (lane == 0) put(i, acc);
         }
     }
-    if (advance > 0) {
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            __threadfence();
-            if (atomicAdd(arrive, 1u) == gridDim.x - 1) {
-                ts->start += advance;
-                ts->t += 1;
-                *arrive = 0u;
-            }
-        }
-    }
+    if (ADAM) adam_advance(a);
 }
 
 // Sets the Adam step count (eager steps outside a replayed graph).
@@ -1230,8 +1270,10 @@ struct dp_mlp {
     unsigned char* Wsteps = nullptr;   // hidden weights as the inference kernel's K steps
     float* coord = nullptr;            // normalised node coordinates per dimension (4 x kCoordMax)
     float* loss = nullptr;
-    float* part = nullptr;             // partial sums of the backward pass (kPartFloats)
-    float* red = nullptr;              // per-row-tile sums of the fused backward GEMMs (cap / 128 x 5 x 256)
+    // partial sums of the backward pass: the weight gradients' splits (W3, then
+    // W2), the output layer's blocks, and the bias and first-layer gradients'
+    // row tiles or blocks (1 and 5 x 256 floats each)
+    float *part = nullptr, *out_part = nullptr, *red1 = nullptr, *red5 = nullptr;
     unsigned* arrive = nullptr;        // blocks of the Adam kernel that have finished (0 between launches)
     int* err = nullptr;
     float* h_loss = nullptr;           // pinned
@@ -1251,7 +1293,8 @@ void free_mlp(dp_mlp* m)
     cudaSetDevice(m->device);
     if (m->st) cudaStreamSynchronize(m->st);
     void* ps[] = {m->P, m->G, m->Am, m->Av, m->W2b, m->W3b, m->W2T, m->W3T, m->x, m->t, m->z1, m->z2, m->z3, m->y,
-                  m->h1, m->h2, m->h3, m->dz1, m->dz2, m->dz3, m->states, m->Wsteps, m->coord, m->loss, m->part, m->red, m->arrive, m->err};
+                  m->h1, m->h2, m->h3, m->dz1, m->dz2, m->dz3, m->states, m->Wsteps, m->coord, m->loss, m->part,
+                  m->out_part, m->red1, m->red5, m->arrive, m->err};
     for (void* p : ps)
         if (p) cudaFree(p);
     if (m->h_loss) cudaFreeHost(m->h_loss);
@@ -1298,14 +1341,11 @@ cudaError_t raise_smem_limit(K kernel, int bytes, std::atomic<bool> (&done)[kMax
 // Batches from this size on run the persistent GEMMs.
 constexpr int kManyRows = 16384;
 
-// Partial sums of the backward pass (one buffer, reused by each reduction in
-// turn): split-K tiles of a weight gradient, the output layer's per-block
-// sums, and below kManyRows rows the feature reductions' per-block sums (the
-// persistent backward GEMMs write their per-tile sums to dp_mlp::red
-// instead).  Split-K 32 for the weight gradients (fewer splits serialise the
-// K loop of each CTA, more write more partial tiles).
+// Most splits of the weight gradients (fewer serialise the K loop of each CTA,
+// more write more partial tiles), blocks of the output layer, and blocks of the
+// feature reductions below kManyRows rows (the persistent backward GEMMs sum
+// per row tile instead).
 constexpr int kSplitMax = 32, kOutBlocks = 1024, kRedBlocks = 256;
-constexpr size_t kPartFloats = (size_t)kSplitMax * kH * kH;   // >= kOutBlocks * kOutPart, kRedBlocks * 5 * kH
 
 // The persistent kernel over rows (a multiple of 128, at least kManyRows) with
 // K = 256; RED > 0 (backward): the per-tile sums into red.
@@ -1338,14 +1378,15 @@ cudaError_t gemm(dp_mlp* m, const bf16* A, int lda, const bf16* B, int ldb, int 
     return cudaGetLastError();
 }
 
-// dz^T h of `rows` rows (a multiple of 256) as `splits` partial tiles in m->part
-cudaError_t weight_gradient(dp_mlp* m, const bf16* dz, const bf16* h, int rows, int splits)
+// dW3 and dW2 over `rows` rows (a multiple of 256) as `splits` partial tiles each in m->part
+cudaError_t weight_gradients(dp_mlp* m, int rows, int splits)
 {
     static std::atomic<bool> attr[kMaxDevices];
     cudaError_t e = raise_smem_limit(mlp_wgrad_kernel, kWgSmem, attr);
     if (e != cudaSuccess) return e;
-    mlp_wgrad_kernel<<<dim3(kH / kTileM, kH / kTileN, splits), kWgThreads, kWgSmem, m->st>>>(dz, h, rows / splits, m->part,
-                                                                                          m->err, m->wait_polls);
+    const WgPair p{{m->dz3, m->dz2}, {m->h2, m->h1}};
+    mlp_wgrad_kernel<<<dim3(kH / kTileM, kH / kTileN, 2 * splits), kWgThreads, kWgSmem, m->st>>>(p, splits, rows / splits, m->part,
+                                                                                              m->err, m->wait_polls);
     return cudaGetLastError();
 }
 
@@ -1387,93 +1428,82 @@ int infer(dp_mlp* m, int count, const Geo<double>& g, const InferGrid& ig)
     return DP_OK;
 }
 
+// Adam (beta1 0.9, beta2 0.999, eps 1e-8) with the step count in m->ts
+AdamArgs adam_args(dp_mlp* m, double lr, int advance)
+{
+    return AdamArgs{m->P, m->Am, m->Av, (float)lr, 0.9f, 0.999f, 1e-8f, m->ts, m->W2b, m->W3b, m->W2T, m->W3T, m->arrive,
+                    advance};
+}
+
 // Gradients of the mean squared error over a batch of `count` rows (count a
-// multiple of 512; m->x / m->t hold the batch, or gv gives it) into m->G, the loss sum added
-// to m->loss.  The output layer and its backward pass run in one kernel.
-int forward_backward(dp_mlp* m, int count, float inv_n, const GridView* gv = nullptr)
+// multiple of 512; m->x / m->t hold the batch, or gv gives it), the loss sum
+// added to m->loss.  The output layer and its backward pass run in one kernel.
+// The gradients go to m->G, or with adam straight into a step of it.
+int forward_backward(dp_mlp* m, int count, float inv_n, const GridView* gv = nullptr, const AdamArgs* adam = nullptr)
 {
     const int rows = count;
     int rc;
     if ((rc = forward_hidden(m, rows, gv))) return rc;
     // every gradient sum goes through per-block partial sums and a reduction
     // in a fixed order, so that a training run is reproducible bit for bit
-    auto seg = [](const float* part, int n_part, int stride, int len, float* out, int accumulate) {
-        RedSeg r{part, n_part, stride, len, out, accumulate, len <= 8192 ? 1 : 0, 0};   // short: a warp each
-        r.blocks = r.warp ? (len + 7) / 8 : (len + 255) / 256;
-        return r;
-    };
-    auto reduce2 = [&](const RedSeg& a, const RedSeg& b) {   // both in one launch
-        sum_segments_kernel<<<a.blocks + b.blocks, 256, 0, m->st>>>(a, b);
-        return cudaGetLastError();
-    };
-    auto reduce = [&](const float* part, int n_part, int stride, int len, float* out, int accumulate) {
-        return reduce2(seg(part, n_part, stride, len, out, accumulate), RedSeg{});
-    };
     const int ob = (int)std::min<long long>(std::min<long long>((count + 7) / 8, 2LL * m->sm_count), kOutBlocks);
-    out_train_kernel<<<ob, 256, 0, m->st>>>(m->h3, m->P, m->t, m->z3, count, inv_n, m->dz3, m->part);
+    out_train_kernel<<<ob, 256, 0, m->st>>>(m->h3, m->P, m->t, m->z3, count, inv_n, m->dz3, m->out_part);
     MCK(cudaGetLastError());
-    MCK(reduce2(seg(m->part, ob, kOutPart, 4 * kH + 3, m->G + kOffB3, 0),      // db3, dW4, db4
-                seg(m->part + 4 * kH + 3, ob, kOutPart, 1, m->loss, 1)));       // the loss sum, accumulated
-    // split-K of the weight-gradient GEMMs: a divisor of rows / 256, at most kSplitMax
-    int ks = std::min(rows / kKC, kSplitMax);
-    while ((rows / kKC) % ks) --ks;
+    int nb;   // partial sums of the bias and first-layer gradients
     if (rows >= kManyRows) {
         // persistent backward GEMMs with the bias and first-layer gradients
-        // summed per row tile in their epilogues (dz1 is never stored)
-        const int tiles = rows / kTileM;
-        // layer 3: dz2 = (dz3 W3) * GELU'(z2) with db2; dW3 = dz3^T h2
+        // summed per row tile in their epilogues (dz1 is never stored):
+        // layer 3, dz2 = (dz3 W3) * GELU'(z2) with db2; layer 2,
+        // dz1 = (dz2 W2) * GELU'(z1) summed into dW1 = dz1^T x and db1
+        nb = rows / kTileM;
         MCK((persistent<kEpiBwd, 1>(m, m->dz3, kH, m->W3T, kH, rows, nullptr, nullptr, m->z2, m->dz2, nullptr,
-                                    m->red)));
-        MCK(weight_gradient(m, m->dz3, m->h2, rows, ks));
-        MCK(reduce2(seg(m->part, ks, kH * kH, kH * kH, m->G + kOffW3, 0), seg(m->red, tiles, kH, kH, m->G + kOffB2, 0)));
-        // layer 2: dz1 = (dz2 W2) * GELU'(z1) summed into dW1 = dz1^T x and
-        // db1; dW2 = dz2^T h1
+                                    m->red1)));
         MCK((persistent<kEpiBwd, 5>(m, m->dz2, kH, m->W2T, kH, rows, nullptr, nullptr, m->z1, nullptr, m->x,
-                                    m->red)));
-        MCK(weight_gradient(m, m->dz2, m->h1, rows, ks));
-        MCK(reduce2(seg(m->part, ks, kH * kH, kH * kH, m->G + kOffW2, 0),
-                    seg(m->red, tiles, 5 * kH, 5 * kH, m->G + kOffW1, 0)));
-        return DP_OK;
+                                    m->red5)));
+    } else {
+        // the same with dz1 stored, db2 = sum dz2 and dW1, db1 in passes of
+        // their own of at most kRedBlocks blocks
+        const int chunk = std::max(64, (rows + kRedBlocks - 1) / kRedBlocks);
+        nb = (rows + chunk - 1) / chunk;
+        MCK(gemm<kEpiBwd>(m, m->dz3, kH, m->W3T, kH, rows, nullptr, nullptr, m->z2, m->dz2));
+        MCK(gemm<kEpiBwd>(m, m->dz2, kH, m->W2T, kH, rows, nullptr, nullptr, m->z1, m->dz1));
+        feat_reduce_kernel<0><<<nb, 256, 0, m->st>>>(m->dz2, nullptr, rows, chunk, m->red1);
+        MCK(cudaGetLastError());
+        feat_reduce_kernel<4><<<nb, 256, 0, m->st>>>(m->dz1, m->x, rows, chunk, m->red5);
+        MCK(cudaGetLastError());
     }
-    // rows per block of the feature reductions: at most kRedBlocks blocks
-    const int chunk = std::max(64, (rows + kRedBlocks - 1) / kRedBlocks);
-    const int nb = (rows + chunk - 1) / chunk;
-    // layer 3: dz2 = (dz3 W3) * GELU'(z2); dW3 = dz3^T h2
-    MCK(gemm<kEpiBwd>(m, m->dz3, kH, m->W3T, kH, rows, nullptr, nullptr, m->z2, m->dz2));
-    MCK(weight_gradient(m, m->dz3, m->h2, rows, ks));
-    MCK(reduce(m->part, ks, kH * kH, kH * kH, m->G + kOffW3, 0));
-    // layer 2: dz1 = (dz2 W2) * GELU'(z1); dW2 = dz2^T h1; db2 = sum dz2
-    MCK(gemm<kEpiBwd>(m, m->dz2, kH, m->W2T, kH, rows, nullptr, nullptr, m->z1, m->dz1));
-    MCK(weight_gradient(m, m->dz2, m->h1, rows, ks));
-    MCK(reduce(m->part, ks, kH * kH, kH * kH, m->G + kOffW2, 0));
-    feat_reduce_kernel<0><<<nb, 256, 0, m->st>>>(m->dz2, nullptr, rows, chunk, m->part);
-    MCK(cudaGetLastError());
-    MCK(reduce(m->part, nb, kH, kH, m->G + kOffB2, 0));
-    // layer 1: dW1 = dz1^T x, db1 = sum dz1 (contiguous in G)
-    feat_reduce_kernel<4><<<nb, 256, 0, m->st>>>(m->dz1, m->x, rows, chunk, m->part);
-    MCK(cudaGetLastError());
-    MCK(reduce(m->part, nb, kH * 4 + kH, kH * 4 + kH, m->G + kOffW1, 0));
-    return DP_OK;
-}
-
-// Adam (beta1 0.9, beta2 0.999, eps 1e-8) with the gradient in m->G and the
-// step count in m->ts, then the BF16 copies of the weights.
-int adam_launch(dp_mlp* m, double lr, int advance = 0)
-{
-    adam_kernel<<<(kParams + 255) / 256, 256, 0, m->st>>>(m->P, m->G, m->Am, m->Av, kParams, (float)lr, 0.9f, 0.999f,
-                                                          1e-8f, m->ts, m->W2b, m->W3b, m->W2T, m->W3T, m->arrive,
-                                                          advance);
+    // dW3 = dz3^T h2 and dW2 = dz2^T h1; splits: a divisor of rows / 256
+    int ks = std::min(rows / kKC, kSplitMax);
+    while ((rows / kKC) % ks) --ks;
+    MCK(weight_gradients(m, rows, ks));
+    RedSegs r{};
+    int blocks = 0, q = 0;
+    auto seg = [&](const float* part, int n_part, int stride, int len, int at) {
+        blocks += len > kRedLong ? (len + 255) / 256 : (len + 7) / 8;
+        r.s[q++] = RedSeg{part, n_part, stride, len, at, blocks};
+    };
+    seg(m->part, ks, kH * kH, kH * kH, kOffW3);
+    seg(m->part + (size_t)ks * kH * kH, ks, kH * kH, kH * kH, kOffW2);
+    seg(m->out_part, ob, kOutPart, 4 * kH + 3, kOffB3);          // db3, dW4, db4
+    seg(m->red1, nb, kH, kH, kOffB2);
+    seg(m->red5, nb, 5 * kH, 5 * kH, kOffW1);                    // dW1, db1
+    seg(m->out_part + 4 * kH + 3, ob, kOutPart, 1, -1);          // the loss
+    if (adam) reduce_kernel<true><<<blocks, 256, 0, m->st>>>(r, *adam, nullptr, m->loss);
+    else reduce_kernel<false><<<blocks, 256, 0, m->st>>>(r, AdamArgs(), m->G, m->loss);
     MCK(cudaGetLastError());
     return DP_OK;
 }
 
-// One Adam step with the gradient in m->G (the next step count).
+// One Adam step with the gradient in m->G (the next step count), then the BF16
+// copies of the weights.
 int adam_step(dp_mlp* m, double lr)
 {
     ++m->step;
     set_step_kernel<<<1, 1, 0, m->st>>>(m->ts, (int)m->step);
     MCK(cudaGetLastError());
-    return adam_launch(m, lr);
+    adam_kernel<<<(kParams + 255) / 256, 256, 0, m->st>>>(adam_args(m, lr, 0), m->G, kParams);
+    MCK(cudaGetLastError());
+    return DP_OK;
 }
 
 int check_err(dp_mlp* m)
@@ -1501,14 +1531,13 @@ namespace {
 // step's start and count.  Replayable: no argument changes between steps.
 int train_step(dp_mlp* m, const GridView& gv, int B, double lr)
 {
-    int rc;
-    if ((rc = forward_backward(m, B, 1.0f / (3.0f * B), &gv))) return rc;
-    return adam_launch(m, lr, B);   // with the next step's start and count
+    const AdamArgs adam = adam_args(m, lr, B);   // with the next step's start and count
+    return forward_backward(m, B, 1.0f / (3.0f * B), &gv, &adam);
 }
 
 // The epochs of dp_mlp_train_grid.  The first step runs as launched (it also
 // sets the kernels' attributes); the next one is captured as a CUDA graph
-// and every later step replays it, which removes the host's 12 launches
+// and every later step replays it, which removes the host's launches
 // per step.
 int train_grid_steps(dp_mlp* m, const GridView& gv, const dp_mlp_train_opts* o, dp_mlp_train_stats* stats)
 {
@@ -1625,8 +1654,10 @@ int dp_mlp_create(const double* lo, const double* hi, int32_t batch_capacity, vo
     A(&m->x, C * 4); A(&m->t, C * 3); A(&m->y, C * 3);
     A(&m->z1, CH); A(&m->z2, CH); A(&m->z3, CH);
     A(&m->h1, CH); A(&m->h2, CH); A(&m->h3, CH); A(&m->dz1, CH); A(&m->dz2, CH); A(&m->dz3, CH);
-    A(&m->states, C * 4); A(&m->Wsteps, 2 * kInferSteps * kInferStep); A(&m->coord, 4 * kCoordMax); A(&m->loss, 1); A(&m->err, 1); A(&m->part, kPartFloats);
-    A(&m->red, C / kTileM * 5 * kH); A(&m->arrive, 1);
+    A(&m->states, C * 4); A(&m->Wsteps, 2 * kInferSteps * kInferStep); A(&m->coord, 4 * kCoordMax); A(&m->loss, 1); A(&m->err, 1);
+    const size_t R = std::max<size_t>(C / kTileM, kRedBlocks) * kH;
+    A(&m->part, 2 * (size_t)kSplitMax * kH * kH); A(&m->out_part, (size_t)kOutBlocks * kOutPart); A(&m->red1, R); A(&m->red5, 5 * R);
+    A(&m->arrive, 1);
     A(&m->ts, 1);
     if (e == cudaSuccess) e = cudaMallocHost(&m->h_loss, sizeof(float));
     if (e == cudaSuccess) e = cudaMallocHost(&m->h_err, sizeof(int));
