@@ -48,6 +48,13 @@ __constant__ int kFib[kMaxFib] = {0, 1, 1, 2, 3, 5, 8, 13, 21, 34, 55, 89, 144, 
                                   1597, 2584, 4181, 6765, 10946, 17711, 28657, 46368, 75025,
                                   121393, 196418, 317811, 514229};
 
+// A kernel launched by launch_after() (dp_host.h) may start while the one before
+// it in the stream finishes: it lets its own successor do the same, and touches
+// no memory that an earlier kernel writes or reads before the wait returns,
+// which is when those have completed.
+__device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 template <typename G> struct V2;
 template <> struct V2<float>  { typedef float2 type; };
 template <> struct V2<double> { typedef double2 type; };

@@ -235,6 +235,8 @@ __global__ void __launch_bounds__(kGmBlock)
 gm_start_kernel(const VV* __restrict__ Vin, const VV* __restrict__ Vnext, VT* __restrict__ q0, int n,
                 double* __restrict__ partial, GmCtl* __restrict__ gc)
 {
+    let_next_start();
+    wait_for_previous();
     __shared__ BlockSums S;
     __shared__ double red[kGmLd];
     Acc<VT> nrm;
@@ -283,6 +285,8 @@ gm_matvec_kernel(const __grid_constant__ Geo<G> g, VT* __restrict__ Q, long long
                  const uint16_t* __restrict__ code, const unsigned long long* __restrict__ feet_lo,
                  const unsigned* __restrict__ feet_hi, const Feet64 f64, const GmCtl* __restrict__ gc)
 {
+    let_next_start();
+    wait_for_previous();
     if (*(const volatile int*)&gc->done) return;
     const VT* x = Q + (size_t)k * ldq;
     VT* w = Q + (size_t)(k + 1) * ldq;
@@ -435,6 +439,8 @@ __global__ void __launch_bounds__(kGmBlock, sizeof(VT) == 4 ? kGmStreamBlocks : 
 gm_dots_kernel(const VT* __restrict__ Q, long long ldq, int n, int k, double* __restrict__ partial,
                GmCtl* __restrict__ gc)
 {
+    let_next_start();
+    wait_for_previous();
     if (*(volatile int*)&gc->done) return;
     __shared__ BlockSums S;
     __shared__ double red[kGmLd];
@@ -501,6 +507,8 @@ __global__ void __launch_bounds__(kGmBlock, sizeof(VT) == 4 ? kGmStreamBlocks : 
 gm_update_kernel(VT* __restrict__ Q, long long ldq, int n, int k, int m, double rtol, double* __restrict__ partial,
                  GmCtl* __restrict__ gc)
 {
+    let_next_start();
+    wait_for_previous();
     if (*(volatile int*)&gc->done) return;
     // the sums of the norm, then the last block's copy of R
     __shared__ union { BlockSums S; double R[kGmMaxRestart * kGmMaxRestart]; } U;
@@ -541,6 +549,8 @@ __global__ void __launch_bounds__(kGmBlock)
 gm_apply_kernel(const VV* __restrict__ Vin, VV* __restrict__ Vnext, const VT* __restrict__ Q, long long ldq, int n,
                 const GmCtl* __restrict__ gc, Ctl* __restrict__ ctl)
 {
+    let_next_start();
+    wait_for_previous();
     __shared__ VT s_coef[kGmMaxRestart + kGmCols];
     const int kk = gc->k;
     for (int i = threadIdx.x; i < kk + kGmCols; i += kGmBlock) s_coef[i] = i < kk ? (VT)gc->coef[i] : (VT)0;
@@ -622,8 +632,7 @@ cudaError_t launch_arnoldi(const GmArgs<G, VT>& a, int k)
     const long long need = ((long long)a.g.n_nodes + kGmBlock - 1) / kGmBlock;
     const long long cap = (long long)per_sm * a.sm_count;
     const int b = (int)(need < cap ? (need < 1 ? 1 : need) : cap);
-    kern<<<b, kGmBlock, 0, a.stream>>>(a.g, a.Q, a.ldq, k, a.code, a.feet_lo, a.feet_hi, a.f64, a.gctl);
-    return cudaGetLastError();
+    return launch_after(kern, b, kGmBlock, 0, a.stream, a.g, a.Q, a.ldq, k, a.code, a.feet_lo, a.feet_hi, a.f64, a.gctl);
 }
 
 template <bool SECOND, typename G, typename VT>
@@ -632,8 +641,7 @@ cudaError_t launch_dots(const GmArgs<G, VT>& a, int n, int k)
     auto kern = gm_dots_kernel<VT, SECOND>;
     static int per_sm = 0;
     const int b = stream_blocks(kern, n, a.sm_count, a.max_blocks, per_sm);
-    kern<<<b, kGmBlock, 0, a.stream>>>(a.Q, a.ldq, n, k, a.partial, a.gctl);
-    return cudaGetLastError();
+    return launch_after(kern, b, kGmBlock, 0, a.stream, a.Q, a.ldq, n, k, a.partial, a.gctl);
 }
 
 template <bool NORM, typename G, typename VT>
@@ -642,8 +650,7 @@ cudaError_t launch_update(const GmArgs<G, VT>& a, int n, int k)
     auto kern = gm_update_kernel<VT, NORM>;
     static int per_sm = 0;
     const int b = stream_blocks(kern, n, a.sm_count, a.max_blocks, per_sm);
-    kern<<<b, kGmBlock, 0, a.stream>>>(a.Q, a.ldq, n, k, a.m, a.rtol, a.partial, a.gctl);
-    return cudaGetLastError();
+    return launch_after(kern, b, kGmBlock, 0, a.stream, a.Q, a.ldq, n, k, a.m, a.rtol, a.partial, a.gctl);
 }
 
 cudaError_t dispatch_arnoldi(const GmArgs<float, float>& a, int k)
@@ -678,8 +685,8 @@ cudaError_t cycle(const GmArgs<G, VT>& a, const VV* Vin, VV* Vnext)
         auto kern = gm_start_kernel<VV, VT>;
         static int per_sm = 0;
         const int b = stream_blocks(kern, n, a.sm_count, a.max_blocks, per_sm);
-        kern<<<b, kGmBlock, 0, a.stream>>>(Vin, Vnext, a.Q, n, a.partial, a.gctl);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        e = launch_after(kern, b, kGmBlock, 0, a.stream, Vin, Vnext, a.Q, n, a.partial, a.gctl);
+        if (e != cudaSuccess) return e;
     }
     for (int k = 0; k < a.m; ++k) {
         if ((e = dispatch_arnoldi(a, k)) != cudaSuccess) return e;
@@ -691,8 +698,7 @@ cudaError_t cycle(const GmArgs<G, VT>& a, const VV* Vin, VV* Vnext)
     auto kern = gm_apply_kernel<VV, VT>;
     static int per_sm = 0;
     const int b = stream_blocks(kern, n, a.sm_count, a.max_blocks, per_sm);
-    kern<<<b, kGmBlock, 0, a.stream>>>(Vin, Vnext, a.Q, a.ldq, n, a.gctl, a.ctl);
-    return cudaGetLastError();
+    return launch_after(kern, b, kGmBlock, 0, a.stream, Vin, Vnext, a.Q, a.ldq, n, a.gctl, a.ctl);
 }
 
 }  // namespace

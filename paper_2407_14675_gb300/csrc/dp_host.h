@@ -194,4 +194,26 @@ constexpr double kFoot8Zone = 16.0;
 cudaError_t launch_feet(const Geo<float>& g, const uint16_t* code, unsigned long long* feet_lo, unsigned* feet_hi,
                         int dyn, int reduced, int sm_count, cudaStream_t st);
 
+// Launches a kernel that begins with let_next_start() and wait_for_previous()
+// so that its blocks may be resident before the kernel ahead of it in the stream
+// has finished: a sweep of a small grid is a few microseconds, of which the start
+// of a launch is one or two (coarse-to-fine solve of 61^4, 3,600 launches: 112.5
+// ms, 102.6 so).  In replayed graphs (the batch, the network's training) it gave
+// nothing, and they launch plainly.
+template <typename... P, typename... A>
+cudaError_t launch_after(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, A... args)
+{
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t c = {};
+    c.gridDim = grid;
+    c.blockDim = block;
+    c.dynamicSmemBytes = smem;
+    c.stream = stream;
+    c.attrs = attr;
+    c.numAttrs = 1;
+    return cudaLaunchKernelEx(&c, kernel, P(args)...);
+}
+
 }  // namespace dpk

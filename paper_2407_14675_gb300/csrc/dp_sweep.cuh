@@ -743,6 +743,8 @@ sweep_kernel(const __grid_constant__ Geo<G> g, const S* __restrict__ Vin, S* __r
              int check_prev, double tol, const Feet64 f64, int feet8)
 {
     constexpr bool kSearch = MODE == kVI || MODE == kVIDiag || MODE == kImproveFull || MODE == kImproveWalk;
+    let_next_start();
+    wait_for_previous();
     if (*(volatile int*)&ctl->stop) return;
     if (check_prev) {
         unsigned long long bits = *(volatile unsigned long long*)&ring[(sweep - 1) & ring_mask];
@@ -809,10 +811,8 @@ cudaError_t launch_sized(const SweepLaunch<G, S>& L)
     // FP64 searches: as many blocks as nodes need, handed out as SMs come free
     int blocks = (int)(need < cap || search64_blocks<G, S, MODE>() ? need : cap);
     if (blocks < 1) blocks = 1;
-    kern<<<blocks, B, smem, L.stream>>>(L.g, L.Vin, L.Vout, L.code, L.feet_lo, L.feet_hi, L.inc, L.acc, L.V64,
-                                      L.incr_flags, L.ctl, L.ring, L.ring_mask, L.sweep, L.check_prev, L.tol, L.f64,
-                                      L.feet8);
-    return cudaGetLastError();
+    return launch_after(kern, blocks, B, smem, L.stream, L.g, L.Vin, L.Vout, L.code, L.feet_lo, L.feet_hi, L.inc, L.acc,
+                        L.V64, L.incr_flags, L.ctl, L.ring, L.ring_mask, L.sweep, L.check_prev, L.tol, L.f64, L.feet8);
 }
 
 template <typename G, typename S, int MODE, bool REDUCED, int DYN>
