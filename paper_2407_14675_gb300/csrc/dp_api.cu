@@ -1709,7 +1709,7 @@ int dp_warm_start_from_grid(const dp_grid* src, dp_grid* dst, double* ms_out)
     CK(cudaEventRecord(e0, dst->st));
     cudaError_t e = launch_prolong(src->g64, Vs, src64 ? 0 : 1, src->code, src->d.reduced,
                                    src->d.dynamics == DP_DYN_POLAR, dst->g64, dst->V[dst->cur], dst->fp32, dst->code,
-                                   dst->M, dst->st);
+                                   dst->M, dst->sm_count, dst->st);
     if (e == cudaSuccess) e = cudaEventRecord(e1, dst->st);
     if (e == cudaSuccess) e = cudaEventSynchronize(e1);
     float ms = 0.0f;

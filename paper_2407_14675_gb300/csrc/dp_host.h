@@ -131,7 +131,7 @@ cudaError_t launch_widen(const float* src, double* dst, int n, cudaStream_t st);
 cudaError_t launch_box_index(const Geo<double>& g, long long* out, cudaStream_t st);
 cudaError_t launch_prolong(const Geo<double>& gs, const void* Vs, int src_fp32, const uint16_t* Cs, int src_reduced,
                            int periodic, const Geo<double>& gd, void* Vd, int fp32_dst, uint16_t* Cd, double Md,
-                           cudaStream_t st);
+                           int sm_count, cudaStream_t st);
 
 // Policy evaluation by restarted GMRES (§3: with the control frozen, Eq. (13)
 // is the sparse linear system (I - beta W_f) V = b).  One cycle starts from
