@@ -563,6 +563,20 @@ __device__ __forceinline__ float ld_coherent(const float* p)
 // FP32 values and blend: the same differences, two per paired instruction,
 // written straight into the pairs (x, x + 4) of Corners<float>: row rb and
 // row rb + 2 of the same v_t corner.  COH: coherent loads (ld_coherent).
+__device__ __forceinline__ void set_corners_f32(const float v00[4], const float v01[4], const float v10[4],
+                                                const float v11[4], float vj, Corners<float>& K)
+{
+    const unsigned long long jj = pack2(vj, vj);
+#pragma unroll
+    for (int rb = 0; rb < 2; ++rb) {
+        const unsigned long long lo0 = pack2(v00[rb], v00[rb + 2]), lo1 = pack2(v10[rb], v10[rb + 2]);
+        K.q0[2 * rb] = sub2(lo0, jj);
+        K.qd[2 * rb] = sub2(pack2(v01[rb], v01[rb + 2]), lo0);
+        K.q0[2 * rb + 1] = sub2(lo1, jj);
+        K.qd[2 * rb + 1] = sub2(pack2(v11[rb], v11[rb + 2]), lo1);
+    }
+}
+
 template <bool COH>
 __device__ __forceinline__ void load_rows_f32(const float* __restrict__ V, const int base[4], int n_m, float vj,
                                               Corners<float>& K, int up = 1)
@@ -583,14 +597,20 @@ __device__ __forceinline__ void load_rows_f32(const float* __restrict__ V, const
             v11[rb] = __ldg(p + n_m + up);
         }
     }
-    const unsigned long long jj = pack2(vj, vj);
-#pragma unroll
-    for (int rb = 0; rb < 2; ++rb) {
-        const unsigned long long lo0 = pack2(v00[rb], v00[rb + 2]), lo1 = pack2(v10[rb], v10[rb + 2]);
-        K.q0[2 * rb] = sub2(lo0, jj);
-        K.qd[2 * rb] = sub2(pack2(v01[rb], v01[rb + 2]), lo0);
-        K.q0[2 * rb + 1] = sub2(lo1, jj);
-        K.qd[2 * rb + 1] = sub2(pack2(v11[rb], v11[rb + 2]), lo1);
+    set_corners_f32(v00, v01, v10, v11, vj, K);
+}
+
+// p + k.  SMALL (an array below 4 GB): by a 32-bit byte offset, which a load
+// adds to a base that all lanes share by itself, instead of a 64-bit address
+// formed in every lane.
+template <bool SMALL, typename T>
+__device__ __forceinline__ T* at_node(T* p, int k)
+{
+    if constexpr (SMALL) {
+        typedef typename std::conditional<std::is_const<T>::value, const char, char>::type C;
+        return reinterpret_cast<T*>(reinterpret_cast<C*>(p) + (unsigned)k * (unsigned)sizeof(T));
+    } else {
+        return p + k;
     }
 }
 

@@ -175,11 +175,29 @@ __device__ __forceinline__ int foot_kind(unsigned long long w) { return foot8_ki
 
 // Blend at a frozen foot of kind kFootInside: D = I[V] - vj.  W: the word
 // pair (FootWord) or the 8-byte word.
-template <bool REDUCED, typename W>
+template <bool REDUCED, bool SMALL = false, typename W>
 __device__ __forceinline__ float eval_foot(const Geo<float>& g, const float* __restrict__ V, int j, W w, float vj)
 {
     const FootCell f = foot_cell_of(g, w);
     int base[4];
+    if constexpr (SMALL) {
+        // the corner rows' distances are the grid's: they belong to the base
+        foot_rows<REDUCED>(g, j, f.dr, f.dv, f.dt, base);
+        float v00[4], v01[4], v10[4], v11[4];
+        Corners<float> K;
+#pragma unroll
+        for (int rb = 0; rb < 4; ++rb) {
+            const float* V0 = V;
+            if constexpr (!REDUCED) V0 += (rb >> 1) * (long long)g.stride[0] + (rb & 1) * (long long)g.stride[1];
+            const float *p = at_node<true>(V0, base[REDUCED ? rb : 0]), *q = at_node<true>(V0 + g.n_m, base[REDUCED ? rb : 0]);
+            v00[rb] = __ldg(p);
+            v01[rb] = __ldg(p + 1);
+            v10[rb] = __ldg(q);
+            v11[rb] = __ldg(q + 1);
+        }
+        set_corners_f32(v00, v01, v10, v11, vj, K);
+        return K.blend(f.t);
+    }
     foot_rows<REDUCED>(g, j, f.dr, f.dv, f.dt, base);
     Corners<float> K;
     load_rows<float, float>(V, base, g.n_m, vj, K);
@@ -264,7 +282,7 @@ __device__ __forceinline__ int cell_reach(const Geo<float>& g, int j, const int 
 // Sweeps nodes j0, j0 + stride, ... < end of one grid: the per-node work of
 // every sweep mode.  Folds max |V_out - V_in| into resid and non-finite
 // results into bad.
-template <typename G, typename S, int MODE, bool REDUCED, int DYN, bool PREFETCH = true>
+template <typename G, typename S, int MODE, bool REDUCED, int DYN, bool PREFETCH = true, bool SMALL = false>
 __device__ __forceinline__ void sweep_nodes(const Geo<G>& g, const Table<G>& T, const S* __restrict__ Vin,
                                             S* __restrict__ Vout, uint16_t* __restrict__ code,
                                             unsigned long long* __restrict__ feet_lo,
@@ -367,8 +385,8 @@ __device__ __forceinline__ void sweep_nodes(const Geo<G>& g, const Table<G>& T, 
         constexpr bool kF8 = MODE == kEvalFeet8;
         typedef typename std::conditional<kF8, unsigned long long, FootWord>::type FW;
         auto load_foot = [&](int k) -> FW {
-            if constexpr (kF8) return __ldcs(&feet_lo[k]);
-            else return FootWord{__ldcs(&feet_lo[k]), __ldcs(&feet_hi[k])};
+            if constexpr (kF8) return __ldcs(at_node<SMALL>(feet_lo, k));
+            else return FootWord{__ldcs(at_node<SMALL>(feet_lo, k)), __ldcs(at_node<SMALL>(feet_hi, k))};
         };
         const bool first = incr_flags & 1, last = incr_flags & 2;
         int j = j0;
@@ -376,7 +394,7 @@ __device__ __forceinline__ void sweep_nodes(const Geo<G>& g, const Table<G>& T, 
         S v_next = (S)0;
         if (kPrefetch && j < end) {
             w_next = load_foot(j);
-            v_next = Vin[j];
+            v_next = *at_node<SMALL>(Vin, j);
         }
         for (; j < end; j += stride) {
             FW w;
@@ -386,11 +404,11 @@ __device__ __forceinline__ void sweep_nodes(const Geo<G>& g, const Table<G>& T, 
                 vj = v_next;
                 if (j + stride < end) {
                     w_next = load_foot(j + stride);
-                    v_next = Vin[j + stride];
+                    v_next = *at_node<SMALL>(Vin, j + stride);
                 }
             } else {
                 w = load_foot(j);
-                vj = Vin[j];
+                vj = *at_node<SMALL>(Vin, j);
             }
             const int kind = foot_kind(w);
             S vnew = (S)0;
@@ -398,7 +416,7 @@ __device__ __forceinline__ void sweep_nodes(const Geo<G>& g, const Table<G>& T, 
                 float ws = 0.0f;
                 if (kind == kFootInside) {
                     if constexpr (kDiag) ws = foot_self_weight(g, w);
-                    vnew = bellman_value<G, S>(g, vj, eval_foot<REDUCED>(g, Vin, j, w, vj));
+                    vnew = bellman_value<G, S>(g, vj, eval_foot<REDUCED, SMALL>(g, Vin, j, w, vj));
                 } else if (kind == kFootOut) {
                     vnew = bellman_value<G, S>(g, vj, (G)((S)g.M64 - vj));
                 } else if (kind == kFootRecompute) {
@@ -409,7 +427,7 @@ __device__ __forceinline__ void sweep_nodes(const Geo<G>& g, const Table<G>& T, 
                 if constexpr (kDiag) {
                     if (kind != kFootTarget) vnew = diag_step(g, vj, vnew, ws);
                 }
-                Vout[j] = vnew;
+                *at_node<SMALL>(Vout, j) = vnew;
                 resid = fmax(resid, (S)fabs(vnew - vj));
             } else {
                 // increment: d' = beta W d at the frozen policy (no running cost,
@@ -419,7 +437,7 @@ __device__ __forceinline__ void sweep_nodes(const Geo<G>& g, const Table<G>& T, 
                 // off-diagonal weights only, d' = beta (W d - w_jj d_j) / (1 - beta w_jj)
                 float D = 0.0f, ws = 0.0f;
                 if (kind == kFootInside) {
-                    D = eval_foot<REDUCED>(g, Vin, j, w, 0.0f);
+                    D = eval_foot<REDUCED, SMALL>(g, Vin, j, w, 0.0f);
                     if constexpr (kDiag) ws = foot_self_weight(g, w);
                 } else if (kind == kFootRecompute) {
                     D = incr_recompute<REDUCED, DYN>(g, Vin, j, code[j], kDiag ? &ws : nullptr);
@@ -430,10 +448,10 @@ __device__ __forceinline__ void sweep_nodes(const Geo<G>& g, const Table<G>& T, 
                 } else {
                     vnew = fmaf(g.beta_hi, D, g.beta_lo * D);
                 }
-                Vout[j] = vnew;
-                const float sum = (first ? 0.0f : acc[j]) + vnew;
-                if (last) V64[j] += (double)sum;
-                else acc[j] = sum;
+                *at_node<SMALL>(Vout, j) = vnew;
+                const float sum = (first ? 0.0f : *at_node<SMALL>(acc, j)) + vnew;
+                if (last) *at_node<SMALL>(V64, j) += (double)sum;
+                else *at_node<SMALL>(acc, j) = sum;
                 resid = fmax(resid, (S)fabs(vnew));
             }
             bad = bad || !isfinite(vnew);
@@ -734,7 +752,7 @@ constexpr int min_blocks()
                                                                          : 1;
 }
 
-template <typename G, typename S, int MODE, bool REDUCED, int DYN, bool BIG>
+template <typename G, typename S, int MODE, bool REDUCED, int DYN, bool BIG, bool SMALL>
 __global__ void __launch_bounds__(sweep_block<G, S, MODE, REDUCED, BIG>(), min_blocks<G, S, MODE, REDUCED, BIG>())
 sweep_kernel(const __grid_constant__ Geo<G> g, const S* __restrict__ Vin, S* __restrict__ Vout,
              uint16_t* __restrict__ code, unsigned long long* __restrict__ feet_lo, unsigned* __restrict__ feet_hi,
@@ -780,7 +798,7 @@ sweep_kernel(const __grid_constant__ Geo<G> g, const S* __restrict__ Vin, S* __r
     const int j0 = blockIdx.x * B + threadIdx.x, end = g.n_nodes, stride = gridDim.x * B;
     constexpr bool kReach = std::is_same<G, float>::value && (MODE == kImproveFull || MODE == kImproveWalk);
     int reach = 0;
-    sweep_nodes<G, S, MODE, REDUCED, DYN, eval_prefetch<MODE, REDUCED>()>(
+    sweep_nodes<G, S, MODE, REDUCED, DYN, eval_prefetch<MODE, REDUCED>(), SMALL>(
         g, T, Vin, Vout, code, feet_lo, feet_hi, inc, acc, V64, incr_flags, j0, end, stride, resid, bad, f64,
         kReach ? &reach : nullptr, feet8 != 0);
     if constexpr (kReach) {
@@ -791,10 +809,10 @@ sweep_kernel(const __grid_constant__ Geo<G> g, const S* __restrict__ Vin, S* __r
     block_fold<S, B>(resid, bad, &ring[sweep & ring_mask], &ctl->nonfinite);
 }
 
-template <typename G, typename S, int MODE, bool REDUCED, int DYN, bool BIG>
+template <typename G, typename S, int MODE, bool REDUCED, int DYN, bool BIG, bool SMALL>
 cudaError_t launch_sized(const SweepLaunch<G, S>& L)
 {
-    auto kern = sweep_kernel<G, S, MODE, REDUCED, DYN, BIG>;
+    auto kern = sweep_kernel<G, S, MODE, REDUCED, DYN, BIG, SMALL>;
     constexpr int B = sweep_block<G, S, MODE, REDUCED, BIG>();
     constexpr bool kSearch = MODE == kVI || MODE == kVIDiag || MODE == kImproveFull || MODE == kImproveWalk;
     const size_t smem = kSearch ? (size_t)L.g.K * (sizeof(typename V2<G>::type) + (search64_blocks<G, S, MODE>() ? 8 : 0)) +
@@ -815,16 +833,34 @@ cudaError_t launch_sized(const SweepLaunch<G, S>& L)
                         L.V64, L.incr_flags, L.ctl, L.ring, L.ring_mask, L.sweep, L.check_prev, L.tol, L.f64, L.feet8);
 }
 
-template <typename G, typename S, int MODE, bool REDUCED, int DYN>
-cudaError_t launch_one(const SweepLaunch<G, S>& L)
+template <typename G, typename S, int MODE, bool REDUCED, int DYN, bool SMALL>
+cudaError_t launch_blocks(const SweepLaunch<G, S>& L)
 {
     constexpr int Bbig = big_block<MODE, REDUCED>();
     if constexpr (Bbig != kBlock) {
         // large blocks only where every SM gets one
         if ((long long)L.g.n_nodes >= (long long)Bbig * L.sm_count)
-            return launch_sized<G, S, MODE, REDUCED, DYN, true>(L);
+            return launch_sized<G, S, MODE, REDUCED, DYN, true, SMALL>(L);
     }
-    return launch_sized<G, S, MODE, REDUCED, DYN, false>(L);
+    return launch_sized<G, S, MODE, REDUCED, DYN, false, SMALL>(L);
+}
+
+template <typename G, typename S, int MODE, bool REDUCED, int DYN>
+cudaError_t launch_one(const SweepLaunch<G, S>& L)
+{
+    // Sweeps at FP32 frozen feet: 32-bit byte offsets where the 8-byte arrays
+    // stay below 4 GB.  On reduced grids the four corner rows have no common
+    // distance, and eight 64-bit addresses per node cost more than eight 32-bit
+    // offsets to two bases: 121^4 band, plain 0.312 -> 0.302 ms a sweep,
+    // diagonal-solved 0.357 -> 0.343.  On the full box the plain sweep gains
+    // (61^4 66.2 -> 65.5 us), the forms bounded to fewer registers lose
+    // (diagonal-solved 83.0 -> 85.0 us, the increments spill).
+    constexpr bool kOffsets = MODE == kEvalFeet8 || (REDUCED && (MODE == kEvalFeet || MODE == kIncr ||
+                                                                 MODE == kEvalFeetDiag || MODE == kIncrDiag));
+    if constexpr (kOffsets) {
+        if (L.g.n_nodes < (1 << 29)) return launch_blocks<G, S, MODE, REDUCED, DYN, true>(L);
+    }
+    return launch_blocks<G, S, MODE, REDUCED, DYN, false>(L);
 }
 
 template <typename G, typename S, int DYN, bool REDUCED>
