@@ -745,6 +745,7 @@ int run_loop(dp_grid* g, const Geo<G>& geo, const S* V, const double* x0, int n,
     L.x_final = x_final;
     L.dyn = g->d.dynamics;
     L.reduced = g->d.reduced;
+    L.sm_count = g->sm_count;
     L.stream = g->st;
     CK(launch_loop(L));
     return DP_OK;

@@ -101,6 +101,7 @@ struct LoopLaunch {
     double* x_final;         // n x 4 (closed loop)
     int dyn;
     int reduced;
+    int sm_count;
     cudaStream_t stream;
 };
 
