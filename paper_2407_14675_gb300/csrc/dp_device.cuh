@@ -1167,7 +1167,10 @@ __device__ __forceinline__ int walk_table(E& ev, const Table<G>& T, int k0, type
 // The bracket is [a, a + f] with f = F[n] and inner points a + F[n-2] and
 // a + F[n-1], whose values are f1 and f2: the state is a, the two values and
 // two Fibonacci numbers, stepped by subtraction (the search is bound by the
-// integer pipe, so the points themselves and table lookups would cost it).
+// integer pipe, so the points themselves and table lookups would cost it).  With
+// both points kept, the numbers looked up by each lane's own index, the angles
+// from the global tables and the cell tested coordinate by coordinate a walk
+// sweep of the 121^4 band took 4.49 ms and of 61^4 1.17, now 3.65 and 1.00.
 template <class E, typename G>
 __device__ __forceinline__ int fibonacci_refine(E& ev, const Table<G>& T, int n0, int fib_stop, int k,
                                                 typename E::R Dk, typename E::R& Dbest)
