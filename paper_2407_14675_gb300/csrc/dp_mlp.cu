@@ -8,9 +8,9 @@
 // The two 256 x 256 layers (98.6 % of the FLOPs) run on the fifth-generation
 // tensor cores: tcgen05.mma kind::f16, BF16 operands staged in shared memory,
 // FP32 accumulators in TMEM, fused epilogues (bias + GELU forward, GELU'
-// backward, split-K atomic accumulation for weight gradients).  The 4-wide
-// input layer, the 3-wide output layer, the reductions and Adam run on the
-// CUDA cores.
+// backward, split-K partial tiles for weight gradients).  The 4-wide input
+// layer, the 3-wide output layer, the reductions and Adam run on the CUDA
+// cores.  Inference over a grid is one kernel for all layers.
 #include <algorithm>
 #include <atomic>
 #include <cmath>
@@ -325,7 +325,8 @@ mlp_wgrad_kernel(const __grid_constant__ WgPair p, int splits, int k_per_cta, fl
             float v[32];
             tmem_ld32(tmem + ((unsigned)((warp & 3) * 32) << 16) + c0 + h, v);
 #pragma unroll
-            for (int q = 0; q < 32; q += 4) *reinterpret_cast<float4*>(dst + h + q) = make_float4(v[q], v[q + 1], v[q + 2], v[q + 3]);
+            for (int q = 0; q < 32; q += 4)
+                *reinterpret_cast<float4*>(dst + h + q) = make_float4(v[q], v[q + 1], v[q + 2], v[q + 3]);
         }
     }
     fence_before_sync();
@@ -333,8 +334,7 @@ mlp_wgrad_kernel(const __grid_constant__ WgPair p, int splits, int k_per_cta, fl
     if (warp == 0) tmem_dealloc(tmem, kTileN);
 }
 
-// GEMM of a large batch (inference over a grid, and the training steps'
-// hidden layers), persistent: each CTA takes one 128-column half of the
+// GEMM of a large batch's hidden layer in a training step, persistent: each CTA takes one 128-column half of the
 // layer (its 128 x 256 slice of the weights stays in shared memory, 64 KB)
 // and walks row tiles blockIdx.x, blockIdx.x + gridDim.x, ...  The next
 // tile's 128 x 256 activations are copied (cp.async) into the second of two

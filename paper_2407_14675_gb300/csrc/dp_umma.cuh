@@ -3,7 +3,8 @@
 // descriptors, the BF16 MMA with FP32 accumulation in TMEM, completion via an
 // mbarrier (bounded wait), and TMEM -> register loads.
 //
-// Operand layout in shared memory: K-major, no swizzle, as 8 x 8 "core
+// Operand layouts in shared memory: the training step's GEMMs use the 128-byte
+// swizzle (umma_desc_sw128()); the inference kernel K-major, no swizzle, 8 x 8 "core
 // matrices" of 16-bit elements (8 rows of 16 bytes, 128 contiguous bytes).
 // For a tile of R rows and KC columns of K, core matrix (row block rb, K block
 // kb) sits at byte ((rb * (KC / 8)) + kb) * 128; the next core matrix along K
