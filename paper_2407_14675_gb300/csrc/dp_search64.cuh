@@ -115,20 +115,30 @@ struct Search64 {
         b0 = (float)nd.b0, b1 = (float)nd.b1, g1 = (float)nd.g1, d1 = (float)nd.d1;
         b2 = (float)nd.b2, g2 = (float)nd.g2, e2 = (float)nd.e2, g3 = kPolar ? (float)nd.g3 : 0.0f;
         const float L[4] = {fabsf(b0), fabsf(b1) + fabsf(g1) + fabsf(d1), fabsf(b2) + fabsf(g2) + fabsf(e2), fabsf(g3)};
-        face = 4e-6f * (1.0f + L[0] + L[1] + L[2] + L[3]);
-        // cell and fractions: the cell from the FP32 displacement, which decides
-        // it wherever the fraction is clear of a face (the displacement's FP32
-        // rounding is part of that margin)
-        bool in = true, in_all = true, box = !ev.outm, far = ev.outm;
+        // How near a face is too near.  The fractions come from the FP32
+        // displacement, off by up to 6e-8 of it (2^-24): 3.1e-5 of a cell at 512
+        // cells.  It enters every angle's fractions through mid[], so it is in
+        // the margin of all of them, not of the first angle alone.  The rest: a
+        // fraction is at most nine FP32 roundings of terms up to L[d] and five
+        // of sums up to 1 + L[d], 6e-8 each.
+        float um = 0.0f;
 #pragma unroll
         for (int d = 0; d < kDims; ++d) {
             uf[d] = (float)u[d];
-            const float fi = floorf(uf[d]), margin = face + 3e-7f * fabsf(uf[d]), r = fmaf(1.001f * reach, L[d], margin);
+            um = fmaxf(um, fabsf(uf[d]));
+        }
+        face = fmaf(3e-7f, um, 4e-6f * (1.0f + L[0] + L[1] + L[2] + L[3]));
+        // cell and fractions: the cell from the FP32 displacement, which decides
+        // it wherever the fraction is clear of a face
+        bool in = true, in_all = true, box = !ev.outm, far = ev.outm;
+#pragma unroll
+        for (int d = 0; d < kDims; ++d) {
+            const float fi = floorf(uf[d]), r = fmaf(1.001f * reach, L[d], face);
             fl[d] = (double)fi;
             t[d] = u[d] - fl[d];
             tf[d] = uf[d] - fi;
             cl[d] = ev.i[d] + (int)fi;
-            in = in && tf[d] > margin && tf[d] < 1.0f - margin;
+            in = in && tf[d] > face && tf[d] < 1.0f - face;
             in_all = in_all && tf[d] > r && tf[d] < 1.0f - r;
             if (d < 3) {
                 box = box && (unsigned)cl[d] <= (unsigned)(g.n[d] - 2);
@@ -209,9 +219,6 @@ struct Search64 {
         acc = h12 * g1 * g2;
         // largest corner difference, from the exponents and leading bits
         const float E0 = top(e, 8);
-        float um = 2.0f;
-#pragma unroll
-        for (int d = 0; d < 3; ++d) um = fmaxf(um, (float)abs(cl[d] - ev.i[d]) + 1.0f);
         const float Hs = fabsf(h01) + fabsf(h02) + fabsf(h12), Ls = L[0] + L[1] + L[2], X = fabsf(d1) + fabsf(e2);
         // below FP32's range the bounds would not hold (a flat value: all ties)
         if (!(E0 * Ls > 1e-20f)) return kSearchOpen;
@@ -219,7 +226,7 @@ struct Search64 {
         // slopes, per radian from theta_0: the H terms' rounding and F, Q parts, the angle coordinate's cross terms
         eh = fmaf(8e-6f * hh, Ls, 6.0f * hh * X) + 16.0f * E3 * L[3] * Ls;
         et = 3.0f * h012 * L[0] * L[1] * L[2];   // and H_012, per radian squared
-        noise = 2.5e-15f * E0 * (um + 3.0f);   // half the rounding of a difference: slopes are at most 2 E0
+        noise = 2.5e-15f * E0 * (um + 5.0f);   // half the rounding of a difference: slopes are at most 2 E0
         eps = fmaf(1e-6f, fabsf(S) + fabsf(C), 4e-6f * (fabsf(F) + fabsf(Q))) + 2.0f * eh + 3.0f * et + 2.0f * noise;
         return kSearchCell;
     }
@@ -231,7 +238,8 @@ struct Search64 {
         const float fq = fmaf(F, fmaf(s, c, -s0 * c0), Q * dc * (c + c0));
         return fmaf(S, ds, fmaf(C, dc, fq)) + fmaf(fmaf(ass, ds, asc * dc), ds, acc * dc * dc);
     }
-    // The foot's fractions keep `by` from the faces (by >= face).
+    // The foot keeps `face` from the cell's faces, and all that is within
+    // `reach` radians of it does.
     __device__ __forceinline__ bool inside(float s, float c, float reach = 0.0f) const
     {
         const float t0 = fmaf(b0, s, mid[0]), t1 = fmaf(b1, s, fmaf(c, fmaf(d1, c, g1), mid[1]));
