@@ -26,10 +26,37 @@
 //   sinc(h) (p cos m - q sin m) + sinc(2 h) (v cos 2m - w sin 2m),
 //   p = S c_k - C s_k, q = S s_k + C c_k (FP64, then rounded),
 //   v = F cos 2 theta_k - Q sin 2 theta_k, w = F sin 2 theta_k + Q cos 2 theta_k.
-// The bounds collect the FP32 rounding of each term, the H terms' F and Q
-// parts and curvature over the interval, the H_012 term, and the rounding of
-// the FP64 evaluations, which at the end of a refinement is what limits it.
 // A point counts only where its fractions are clear of the cell's faces.
+//
+// The bounds, with e = 6e-8 (2^-24) for an FP32 rounding and L_d = |B_d| + |C_d|
+// + |F_d| + 2 |Q_d|, so that L_d times the distance |ds| + |dc| bounds a
+// fraction's change, and X = |F| + 2 |Q| the part of it that is not linear:
+//   f at table angles: S (ds) is S's rounding, the two sines' (e / 2 each, ds
+//     up to 2), the product's and two sums': below 10 e |S|, 1e-6 is 16; F and
+//     Q with three roundings each and differences of products up to 1: below
+//     20 e, 4e-6 is 67;
+//   slopes: p, cos m, the product, k1 and two sums, 8 e |p| (6e-7 is 10); q with
+//     sin m of |m| <= 0.22 and m's own rounding, 12 e |m| |q| (8e-7 is 13); v and
+//     w: F and Q 3 e each, the sine and cosine of 2 theta_k 2.5 e, which with
+//     their own rounding leaves 13 e hypot(v, w), the evaluation 5 e, and sinc(2 h)
+//     cut off after h^4, 64 h^6 / 5040 = 8e-7 of it for h = 0.2 (1.5e-6 is 25);
+//   the H terms: their F and Q parts, sum H (2 L X + X^2) <= 3 Hs Ls X over the
+//     circle (chords up to 2: twice 9 here) and, as a slope per radian, 6 Hs Ls X
+//     of the distance along s and c, which is up to sqrt 2 of the arc (9); their
+//     rounding, ten e of sum H L L (8e-6 Hs Ls), and that of ds and us at a
+//     distance of nothing, 5 e of the form's coefficients (4e-7); the slope's
+//     variation over [m - h, m + h], a third derivative of at most six times
+//     those, h^2 / 6 of it (2 h^2); H_012: 8 L0 L1 L2 of the value (9), 3 L0 L1 L2
+//     times the distance squared of the slope;
+//   noise, the rounding of one FP64 evaluation (2^-53 = 1.1e-16): a displacement
+//     is two roundings of itself and three of L_d, its angle's sine and cosine
+//     3.5e-16 of L_d, a slope in a fraction at most 2 E0, so in three or four
+//     fractions 1.8e-15 E0 um + 1.8e-15 E0 Ls + 0.9e-15 E0, and the blend 15 to 20
+//     roundings of E0 (2.5e-15 E0 (um + 5 + Ls)).  E0 bounds the corners on both
+//     sides of the angle coordinate, which an angle's evaluation blends anew.
+// tests/host/search64_bounds.cpp measures how much of them the errors take: at
+// most 0.97 (the H terms, whose bounds are attained), 0.74 by rounding and the
+// series, 0.15 of the noise.
 //
 // Measured (GB300, with one-round blocks of 64): a value-iteration sweep of
 // 17^4, 16 angles, 50 us, evaluating every angle 166; a walk sweep of a
@@ -51,8 +78,9 @@ struct SlopeModel {
     float ass, asc, acc;                // quadratic form of the H terms, around theta_0
     float e0, e1, e2, noise;            // bound: e0 + e1 am + e2 h^2 + noise / h, am = |m| + h
 
-    // Sign of D(x_k + xb) - D(x_k + xa), x_k the code of theta_k; 0: not decided.
-    __device__ __forceinline__ int order(int xa, int xb) const
+    // Mean slope of D between the codes x_k + xa and x_k + xb, x_k the code of
+    // theta_k, and its bound.
+    __device__ __forceinline__ float mean(int xa, int xb, float& err) const
     {
         const float m = 0.5f * kCodeAngle * (float)(xa + xb), h = 0.5f * kCodeAngle * fabsf((float)(xb - xa));
         const float m2 = m * m, h2 = h * h;
@@ -64,8 +92,14 @@ struct SlopeModel {
         const float k2 = fmaf(h2, fmaf(h2, 16.0f / 120.0f, -4.0f / 6.0f), 1.0f);
         const float as = ds + us, ac = dc + uc;
         const float hq = fmaf(2.0f * ass, as, asc * ac) * (ck + uc) - fmaf(asc, as, 2.0f * acc * ac) * (sk + us);
-        const float mu = fmaf(k1, fmaf(p, cs, -q * sn), fmaf(k2, fmaf(v, c2, -w * s2), hq));
-        const float err = fmaf(fabsf(m) + h, e1, e0) + fmaf(e2, h2, __fdividef(noise, h));
+        err = fmaf(fabsf(m) + h, e1, e0) + fmaf(e2, h2, __fdividef(noise, h));
+        return fmaf(k1, fmaf(p, cs, -q * sn), fmaf(k2, fmaf(v, c2, -w * s2), hq));
+    }
+    // Sign of D(x_k + xb) - D(x_k + xa); 0: not decided.
+    __device__ __forceinline__ int order(int xa, int xb) const
+    {
+        float err;
+        const float mu = mean(xa, xb, err);
         if (!(fabsf(mu) > err)) return 0;
         return (mu > 0.0f) == (xb > xa) ? 1 : -1;
     }
@@ -114,7 +148,7 @@ struct Search64 {
         heun_cells<double, DYN>(g, ev.sp, nd, sd, cd, u);
         b0 = (float)nd.b0, b1 = (float)nd.b1, g1 = (float)nd.g1, d1 = (float)nd.d1;
         b2 = (float)nd.b2, g2 = (float)nd.g2, e2 = (float)nd.e2, g3 = kPolar ? (float)nd.g3 : 0.0f;
-        const float L[4] = {fabsf(b0), fabsf(b1) + fabsf(g1) + fabsf(d1), fabsf(b2) + fabsf(g2) + fabsf(e2), fabsf(g3)};
+        const float L[4] = {fabsf(b0), fabsf(b1) + fabsf(g1) + 2.0f * fabsf(d1), fabsf(b2) + fabsf(g2) + fabsf(e2), fabsf(g3)};
         // How near a face is too near.  The fractions come from the FP32
         // displacement, off by up to 6e-8 of it (2^-24): 3.1e-5 of a cell at 512
         // cells.  It enters every angle's fractions through mid[], so it is in
@@ -217,16 +251,18 @@ struct Search64 {
         ass = h01 * b0 * b1 + h02 * b0 * b2 + h12 * b1 * b2;
         asc = h01 * b0 * g1 + h02 * b0 * g2 + h12 * (b1 * g2 + g1 * b2);
         acc = h12 * g1 * g2;
-        // largest corner difference, from the exponents and leading bits
-        const float E0 = top(e, 8);
-        const float Hs = fabsf(h01) + fabsf(h02) + fabsf(h12), Ls = L[0] + L[1] + L[2], X = fabsf(d1) + fabsf(e2);
+        // largest corner difference, from the exponents and leading bits (the
+        // angle coordinate is blended for every angle: its corners on both sides,
+        // which may cancel at this fraction)
+        const float E0 = top(e, 8) + (kPolar ? top(ev.K.de, 8) : 0.0f);
+        const float Hs = fabsf(h01) + fabsf(h02) + fabsf(h12), Ls = L[0] + L[1] + L[2], X = 2.0f * fabsf(d1) + fabsf(e2);
         // below FP32's range the bounds would not hold (a flat value: all ties)
         if (!(E0 * Ls > 1e-20f)) return kSearchOpen;
         const float hh = Hs * Ls;
         // slopes, per radian from theta_0: the H terms' rounding and F, Q parts, the angle coordinate's cross terms
-        eh = fmaf(8e-6f * hh, Ls, 6.0f * hh * X) + 16.0f * E3 * L[3] * Ls;
+        eh = fmaf(8e-6f * hh, Ls, 9.0f * hh * X) + 16.0f * E3 * L[3] * Ls;
         et = 3.0f * h012 * L[0] * L[1] * L[2];   // and H_012, per radian squared
-        noise = 2.5e-15f * E0 * (um + 5.0f);   // half the rounding of a difference: slopes are at most 2 E0
+        noise = 2.5e-15f * E0 * (um + 5.0f + Ls);   // half the rounding of a difference: slopes are at most 2 E0
         eps = fmaf(1e-6f, fabsf(S) + fabsf(C), 4e-6f * (fabsf(F) + fabsf(Q))) + 2.0f * eh + 3.0f * et + 2.0f * noise;
         return kSearchCell;
     }
@@ -362,33 +398,39 @@ struct Search64 {
         return in;
     }
 
+    // The slopes around table angle k.
+    __device__ __forceinline__ SlopeModel slopes(const Table<double>& T, int k) const
+    {
+        SlopeModel M;
+        const double sd = T.sc[k].x, cd = T.sc[k].y;
+        M.sk = T.scf[k].x;
+        M.ck = T.scf[k].y;
+        M.p = (float)(Sd * cd - Cd * sd);
+        M.q = (float)(Sd * sd + Cd * cd);
+        const float c2 = fmaf(-2.0f * M.sk, M.sk, 1.0f), s2 = 2.0f * M.sk * M.ck;
+        M.v = fmaf(F, c2, -Q * s2);
+        M.w = fmaf(F, s2, Q * c2);
+        M.ds = M.sk - s0;
+        M.dc = M.ck - c0;
+        M.ass = ass; M.asc = asc; M.acc = acc;
+        const float far = fabsf(M.ds) + fabsf(M.dc);   // at least the distance along s and c
+        const float vw = fabsf(M.v) + fabsf(M.w);
+        M.e1 = fmaf(8e-7f, fabsf(M.q), eh) + et * (far + 0.5f) * 3.0f;
+        const float A = fabsf(ass) + fabsf(asc) + fabsf(acc);
+        M.e0 = fmaf(1.5e-6f, vw, fmaf(6e-7f, fabsf(M.p), 4e-7f * A)) + far * fmaf(et, far, eh);
+        M.e2 = 2.0f * A;
+        M.noise = noise;
+        return M;
+    }
+
     // fibonacci_refine() from table angle k, with its result: the chosen code.
     // False where the bracket reaches out of the cell.
     __device__ __forceinline__ bool refine(const Table<double>& T, int n0, int fib_stop, int k, int& code) const
     {
         const int xk = T.code[k];
         const int a0 = (k == 0 ? T.code[T.K - 1] - kCodes : T.code[k - 1]) - xk, hi = T.code[k + 1] - xk, L = hi - a0;
-        SlopeModel M;
-        {
-            const double sd = T.sc[k].x, cd = T.sc[k].y;
-            M.sk = T.scf[k].x;
-            M.ck = T.scf[k].y;
-            if (!inside(M.sk, M.ck, kCodeAngle * (float)max(hi, -a0) * 1.001f)) return false;
-            M.p = (float)(Sd * cd - Cd * sd);
-            M.q = (float)(Sd * sd + Cd * cd);
-            const float c2 = fmaf(-2.0f * M.sk, M.sk, 1.0f), s2 = 2.0f * M.sk * M.ck;
-            M.v = fmaf(F, c2, -Q * s2);
-            M.w = fmaf(F, s2, Q * c2);
-            M.ds = M.sk - s0;
-            M.dc = M.ck - c0;
-            M.ass = ass; M.asc = asc; M.acc = acc;
-            const float far = fabsf(M.ds) + fabsf(M.dc);   // at least the distance along s and c
-            const float vw = fabsf(M.v) + fabsf(M.w);
-            M.e1 = fmaf(8e-7f, fabsf(M.q), eh) + et * (far + 0.5f) * 2.0f;
-            M.e0 = fmaf(6e-7f, vw, 4e-7f * fabsf(M.p)) + far * fmaf(et, far, eh);
-            M.e2 = 2.0f * (fabsf(ass) + fabsf(asc) + fabsf(acc));
-            M.noise = noise;
-        }
+        if (!inside(T.scf[k].x, T.scf[k].y, kCodeAngle * (float)max(hi, -a0) * 1.001f)) return false;
+        const SlopeModel M = slopes(T, k);
         // D(xk + xb) < D(xk + xa) (or <=)
         auto better = [&](int xb, int xa, bool or_equal) {
             const int o = M.order(xa, xb);

@@ -7,6 +7,9 @@ angle within 2e-5 of a cell face, where a rounding decides which cell an angle
 is in, with displacements from a fraction of a cell to the longest that a
 dimension of 1,024 nodes allows (the FP32 displacement is off by 3e-5 of a cell
 there), and the periodic angle and reduced node sets among them.
+
+The bounds that the decisions rest on are measured against extended precision:
+no error may be larger than its bound, whichever term dominates.
 """
 import os
 import shutil
@@ -23,7 +26,7 @@ def compile_host(tmp, name):
     from paper_2407_14675_gb300 import build
     cuda = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(build.nvcc()))), "include")
     exe = str(tmp / name)
-    subprocess.run([shutil.which("g++") or "g++", "-std=c++17", "-O2", "-ffp-contract=off", "-I" + cuda, "-I" + HOST,
+    subprocess.run([shutil.which("g++") or "g++", "-std=gnu++17", "-O2", "-ffp-contract=off", "-I" + cuda, "-I" + HOST,
                     "-I" + CSRC, os.path.join(HOST, name + ".cpp"), "-o", exe], check=True)
     return exe
 
@@ -43,3 +46,17 @@ def test_the_model_decides_as_fp64_does(searches, cells, thrust, angles, kind):
     n, model, wrong = map(int, out.split())
     assert n == count and wrong == 0
     assert model > 0.01 * count    # the model is what was tested
+
+
+@pytest.fixture(scope="module")
+def bounds(tmp_path_factory):
+    return compile_host(tmp_path_factory.mktemp("host"), "search64_bounds")
+
+
+@pytest.mark.parametrize("polar", [0, 1])
+@pytest.mark.parametrize("angles", [16, 30, 64, 1024])
+def test_errors_stay_within_their_bounds(bounds, angles, polar):
+    out = subprocess.run([bounds, "1", "400000", str(angles), str(polar)], check=True, capture_output=True, text=True).stdout
+    slope, value, fraction, fp64, looked = map(float, out.split())
+    assert looked > 300000
+    assert max(slope, value, fraction, fp64) <= 1.0
