@@ -151,8 +151,8 @@ loop_kernel(const __grid_constant__ Geo<G> g, const __grid_constant__ LoopLaunch
     __shared__ int s_code[kMaxAngles + 1];
     __shared__ typename V2<G>::type s_sc[kMaxAngles];
     // per state: the node below it, its offset and coordinates (the decision's
-    // inputs), the polar running cost, the decided code
-    __shared__ int s_i[kLoopWarps][4], s_pick[kLoopWarps];
+    // inputs), whether it still flies, the polar running cost, the decided code
+    __shared__ int s_i[kLoopWarps][4], s_live[kLoopWarps], s_pick[kLoopWarps];
     __shared__ G s_u[kLoopWarps][4], s_x[kLoopWarps][4];
     __shared__ double s_cost[kLoopWarps];
     build_table(g, s_code, s_sc);
@@ -203,6 +203,7 @@ loop_kernel(const __grid_constant__ Geo<G> g, const __grid_constant__ LoopLaunch
             s_i[lane >> 2][dl] = (int)fl;
             s_u[lane >> 2][dl] = (G)(sd - fl);
             s_x[lane >> 2][dl] = (G)yw;
+            if (dl == 0) s_live[lane >> 2] = live;
             if (DYN == kDynPolar) {
                 // running cost over tau, Eq. (11)
                 double y4[4];
@@ -215,8 +216,11 @@ loop_kernel(const __grid_constant__ Geo<G> g, const __grid_constant__ LoopLaunch
         // the states of this step; over once none of the block's flies
         if (!__syncthreads_or(warp == 0 && live)) break;
 
-        // --- feedback at y (Eq. (15)); a state that has arrived decides for nothing ---
-        if (w < a.n) {
+        // --- feedback at y (Eq. (15)); the warp of a state that has arrived waits:
+        // on an FP64 grid its decision would take the pipe from the others' (200
+        // steps of eight states an SM of which one flies on, 17^4: 3.9 ms, 8.9 with
+        // the others deciding to the end) ---
+        if (s_live[warp]) {
             G x[4];
 #pragma unroll
             for (int d = 0; d < 4; ++d) {
