@@ -236,8 +236,10 @@ loop_kernel(const __grid_constant__ Geo<G> g, const __grid_constant__ LoopLaunch
             ev.reset();          // cached corners are differences to the old vj
 
             typedef typename CachedEval<G, S, REDUCED, DYN>::R R;
+            // (a lane without a better angle names its own index: where no angle
+            // compares, as with values that a diverged sweep left NaN, index 0 wins)
             R Db = ginf<R>();
-            int kb = 0x7fffffff;
+            int kb = lane;
             for (int k = lane; k < g.K; k += 32) {
                 R D = ev.at_sc(T.sc[k].x, T.sc[k].y);
                 if (better<R, S>(D, k, Db, kb)) { Db = D; kb = k; }
