@@ -19,6 +19,7 @@
 
 #include "dp.h"
 #include "dp_host.h"
+#include "dp_pinned.h"
 
 using namespace dpk;
 
@@ -118,10 +119,9 @@ struct dp_grid {
     int gm_blocks = 0;
     GmCtl* gm_ctl = nullptr;
     GmTail* h_gm = nullptr;              // pinned, one per cycle of a round
-    // states and results of feedback and closed loop (pinned, read and written
-    // by the kernel in place; grown up to kLoopPinned states)
-    double* h_loop = nullptr;
-    int loop_cap = 0;
+    // states and results of feedback and closed loop (read and written by the
+    // kernel in place; grown up to kLoopPinned states)
+    PinnedDoubles loop;
 
     Geo<double> g64;
     Geo<float> g32;
@@ -158,7 +158,7 @@ void free_grid(dp_grid* g)
     if (g->h_ctl) cudaFreeHost(g->h_ctl);
     if (g->h_ring) cudaFreeHost(g->h_ring);
     if (g->h_gm) cudaFreeHost(g->h_gm);
-    if (g->h_loop) cudaFreeHost(g->h_loop);
+    g->loop.release();
     delete g;
 }
 
@@ -767,29 +767,16 @@ int loop_common(const dp_grid* cg, const double* states, int n, double tau, doub
     // once and writes once over the host link: a call is one launch and one
     // synchronisation.  With a device buffer allocated and freed around the call
     // (the synchronisation hands its pages back) and a copy each way a decision
-    // for 8 states took 194 us, of which the kernel is 11; larger calls keep
-    // that form.
+    // for 8 states took 194 us, of which the kernel is 11; larger calls, and calls
+    // for which the host has no page-locked memory left, keep that form.
     double* d_buf = nullptr;
     const size_t nb = (size_t)n * kLoopDoubles;
-    const bool pinned = n <= kLoopPinned;
-    if (pinned) {
-        static_assert(sizeof(double) == sizeof(*g->h_ring), "ring entries");
-        if (nb <= (size_t)kRing) {
-            d_buf = (double*)g->h_ring;
-        } else {
-            if (n > g->loop_cap) {
-                const int cap = std::min(kLoopPinned, 2 * n);
-                double* p = nullptr;
-                CK(cudaMallocHost((void**)&p, (size_t)cap * kLoopDoubles * sizeof(double)));
-                if (g->h_loop) cudaFreeHost(g->h_loop);   // no call is in flight: each one synchronises
-                g->h_loop = p;
-                g->loop_cap = cap;
-            }
-            d_buf = g->h_loop;
-        }
-        memcpy(d_buf, states, sizeof(double) * 4 * n);
-    } else
-        CK(cudaMallocAsync(&d_buf, nb * sizeof(double), g->st));
+    static_assert(sizeof(double) == sizeof(*g->h_ring), "ring entries");
+    if (nb <= (size_t)kRing) d_buf = (double*)g->h_ring;
+    else if (n <= kLoopPinned) d_buf = g->loop.reserve(nb, (size_t)kLoopPinned * kLoopDoubles);   // no call is in flight: each one synchronises
+    const bool pinned = d_buf != nullptr;
+    if (pinned) memcpy(d_buf, states, sizeof(double) * 4 * n);
+    else CK(cudaMallocAsync(&d_buf, nb * sizeof(double), g->st));
     double* d_x0 = d_buf;
     double* d_a = d_buf + 4 * (size_t)n;
     double* d_q = d_a + n;
