@@ -95,11 +95,12 @@ struct dp_grid {
     bool store_feet8 = true;                // what the next FP32-value improvements store
     int foot_format = DP_FOOT_AUTO;         // dp_set_foot_format
     double2* dyn_tables = nullptr;          // FP64 grids: tables of the one-step map, one allocation:
-    double2 *row_dyn = nullptr, *mass_dyn = nullptr;   //   rows, mass nodes, coordinates, running cost
-    double *coord = nullptr, *run_cost = nullptr;
+    double2 *row_dyn = nullptr, *mass_dyn = nullptr;   //   rows, mass nodes, coordinates
+    double *coord = nullptr, *run_cost = nullptr;      // polar grids: the running cost per node
     Feet64 f64;                             // frozen feet of FP64 grids
     bool feet64_valid = false;
     bool diag64_valid = false;              // f64.r holds the factors of these feet
+    bool diag64_tried = false;              // its memory was asked for since they were stored
     float* acc = nullptr;                   // FP64-value polish: running sum of increments
     int* wave_sync = nullptr;               // FP32 grids: counters of the multi-level evaluation
     Ctl* ctl = nullptr;
@@ -144,6 +145,20 @@ int dalloc(dp_grid* g, T** p, size_t count)
     return DP_OK;
 }
 
+// Device memory that a grid is faster with but can do without: false where
+// there is none, with no error left behind.
+template <typename T>
+bool dalloc_spare(dp_grid* g, T** p, size_t count)
+{
+    if (cudaMalloc((void**)p, count * sizeof(T)) != cudaSuccess) {
+        *p = nullptr;
+        cudaGetLastError();
+        return false;
+    }
+    g->device_bytes += (long long)(count * sizeof(T));
+    return true;
+}
+
 void free_grid(dp_grid* g)
 {
     if (!g) return;
@@ -152,7 +167,7 @@ void free_grid(dp_grid* g)
     void* ps[] = {g->rows, g->row_org, g->lines, g->hi64, g->lo64, g->hi32, g->lo32, g->V[0], g->V[1], g->V64[0],
                   g->V64[1], g->code, g->feet_lo, g->feet_hi, g->acc, g->ctl, g->ring, g->staging,
                   g->scratch64, g->gm_Q, g->gm_partial, g->gm_ctl, g->f64.t,
-                  g->wave_sync, g->dyn_tables};
+                  g->f64.r, g->wave_sync, g->dyn_tables, g->run_cost};
     for (void* p : ps)
         if (p) cudaFree(p);
     if (g->h_ctl) cudaFreeHost(g->h_ctl);
@@ -370,7 +385,7 @@ cudaError_t enqueue_sweep(dp_grid* g, int pmode, long long t, int check_prev, do
         }
         if (store_of(g) == kStoreF64) {
             g->feet64_valid = g->f64.w != nullptr;
-            g->diag64_valid = false;
+            g->diag64_valid = g->diag64_tried = false;
         }
     }
     const int mode = internal_mode(g, pmode);
@@ -380,9 +395,16 @@ cudaError_t enqueue_sweep(dp_grid* g, int pmode, long long t, int check_prev, do
         double* out = (double*)g->V[(g->cur + a + 1) & 1];
         SweepLaunch<double, double> L = sweep_launch<double, double>(g, g->g64, in, out, mode, t, check_prev, tol);
         if (mode == kEvalFeet64Diag) {
-            // the first such sweep of these feet stores their diagonal factors
-            L.incr_flags = g->diag64_valid ? 0 : 1;
-            g->diag64_valid = true;
+            // The first such sweep of these feet stores their diagonal factors,
+            // in memory that the grid's first one allocates (8 bytes a node);
+            // without it every sweep forms them (Example 1 0.32 ms, 0.25 stored).
+            if (!g->f64.r && !g->diag64_tried) {
+                dalloc_spare(g, &g->f64.r, g->n_active);
+                g->diag64_tried = true;
+                L.f64 = g->f64;
+            }
+            L.incr_flags = g->diag64_valid ? 0 : g->f64.r ? 3 : 1;
+            g->diag64_valid = g->f64.r != nullptr;
         }
         return launch_sweep(L);
     }
@@ -1161,12 +1183,11 @@ int dp_grid_create(const dp_grid_desc* desc, dp_grid** out)
         return bail(rc);
     if (!g->fp32) {
         // FP64 frozen feet, one allocation: fractions (32 bytes a node), then
-        // words, constants and diagonal factors
+        // words and constants
         const size_t n = (size_t)g->n_active;
-        if ((rc = dalloc(g, &g->f64.t, n * 7 / 2 + 1))) return bail(rc);
+        if ((rc = dalloc(g, &g->f64.t, 3 * n))) return bail(rc);
         g->f64.w = (unsigned long long*)(g->f64.t + 2 * n);
         g->f64.c = (double*)(g->f64.w + n);
-        g->f64.r = g->f64.c + n;
     }
     if ((rc = dalloc(g, &g->ctl, 1))) return bail(rc);
     if ((rc = dalloc(g, &g->ring, kRing))) return bail(rc);
@@ -1182,14 +1203,16 @@ int dp_grid_create(const dp_grid_desc* desc, dp_grid** out)
     if (!g->fp32 && d.dynamics != DP_DYN_UNIT_SPEED) {
         const bool polar = d.dynamics == DP_DYN_POLAR;
         const size_t nr = 2 * (size_t)g->n_rows, nm = 2 * (size_t)(polar ? 1 : d.n[3]), nc = 2 * (size_t)kCoordStride;
-        if ((rc = dalloc(g, &g->dyn_tables, nr + nm + nc + (polar ? ((size_t)g->n_active + 1) / 2 : 0)))) return bail(rc);
-        g->row_dyn = g->dyn_tables;
-        g->mass_dyn = g->row_dyn + nr;
-        g->coord = (double*)(g->mass_dyn + nm);
-        if (polar) g->run_cost = g->coord + 2 * nc;
-        fill_geo(g, g->g64);
-        if ((e = launch_dyn_tables(g->g64, g->row_dyn, g->mass_dyn, g->coord, g->run_cost, g->st)) != cudaSuccess)
-            return bail(fail(DP_ECUDA, "one-step map tables: %s", cudaGetErrorString(e)));
+        // without memory for them the sweeps compute these parts at the node
+        if (dalloc_spare(g, &g->dyn_tables, nr + nm + nc)) {
+            g->row_dyn = g->dyn_tables;
+            g->mass_dyn = g->row_dyn + nr;
+            g->coord = (double*)(g->mass_dyn + nm);
+            if (polar) dalloc_spare(g, &g->run_cost, g->n_active);
+            fill_geo(g, g->g64);
+            if ((e = launch_dyn_tables(g->g64, g->row_dyn, g->mass_dyn, g->coord, g->run_cost, g->st)) != cudaSuccess)
+                return bail(fail(DP_ECUDA, "one-step map tables: %s", cudaGetErrorString(e)));
+        }
     }
     fill_geo(g, g->g64);
     fill_geo(g, g->g32);

@@ -681,7 +681,8 @@ struct FootWord {
 // Eq. (11), computed in another kernel, to an ulp of the constant.
 // The first diagonal-solved sweep after an improvement also stores the node's
 // factor 1 / (1 - beta w_jj) in r, which the later ones read (8 bytes instead
-// of 16 of the 59 FP64 operations a node took).
+// of 16 of the 59 FP64 operations a node took).  The grid's first such sweep
+// allocates r; without memory for it (NULL) every sweep forms the factors.
 struct Feet64 {
     unsigned long long* w = nullptr;
     double2* t = nullptr;

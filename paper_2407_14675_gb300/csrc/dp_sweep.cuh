@@ -309,7 +309,7 @@ __device__ __forceinline__ void sweep_nodes(const Geo<G>& g, const Table<G>& T, 
         // diagonal factor formed in every sweep and FP64 comparisons.
         constexpr bool kDiag = MODE == kEvalFeet64Diag;
         constexpr bool kPer = DYN == kDynPolar;
-        const bool first = incr_flags & 1;   // diagonal-solved: store the factors
+        const bool first = incr_flags & 1, keep = incr_flags & 2;   // diagonal-solved: form the factors, store them
         constexpr unsigned long long kInf = 0x7ff0000000000000ull;
         unsigned long long rbits = 0;
         // Whole rounds of the grid, then the remaining nodes in equal shares per
@@ -359,7 +359,7 @@ __device__ __forceinline__ void sweep_nodes(const Geo<G>& g, const Table<G>& T, 
                 if constexpr (kDiag) {
                     if (first) {
                         rd = recip_newton(1.0 - g.beta64 * ws);
-                        __stcs(&f64.r[j], rd);
+                        if (keep) __stcs(&f64.r[j], rd);
                     }
                     q = (double)vj + (q - (double)vj) * rd;   // diag_step()
                 }
