@@ -451,18 +451,19 @@ typedef struct dp_batch_stats {
 int dp_batch_create(const dp_grid_desc* descs, int32_t count, void* stream, dp_batch** out);
 int dp_batch_destroy(dp_batch* batch);
 /* Sizes and tuning of a batch; every output pointer is nullable.
- * nodes_target: nodes inside the targets (never updated).  item_eval /
- * item_improve: nodes per work item of the evaluation and improvement
- * launches. */
+ * nodes_target: nodes inside the targets (never updated).  item_improve: nodes
+ * per work item of the improvement launches.  item_eval: as set; evaluation
+ * launches give every block an equal share of the nodes and do not depend on
+ * it. */
 int dp_batch_get_info(const dp_batch* batch, int32_t* count, int64_t* nodes_total, int64_t* nodes_target,
                       int32_t* item_eval, int32_t* item_improve, int64_t* device_bytes);
 /* Sets the work-item sizes (multiples of 256 in [256, 2^20]). */
 int dp_batch_set_items(dp_batch* batch, int32_t item_eval, int32_t item_improve);
-/* Times the candidate work-item sizes (512 .. 32768 nodes) of the evaluation
- * and walk-improvement launches on this batch with CUDA events and keeps the
- * fastest of each (returned through the nullable outputs).  It runs sweeps,
- * so it leaves every transfer at V = 0 and policy code 0: call it before
- * setting a warm start. */
+/* Times the work-item size in use and the candidates (512 .. 32768 nodes) of
+ * the walk-improvement launches on this batch with CUDA events and keeps the
+ * one in use unless another is faster (both item sizes returned through the
+ * nullable outputs).  It runs sweeps, so it leaves every transfer at V = 0 and
+ * policy code 0: call it before setting a warm start. */
 int dp_batch_autotune(dp_batch* batch, int32_t* item_eval, int32_t* item_improve);
 /* Modified policy iteration of every transfer with the options of
  * dp_policy_iterate (tol, max_sweeps = improvement budget per transfer,

@@ -7,9 +7,9 @@
 // persistent launch over all transfers: a block walks a list of work items
 // (a transfer and a run of `item` consecutive nodes), loads that transfer's
 // geometry and angle table into shared memory when the transfer changes, and
-// runs the same per-node code as a single grid's sweep.  Item sizes follow a
-// rule or are picked by timing the candidates on the batch itself
-// (dp_batch_autotune).
+// runs the same per-node code as a single grid's sweep.  Improvement items follow
+// a rule or are picked by timing the candidates on the batch itself
+// (dp_batch_autotune); evaluation launches take equal shares.
 //
 // Modified policy iteration (§3, Eq. (13)/(14), 1 improvement + n_eval
 // evaluation sweeps per outer step) runs per transfer as a small state
@@ -105,7 +105,7 @@ struct BArgs {
     unsigned* feet_hi;
     float* acc;
     int count;
-    int item_eval, item_imp;       // nodes per work item
+    int item_imp;                  // nodes per work item of the improvements
 };
 
 // One of two buffers by a runtime bit, without indexing the parameter array
@@ -125,12 +125,15 @@ __device__ __forceinline__ void load_geo(Geo<float>& dst, const Geo<float>* src)
 }
 
 // A block's share of a list's items, for the launches whose nodes cost the
-// same: equal runs of consecutive items, [lo, hi) of `total`.  run_of() takes
-// the part of it in one transfer, a run of consecutive nodes, off its front.
+// same: equal runs of consecutive items of kShareItem nodes, [lo, hi) of
+// `total`.  run_of() takes the part of it in one transfer, a run of consecutive
+// nodes, off its front.  (Coarser items would only make the shares less equal.)
 // Handed out one by one, items of 8192 nodes left the last round of blocks
 // half empty, and smaller ones paid for each item's start and residual.
 // Evaluation sweeps one by one and by shares: 16 transfers (8.5M nodes) 62.9
 // and 50.7 us, 3 (476,187 nodes) 13.8 and 9.8, 200 (63M) 395 and 333.
+constexpr int kShareItem = kBlock;
+
 struct Share {
     int lo, hi;
     __device__ Share(int total)
@@ -157,13 +160,13 @@ __device__ __forceinline__ int item_transfer(const int* pre, int count, int it)
 }
 
 // t: the transfer of the run before (-1: none yet).
-__device__ __forceinline__ Run run_of(Share& s, const int* pre, int count, int t, int item, const Geo<float>* geo)
+__device__ __forceinline__ Run run_of(Share& s, const int* pre, int count, int t, const Geo<float>* geo)
 {
     if (t < 0) t = item_transfer(pre, count, s.lo);
     else while (__ldg(&pre[t + 1]) <= s.lo) ++t;
     const int p0 = __ldg(&pre[t]), stop = min(s.hi, __ldg(&pre[t + 1]));
-    const long long end = (long long)(stop - p0) * item;
-    const Run r{t, (s.lo - p0) * item, (int)min(end, (long long)__ldg(&geo[t].n_nodes))};
+    const long long end = (long long)(stop - p0) * kShareItem;
+    const Run r{t, (s.lo - p0) * kShareItem, (int)min(end, (long long)__ldg(&geo[t].n_nodes))};
     s.lo = stop;
     return r;
 }
@@ -174,7 +177,7 @@ __global__ void __launch_bounds__(kBlock) batch_widen_kernel(const BArgs a)
     const int* pre = a.prefix + kLWiden * (a.count + 1);
     Share share(pre[a.count]);
     for (int t = -1; share.lo < share.hi;) {
-        const Run r = run_of(share, pre, a.count, t, a.item_eval, a.geo);
+        const Run r = run_of(share, pre, a.count, t, a.geo);
         t = r.t;
         const BState& S = a.st[t];
         const float* src = pick(a.V32, S.cur) + a.off[t];
@@ -256,7 +259,7 @@ __global__ void __launch_bounds__(kBatchEvalBlock, 2) batch_eval_kernel(const BA
     Share share(pre[a.count]);
     const Table<float> T{nullptr, nullptr, 0};
     for (int cur_t = -1; share.lo < share.hi;) {
-        const Run r = run_of(share, pre, a.count, cur_t, a.item_eval, a.geo);
+        const Run r = run_of(share, pre, a.count, cur_t, a.geo);
         const int t = r.t, first = r.first, end = r.end;
         __syncthreads();   // the previous run is done with the geometry
         load_geo(s_g, &a.geo[t]);
@@ -445,7 +448,7 @@ __global__ void __launch_bounds__(kCtlThreads) batch_ctl_kernel(const BArgs a, B
             ctl_update(s, P, a.geo[t].M64, stage);
             a.st[t] = s;
             const int n = a.geo[t].n_nodes;
-            const int ne = (n + a.item_eval - 1) / a.item_eval, ni = (n + a.item_imp - 1) / a.item_imp;
+            const int ne = (n + kShareItem - 1) / kShareItem, ni = (n + a.item_imp - 1) / a.item_imp;
             c[kLWiden] = (s.phase == kPh64 && s.widen) ? ne : 0;
             c[kLImp32Full] = (s.phase == kPh32 && s.full_next) ? ni : 0;
             c[kLImp32Walk] = (s.phase == kPh32 && !s.full_next) ? ni : 0;
@@ -550,11 +553,11 @@ struct dp_batch {
     int* d_bad = nullptr;
     BState* h_st = nullptr;        // pinned mirror of d_st
     BParams* h_par = nullptr;      // pinned
-    int item_eval = kBlock, item_imp = 8192;
+    int item_eval = 8192, item_imp = 8192;   // item_eval: kept for the caller (dp_batch_set_items)
     int blocks_widen = 0, blocks_imp32f = 0, blocks_imp32w = 0, blocks_imp64f = 0, blocks_imp64w = 0;
     int blocks_eval = 0, blocks_eval_nf = 0;
     cudaGraphExec_t exec = nullptr;
-    int graph_n_eval = -1, graph_item_eval = 0, graph_item_imp = 0;
+    int graph_n_eval = -1, graph_item_imp = 0;
     bool graph_diag = false;
     long long graph_launches = 0;
     bool feet_valid = false;
@@ -611,7 +614,6 @@ BArgs args_of(const dp_batch* b)
     a.feet_hi = b->feet_hi;
     a.acc = b->acc;
     a.count = b->count;
-    a.item_eval = b->item_eval;
     a.item_imp = b->item_imp;
     return a;
 }
@@ -680,8 +682,7 @@ cudaError_t enqueue_step(const dp_batch* b, int n_eval, bool diag, long long* la
 
 int ensure_graph(dp_batch* b, int n_eval, bool diag)
 {
-    if (b->exec && b->graph_n_eval == n_eval && b->graph_diag == diag && b->graph_item_eval == b->item_eval &&
-        b->graph_item_imp == b->item_imp)
+    if (b->exec && b->graph_n_eval == n_eval && b->graph_diag == diag && b->graph_item_imp == b->item_imp)
         return DP_OK;
     if (b->exec) {
         cudaGraphExecDestroy(b->exec);
@@ -707,7 +708,6 @@ int ensure_graph(dp_batch* b, int n_eval, bool diag)
     }
     b->graph_n_eval = n_eval;
     b->graph_diag = diag;
-    b->graph_item_eval = b->item_eval;
     b->graph_item_imp = b->item_imp;
     b->graph_launches = launches;
     return DP_OK;
@@ -1030,28 +1030,25 @@ int dp_batch_autotune(dp_batch* b, int32_t* item_eval, int32_t* item_improve)
     if ((rc = set_params(b, nullptr, 1))) return rc;
     // a full improvement from V = 0 gives every node a policy and frozen foot
     if ((rc = manual_sweep(b, DP_SWEEP_IMPROVE_FULL, nullptr))) return rc;
-    double best_e = INFINITY, best_i = INFINITY;
-    int pick_e = b->item_eval, pick_i = b->item_imp;
-    const int keep_e = b->item_eval, keep_i = b->item_imp;
-    for (int cand : kItemCandidates) {
-        b->item_eval = cand;
-        b->item_imp = keep_i;
-        double t_e = 0.0, t_i = 0.0, ms = 0.0;
-        if ((rc = manual_sweep(b, DP_SWEEP_EVAL, nullptr))) return rc;   // warm-up
-        for (int r = 0; r < 3; ++r) {
-            if ((rc = manual_sweep(b, DP_SWEEP_EVAL, &ms))) return rc;
-            t_e += ms;
-        }
-        b->item_eval = keep_e;
+    // the item in use first; another has to be 2 % faster, more than the
+    // launches of one differ by
+    const int keep = b->item_imp;
+    int pick_i = keep;
+    double best = INFINITY;
+    for (int k = -1; k < (int)(sizeof kItemCandidates / sizeof *kItemCandidates); ++k) {
+        const int cand = k < 0 ? keep : kItemCandidates[k];
+        if (k >= 0 && cand == keep) continue;
         b->item_imp = cand;
-        for (int r = 0; r < 2; ++r) {
-            if ((rc = manual_sweep(b, DP_SWEEP_IMPROVE_WALK, &ms))) return rc;
-            t_i += ms;
+        double t = INFINITY, ms = 0.0;
+        if (k < 0 && (rc = manual_sweep(b, DP_SWEEP_IMPROVE_WALK, nullptr))) return rc;   // warm-up
+        for (int r = 0; r < 3; ++r) {
+            if ((rc = manual_sweep(b, DP_SWEEP_IMPROVE_WALK, &ms))) break;
+            t = std::min(t, ms);
         }
-        if (t_e < best_e) { best_e = t_e; pick_e = cand; }
-        if (t_i < best_i) { best_i = t_i; pick_i = cand; }
+        b->item_imp = keep;
+        if (rc) return rc;
+        if (t < 0.98 * best) { best = t; pick_i = cand; }
     }
-    b->item_eval = pick_e;
     b->item_imp = pick_i;
     // back to the cold state: V = 0, policy code 0
     for (int t = 0; t < b->count; ++t) b->h_st[t].cur = 0;
@@ -1060,7 +1057,7 @@ int dp_batch_autotune(dp_batch* b, int32_t* item_eval, int32_t* item_improve)
     BCK(cudaMemsetAsync(b->code, 0, sizeof(uint16_t) * b->total, b->st));
     BCK(cudaStreamSynchronize(b->st));
     b->feet_valid = false;
-    if (item_eval) *item_eval = pick_e;
+    if (item_eval) *item_eval = b->item_eval;
     if (item_improve) *item_improve = pick_i;
     return DP_OK;
 }
