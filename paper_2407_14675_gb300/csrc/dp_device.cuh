@@ -51,7 +51,13 @@ __constant__ int kFib[kMaxFib] = {0, 1, 1, 2, 3, 5, 8, 13, 21, 34, 55, 89, 144, 
 // A kernel launched by launch_after() (dp_host.h) may start while the one before
 // it in the stream finishes: it lets its own successor do the same, and touches
 // no memory that an earlier kernel writes or reads before the wait returns,
-// which is when those have completed.
+// which is when those have completed.  The compiler must not move a load ahead
+// of the wait either.  It may do that with a load it takes for read-only (a
+// `const ... __restrict__` parameter, __ldg), which no barrier orders, unless the
+// load stands behind a branch on something read after the wait: a load that
+// might not run is not run early.  So control data is read through plain or
+// volatile pointers, and kernels that do not begin with a test of it take no
+// read-only pointers to what earlier kernels write.
 __device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 

@@ -232,8 +232,7 @@ __device__ __forceinline__ double apply_a_feet64(const Geo<double>& g, const dou
 // r0 = V_next - V_in into Q_0, and ||r0||.
 template <typename VV, typename VT>
 __global__ void __launch_bounds__(kGmBlock)
-gm_start_kernel(const VV* __restrict__ Vin, const VV* __restrict__ Vnext, VT* __restrict__ q0, int n,
-                double* __restrict__ partial, GmCtl* __restrict__ gc)
+gm_start_kernel(const VV* Vin, const VV* Vnext, VT* q0, int n, double* __restrict__ partial, GmCtl* gc)
 {
     let_next_start();
     wait_for_previous();
@@ -283,7 +282,7 @@ template <typename G, typename VT, bool REDUCED, int DYN>
 __global__ void __launch_bounds__(kGmBlock, matvec_min_blocks<G>())
 gm_matvec_kernel(const __grid_constant__ Geo<G> g, VT* __restrict__ Q, long long ldq, int k,
                  const uint16_t* __restrict__ code, const unsigned long long* __restrict__ feet_lo,
-                 const unsigned* __restrict__ feet_hi, const Feet64 f64, const GmCtl* __restrict__ gc)
+                 const unsigned* __restrict__ feet_hi, const Feet64 f64, GmCtl* gc)
 {
     let_next_start();
     wait_for_previous();
@@ -437,7 +436,7 @@ __device__ __forceinline__ void with_width(int w, F f)
 template <typename VT, bool SECOND>
 __global__ void __launch_bounds__(kGmBlock, sizeof(VT) == 4 ? kGmStreamBlocks : 2)
 gm_dots_kernel(const VT* __restrict__ Q, long long ldq, int n, int k, double* __restrict__ partial,
-               GmCtl* __restrict__ gc)
+               GmCtl* gc)
 {
     let_next_start();
     wait_for_previous();
@@ -505,7 +504,7 @@ __device__ __forceinline__ void combine(const VT* __restrict__ Q, long long ldq,
 template <typename VT, bool NORM>
 __global__ void __launch_bounds__(kGmBlock, sizeof(VT) == 4 ? kGmStreamBlocks : 2)
 gm_update_kernel(VT* __restrict__ Q, long long ldq, int n, int k, int m, double rtol, double* __restrict__ partial,
-                 GmCtl* __restrict__ gc)
+                 GmCtl* gc)
 {
     let_next_start();
     wait_for_previous();
@@ -546,8 +545,7 @@ gm_update_kernel(VT* __restrict__ Q, long long ldq, int n, int k, int m, double 
 // correction is summed in the basis precision and added once to V_in.
 template <typename VV, typename VT>
 __global__ void __launch_bounds__(kGmBlock)
-gm_apply_kernel(const VV* __restrict__ Vin, VV* __restrict__ Vnext, const VT* __restrict__ Q, long long ldq, int n,
-                const GmCtl* __restrict__ gc, Ctl* __restrict__ ctl)
+gm_apply_kernel(const VV* Vin, VV* Vnext, const VT* Q, long long ldq, int n, GmCtl* gc, Ctl* ctl)
 {
     let_next_start();
     wait_for_previous();
