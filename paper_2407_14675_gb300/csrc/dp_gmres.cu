@@ -229,6 +229,37 @@ __device__ __forceinline__ double apply_a_feet64(const Geo<double>& g, const dou
     return xj;   // outside or target: no W row
 }
 
+// A pair of floats ends at FP32's range.  Columns [0, ncol) whose sum over the
+// warp's part of the block's share left it (entries of 1e17 and more; one tile
+// of 128 products at a time went to 1e18) are summed again in FP64: column c is
+// the product of w with vector(c).  Every warp calls it after its sums_put()s.
+template <typename VT, class F>
+__device__ __forceinline__ void sums_repair(BlockSums& S, int ncol, const VT* w, F vector, int first, int last, int n)
+{
+    if constexpr (std::is_same<VT, float>::value) {
+        const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+        __syncwarp();
+        for (int c0 = 0; c0 < ncol; c0 += 32) {
+            unsigned bad = __ballot_sync(0xffffffffu, c0 + lane < ncol && !isfinite(S.acc[warp][min(c0 + lane, ncol - 1)]));
+            for (; bad; bad &= bad - 1) {
+                const int c = c0 + __ffs((int)bad) - 1;
+                const VT* q = vector(c);
+                Acc<double> a;
+#pragma unroll 1
+                for (int e = first + (int)threadIdx.x; e < last; e += kGmBlock) {
+                    VT x[4], y[4];
+                    load4(w, 4 * e, n, x);
+                    load4(q, 4 * e, n, y);
+#pragma unroll
+                    for (int s = 0; s < 4; ++s) a.add((double)x[s] * (double)y[s]);
+                }
+                const double v = a.warp_total();
+                if (lane == 0) S.acc[warp][c] = v;
+            }
+        }
+    }
+}
+
 // r0 = V_next - V_in into Q_0, and ||r0||.
 template <typename VV, typename VT>
 __global__ void __launch_bounds__(kGmBlock)
@@ -258,6 +289,7 @@ gm_start_kernel(const VV* Vin, const VV* Vnext, VT* q0, int n, double* __restric
         nrm.add(d);
     }
     sums_put(S, 0, nrm);
+    sums_repair(S, 1, q0, [&](int) { return q0; }, first, last, n);
     if (!sums_finish(S, 1, partial, gc, red)) return;
     if (threadIdx.x == 0) {
         const double b = sqrt(red[0]);
@@ -469,6 +501,7 @@ gm_dots_kernel(const VT* __restrict__ Q, long long ldq, int n, int k, double* __
             for (int c = 0; c < W; ++c) sums_put(S, i0 + c, acc[c]);
         });
     }
+    sums_repair(S, k + 1, w, [&](int c) { return Q + (size_t)c * ldq; }, first, last, n);
     if (!sums_finish(S, k + 1, partial, gc, red)) return;
     for (int i = threadIdx.x; i <= k; i += kGmBlock) {
         const double h = gc->scale[i] * red[i];
@@ -536,6 +569,7 @@ gm_update_kernel(VT* __restrict__ Q, long long ldq, int n, int k, int m, double 
     });
     if constexpr (NORM) {
         sums_put(U.S, 0, nrm);
+        sums_repair(U.S, 1, w, [&](int) { return w; }, first, last, n);
         if (!sums_finish(U.S, 1, partial, gc, red)) return;
         finalize_column(gc, k, m, rtol, red[0], U.R, sh);
     }
