@@ -139,7 +139,7 @@ __device__ __forceinline__ void mma_rows(unsigned tmem, const unsigned char* sA,
 //   Tile rows start at 128 blockIdx.x, columns at 128 blockIdx.y: every thread
 //   issues its 16-byte asynchronous copies of both operands at once, then one
 //   thread issues the 16 MMAs (K = 16 each) and commits them to an mbarrier.
-//   kEpiFwd:    z = acc + bias -> zout (optional, FP32), h = GELU(z) -> hout (bf16)
+//   kEpiFwd:    z = acc + bias -> zout (FP32), h = GELU(z) -> hout (bf16)
 //   kEpiBwd:    dz = acc * GELU'(zin) -> hout (bf16)
 template <int EPI>
 __global__ void __launch_bounds__(128)
@@ -194,7 +194,7 @@ mlp_gemm_kernel(const bf16* __restrict__ A, int lda, const bf16* __restrict__ B,
                 for (int q = 0; q < 16; q += 4) {
                     const float4 b = *(const float4*)(bias + n0 + c0 + q);
                     z[q] = v[q] + b.x; z[q + 1] = v[q + 1] + b.y; z[q + 2] = v[q + 2] + b.z; z[q + 3] = v[q + 3] + b.w;
-                    if (zout) *(float4*)(zout + off + q) = make_float4(z[q], z[q + 1], z[q + 2], z[q + 3]);
+                    *(float4*)(zout + off + q) = make_float4(z[q], z[q + 1], z[q + 2], z[q + 3]);
                 }
 #pragma unroll
                 for (int q = 0; q < 16; ++q) z[q] = gelu(z[q]);
@@ -340,11 +340,10 @@ mlp_wgrad_kernel(const __grid_constant__ WgPair p, int splits, int k_per_cta, fl
 // tile's 128 x 256 activations are copied (cp.async) into the second of two
 // 64 KB buffers while the MMAs and the epilogue of the current tile run.
 // Same staging layout, MMAs and epilogue arithmetic as mlp_gemm_kernel<EPI>
-// (kEpiFwd with optional zout, or kEpiBwd).
+// (kEpiFwd or kEpiBwd).
 // Thirty-two warps: eight per quarter of the TMEM lanes, each taking 16 of
 // the tile's 128 columns in the epilogue (with 16 warps of 32 columns each,
-// fewer warps hide the activation's latency: about 1 % slower training and 2 %
-// slower inference).
+// fewer warps hide the activation's latency: about 1 % slower training).
 constexpr int kPersistSmem = (kTileN + 2 * kTileM) * kKC * 2;   // 192 KB
 constexpr int kPersistThreads = 1024;
 constexpr int kPersistParts = kPersistThreads / 128;            // column parts per TMEM lane quarter
@@ -457,7 +456,7 @@ mlp_persistent_kernel(const bf16* __restrict__ A, int lda, const bf16* __restric
             if (EPI == kEpiFwd) {
                 const float4 z = make_float4(a.x + sBias[c0 + 4 * cc], a.y + sBias[c0 + 4 * cc + 1],
                                              a.z + sBias[c0 + 4 * cc + 2], a.w + sBias[c0 + 4 * cc + 3]);
-                if (zout) *(float4*)(zout + goff(k)) = z;
+                *(float4*)(zout + goff(k)) = z;
                 y[0] = gelu(z.x); y[1] = gelu(z.y); y[2] = gelu(z.z); y[3] = gelu(z.w);
             } else {
                 y[0] = a.x * gelu_grad(zi[k].x); y[1] = a.y * gelu_grad(zi[k].y);
@@ -555,7 +554,7 @@ mlp_persistent_kernel(const bf16* __restrict__ A, int lda, const bf16* __restric
 // g and g + 8, ... are added).
 //
 // GRID: rows are the stored nodes of a grid, whose normalised coordinates
-// come from the table coord (4 x kCoordMax, per dimension), and the outputs
+// come from the table coord (4 x kCoordStride, per dimension), and the outputs
 // become the node's value M clamp(y_0, 0, 1) (0 on target nodes) and the code
 // of atan2(y_2, y_1); otherwise rows are x (rows x 4) and the outputs go to y
 // (rows x 3).
@@ -563,7 +562,6 @@ constexpr int kInferThreads = 512;
 constexpr int kInferSlots = 4;                                     // ring of weight K steps
 constexpr int kInferStep = kH * 16 * 2;                            // bytes of one: 256 rows x 16 columns
 constexpr int kInferSteps = kH / 16;                               // per layer
-constexpr int kCoordMax = 1024;                                    // largest grid dimension
 constexpr int kInferSmemA = kTileM * kKC * 2, kInferSmemW = kInferSlots * kInferStep;
 constexpr int kInferSmemF = 4 * kH + kH + kH + kH + 3 * kH + 4;    // W1 (by input), b1, b2, b3, W4, b4
 constexpr int kInferSmem = kInferSmemA + kInferSmemW + (kInferSmemF + 9 * kTileM) * 4;
@@ -593,7 +591,7 @@ __global__ void coord_table_kernel(const Geo<double> g, Box4 nlo, Box4 nhi, floa
     if (i >= g.n[d]) return;
     const double lo[4] = {nlo.x, nlo.y, nlo.z, nlo.w}, hi[4] = {nhi.x, nhi.y, nhi.z, nhi.w};
     const double xd = g.lo[d] + (double)i * g.h[d];
-    coord[d * kCoordMax + i] = (float)(2.0 * (xd - lo[d]) / (hi[d] - lo[d]) - 1.0);
+    coord[d * kCoordStride + i] = (float)(2.0 * (xd - lo[d]) / (hi[d] - lo[d]) - 1.0);
 }
 
 // GELU of a pair: gelu() of each, the plain multiplications and the addition
@@ -756,8 +754,8 @@ mlp_infer_kernel(const __grid_constant__ Geo<double> g, const __grid_constant__ 
         if (live) {
             if constexpr (GRID) {
                 decode_node(g, (int)s, id);
-                xs = make_float4(__ldg(ig.coord + id[0]), __ldg(ig.coord + kCoordMax + id[1]),
-                                 __ldg(ig.coord + 2 * kCoordMax + id[2]), __ldg(ig.coord + 3 * kCoordMax + id[3]));
+                xs = make_float4(__ldg(ig.coord + id[0]), __ldg(ig.coord + kCoordStride + id[1]),
+                                 __ldg(ig.coord + 2 * kCoordStride + id[2]), __ldg(ig.coord + 3 * kCoordStride + id[3]));
             } else {
                 xs = *reinterpret_cast<const float4*>(x + 4 * s);
             }
@@ -942,8 +940,8 @@ __global__ void __launch_bounds__(256) first_layer_kernel(const __grid_constant_
             if (w == 0) {
                 int id[4];
                 decode_node(g, (int)j, id);
-                const float4 v = make_float4(__ldg(tg.coord + id[0]), __ldg(tg.coord + kCoordMax + id[1]),
-                                             __ldg(tg.coord + 2 * kCoordMax + id[2]), __ldg(tg.coord + 3 * kCoordMax + id[3]));
+                const float4 v = make_float4(__ldg(tg.coord + id[0]), __ldg(tg.coord + kCoordStride + id[1]),
+                                             __ldg(tg.coord + 2 * kCoordStride + id[2]), __ldg(tg.coord + 3 * kCoordStride + id[3]));
                 sx[i] = v;
                 x[row] = v;
             } else {
@@ -1268,7 +1266,7 @@ struct dp_mlp {
     bf16 *h1 = nullptr, *h2 = nullptr, *h3 = nullptr, *dz1 = nullptr, *dz2 = nullptr, *dz3 = nullptr;
     double* states = nullptr;
     unsigned char* Wsteps = nullptr;   // hidden weights as the inference kernel's K steps
-    float* coord = nullptr;            // normalised node coordinates per dimension (4 x kCoordMax)
+    float* coord = nullptr;            // normalised node coordinates per dimension (4 x kCoordStride)
     float* loss = nullptr;
     // partial sums of the backward pass: the weight gradients' splits (W3, then
     // W2), the output layer's blocks, and the bias and first-layer gradients'
@@ -1571,7 +1569,7 @@ int train_grid_steps(dp_mlp* m, const GridView& gv, const dp_mlp_train_opts* o, 
     if ((e = cudaEventCreate(&e0)) != cudaSuccess || (e = cudaEventCreate(&e1)) != cudaSuccess ||
         (e = cudaEventRecord(e0, m->st)) != cudaSuccess)
         return done(fail_cuda("training events", e));
-    coord_table_kernel<<<4, kCoordMax, 0, m->st>>>(gv.g64, nlo, nhi, m->coord);
+    coord_table_kernel<<<4, kCoordStride, 0, m->st>>>(gv.g64, nlo, nhi, m->coord);
     if ((e = cudaGetLastError()) != cudaSuccess) return done(fail_cuda("coordinate table", e));
     for (int ep = 0; ep < o->epochs; ++ep) {
         unsigned long long mult = (next() % (unsigned long long)n) | 1ull;
@@ -1654,7 +1652,7 @@ int dp_mlp_create(const double* lo, const double* hi, int32_t batch_capacity, vo
     A(&m->x, C * 4); A(&m->t, C * 3); A(&m->y, C * 3);
     A(&m->z1, CH); A(&m->z2, CH); A(&m->z3, CH);
     A(&m->h1, CH); A(&m->h2, CH); A(&m->h3, CH); A(&m->dz1, CH); A(&m->dz2, CH); A(&m->dz3, CH);
-    A(&m->states, C * 4); A(&m->Wsteps, 2 * kInferSteps * kInferStep); A(&m->coord, 4 * kCoordMax); A(&m->loss, 1); A(&m->err, 1);
+    A(&m->states, C * 4); A(&m->Wsteps, 2 * kInferSteps * kInferStep); A(&m->coord, 4 * kCoordStride); A(&m->loss, 1); A(&m->err, 1);
     const size_t R = std::max<size_t>(C / kTileM, kRedBlocks) * kH;
     A(&m->part, 2 * (size_t)kSplitMax * kH * kH); A(&m->out_part, (size_t)kOutBlocks * kOutPart); A(&m->red1, R); A(&m->red5, 5 * R);
     A(&m->arrive, 1);
@@ -1803,7 +1801,7 @@ int dp_warm_start(dp_mlp* m, dp_grid* grid, double* ms_out)
     Geo<double> g = gv.g64;
     const Box4 nlo{m->lo[0], m->lo[1], m->lo[2], m->lo[3]};
     const Box4 nhi{m->hi[0], m->hi[1], m->hi[2], m->hi[3]};
-    coord_table_kernel<<<4, kCoordMax, 0, m->st>>>(g, nlo, nhi, m->coord);
+    coord_table_kernel<<<4, kCoordStride, 0, m->st>>>(g, nlo, nhi, m->coord);
     MCK(cudaGetLastError());
     // the value goes to the storage-precision buffer (an FP32 grid holding
     // FP64 values after a polish returns to its FP32 values)

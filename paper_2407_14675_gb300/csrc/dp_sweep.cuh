@@ -281,7 +281,9 @@ __device__ __forceinline__ int cell_reach(const Geo<float>& g, int j, const int 
 
 // Sweeps nodes j0, j0 + stride, ... < end of one grid: the per-node work of
 // every sweep mode.  Folds max |V_out - V_in| into resid and non-finite
-// results into bad.
+// results into bad.  The modes kEvalFeet64* also deal out the last round by
+// block and thread indices: they are for the whole launch of sweep_kernel only
+// (j0 the thread's index in the grid, stride the grid's threads).
 template <typename G, typename S, int MODE, bool REDUCED, int DYN, bool PREFETCH = true, bool SMALL = false>
 __device__ __forceinline__ void sweep_nodes(const Geo<G>& g, const Table<G>& T, const S* __restrict__ Vin,
                                             S* __restrict__ Vout, uint16_t* __restrict__ code,
