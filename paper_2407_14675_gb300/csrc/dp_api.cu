@@ -302,7 +302,7 @@ void fill_geo(const dp_grid* gr, Geo<G>& g)
     while (F2 < Lmin) { long long F3 = F1 + F2; F1 = F2; F2 = F3; ++n; }
     g.fib_n0 = n;
     g.n_m = d.n[3];
-    g.magic_m = ((1ULL << 40) + (unsigned long long)d.n[3] - 1) / (unsigned long long)d.n[3];
+    line_divisor(d.n[3], g.line_mul, g.line_shift);
     g.n_nodes = (int)gr->n_active;
     g.rows = gr->rows;
     g.row_org = gr->row_org;

@@ -96,7 +96,8 @@ struct Geo {
     int fib_n0;                // Fibonacci index of the shortest refinement bracket
     int tlo[4], thi[4];        // target index box, inclusive (tlo > thi: no target)
     int n_m;
-    unsigned long long magic_m;    // ceil(2^40 / n_m): j / n_m for j < 2^40 / (n_m - 1)
+    unsigned line_mul;         // j / n_m of a node j: the upper 32 bits of j line_mul, shifted right by
+    int line_shift;            //   line_shift (line_divisor())
     int n_nodes;               // stored nodes
     const int4* rows;          // per (i_r, i_vr): {first compact index, lo_vt, len, 0}
     const int* row_org;        // reduced grids, per (i_r, i_vr): first compact index - lo_vt * n_m, the
@@ -176,11 +177,24 @@ __device__ __forceinline__ void code_sincos(const Geo<G>& g, int code, G& s, G& 
     angle_sum<G>(__ldg(&g.tab_hi[code >> 8]), __ldg(&g.tab_lo[code & 255]), s, c);
 }
 
+// Division by the mass nodes' number d (2 .. 1024) for every j < 2^31: with
+// 2^(s-1) < d <= 2^s and mul = ceil(2^(31+s) / d), j / d = j mul >> (31 + s) (mul d
+// exceeds 2^(31+s) by less than d <= 2^s, so j times the excess stays below
+// 2^(31+s); Granlund and Montgomery).  mul fits 32 bits and the product 64, for
+// any number of lines.
+__host__ __device__ inline void line_divisor(int d, unsigned& mul, int& shift)
+{
+    int s = 1;
+    while ((1 << s) < d) ++s;
+    mul = (unsigned)(((1ull << (31 + s)) + (unsigned long long)d - 1) / (unsigned long long)d);
+    shift = s - 1;
+}
+
 // Node decode: compact index -> (i_r, i_vr, i_vt, i_m).
 template <typename G>
 __device__ __forceinline__ void decode_node(const Geo<G>& g, int j, int i[4])
 {
-    unsigned line = (unsigned)(((unsigned long long)(unsigned)j * g.magic_m) >> 40);
+    const unsigned line = __umulhi((unsigned)j, g.line_mul) >> g.line_shift;
     i[3] = j - (int)line * g.n_m;
     unsigned L = __ldg(&g.lines[line]);
     i[0] = (int)(L & 1023u);
