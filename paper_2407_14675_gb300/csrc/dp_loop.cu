@@ -24,6 +24,8 @@
 // warp's state, 0.85 ms with eight states' components in one warp (5,000 of 60
 // steps on 31^4: 2.21 and 1.61 ms; a single one, all latency, 7.9 us a step in
 // either).
+#include <climits>
+
 #include "dp_host.h"
 #include "dp_sweep.cuh"
 
@@ -151,8 +153,10 @@ loop_kernel(const __grid_constant__ Geo<G> g, const __grid_constant__ LoopLaunch
     __shared__ int s_code[kMaxAngles + 1];
     __shared__ typename V2<G>::type s_sc[kMaxAngles];
     // per state: the node below it, its offset and coordinates (the decision's
-    // inputs), whether it still flies, the polar running cost, the decided code
-    __shared__ int s_i[kLoopWarps][4], s_live[kLoopWarps], s_pick[kLoopWarps];
+    // inputs; kArrived in place of the index: none to take), the polar running
+    // cost, the decided code
+    constexpr int kArrived = INT_MIN;
+    __shared__ int s_i[kLoopWarps][4], s_pick[kLoopWarps];
     __shared__ G s_u[kLoopWarps][4], s_x[kLoopWarps][4];
     __shared__ double s_cost[kLoopWarps];
     build_table(g, s_code, s_sc);
@@ -200,10 +204,9 @@ loop_kernel(const __grid_constant__ Geo<G> g, const __grid_constant__ LoopLaunch
             const double sd = (yw - lo_d) / h_d;
             double fl = floor(sd);
             fl = fmin(fmax(fl, -4.0), (double)n_d + 4.0);   // keep the index finite
-            s_i[lane >> 2][dl] = (int)fl;
+            s_i[lane >> 2][dl] = live ? (int)fl : kArrived;
             s_u[lane >> 2][dl] = (G)(sd - fl);
             s_x[lane >> 2][dl] = (G)yw;
-            if (dl == 0) s_live[lane >> 2] = live;
             if (DYN == kDynPolar) {
                 // running cost over tau, Eq. (11)
                 double y4[4];
@@ -220,7 +223,7 @@ loop_kernel(const __grid_constant__ Geo<G> g, const __grid_constant__ LoopLaunch
         // on an FP64 grid its decision would take the pipe from the others' (200
         // steps of eight states an SM of which one flies on, 17^4: 3.9 ms, 8.9 with
         // the others deciding to the end) ---
-        if (s_live[warp]) {
+        if (s_i[warp][0] != kArrived) {
             G x[4];
 #pragma unroll
             for (int d = 0; d < 4; ++d) {
