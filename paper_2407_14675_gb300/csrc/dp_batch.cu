@@ -182,7 +182,7 @@ __global__ void __launch_bounds__(kBlock) batch_widen_kernel(const BArgs a)
         const BState& S = a.st[t];
         const float* src = pick(a.V32, S.cur) + a.off[t];
         double* dst = pick(a.V64, S.cur64) + a.off[t];
-        for (int j = r.first + threadIdx.x; j < r.end; j += kBlock) dst[j] = (double)src[j];
+        for (unsigned j = r.first + threadIdx.x; j < (unsigned)r.end; j += kBlock) dst[j] = (double)src[j];
     }
 }
 
@@ -219,7 +219,7 @@ __global__ void __launch_bounds__(kBlock, std::is_same<S, double>::value ? 2 : 3
         BState& st = a.st[t];
         const long long o = a.off[t];
         const int first = (it - pre[t]) * a.item_imp;
-        const int end = min(first + a.item_imp, s_g.n_nodes);
+        const int end = (int)min((unsigned)first + (unsigned)a.item_imp, (unsigned)s_g.n_nodes);
         Table<float> T{s_code, s_sc, s_g.K};
         T.fine = s_fine;
         S resid = (S)0;
@@ -448,7 +448,7 @@ __global__ void __launch_bounds__(kCtlThreads) batch_ctl_kernel(const BArgs a, B
             ctl_update(s, P, a.geo[t].M64, stage);
             a.st[t] = s;
             const int n = a.geo[t].n_nodes;
-            const int ne = (n + kShareItem - 1) / kShareItem, ni = (n + a.item_imp - 1) / a.item_imp;
+            const int ne = (n - 1) / kShareItem + 1, ni = (n - 1) / a.item_imp + 1;
             c[kLWiden] = (s.phase == kPh64 && s.widen) ? ne : 0;
             c[kLImp32Full] = (s.phase == kPh32 && s.full_next) ? ni : 0;
             c[kLImp32Walk] = (s.phase == kPh32 && !s.full_next) ? ni : 0;
@@ -728,7 +728,7 @@ int narrow_all(dp_batch* b)
         const BState& s = b->h_st[t];
         if (s.switch_outer < 0) continue;
         const int n = (int)b->nodes[t];
-        narrow_kernel<<<(n + 255) / 256, 256, 0, b->st>>>(b->V64[s.cur64] + b->off[t], b->V32[s.cur] + b->off[t], n);
+        narrow_kernel<<<(n - 1) / 256 + 1, 256, 0, b->st>>>(b->V64[s.cur64] + b->off[t], b->V32[s.cur] + b->off[t], n);
         BCK(cudaGetLastError());
         b->h_st[t].switch_outer = -1;
     }

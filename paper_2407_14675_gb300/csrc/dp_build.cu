@@ -160,8 +160,8 @@ cudaError_t store_value(const H* src, void* dst, int fp32, int n, const Geo<doub
 {
     cudaError_t e = cudaMemsetAsync(bad, 0, sizeof(int), st);
     if (e != cudaSuccess) return e;
-    check_finite_kernel<H><<<(n + 255) / 256, 256, 0, st>>>(src, n, bad);
-    store_value_kernel<H><<<(n + 255) / 256, 256, 0, st>>>(src, dst, fp32, g, bad);
+    check_finite_kernel<H><<<(n - 1) / 256 + 1, 256, 0, st>>>(src, n, bad);
+    store_value_kernel<H><<<(n - 1) / 256 + 1, 256, 0, st>>>(src, dst, fp32, g, bad);
     return cudaGetLastError();
 }
 
@@ -188,13 +188,13 @@ __global__ void load_value_kernel(const void* src, H* dst, int fp32, int n)
 
 cudaError_t launch_load_value(const void* src, double* dst, int fp32, int n, cudaStream_t st)
 {
-    load_value_kernel<double><<<(n + 255) / 256, 256, 0, st>>>(src, dst, fp32, n);
+    load_value_kernel<double><<<(n - 1) / 256 + 1, 256, 0, st>>>(src, dst, fp32, n);
     return cudaGetLastError();
 }
 
 cudaError_t launch_load_value(const void* src, float* dst, int fp32, int n, cudaStream_t st)
 {
-    load_value_kernel<float><<<(n + 255) / 256, 256, 0, st>>>(src, dst, fp32, n);
+    load_value_kernel<float><<<(n - 1) / 256 + 1, 256, 0, st>>>(src, dst, fp32, n);
     return cudaGetLastError();
 }
 
@@ -206,7 +206,7 @@ __global__ void widen_kernel(const float* src, double* dst, int n)
 
 cudaError_t launch_widen(const float* src, double* dst, int n, cudaStream_t st)
 {
-    widen_kernel<<<(n + 255) / 256, 256, 0, st>>>(src, dst, n);
+    widen_kernel<<<(n - 1) / 256 + 1, 256, 0, st>>>(src, dst, n);
     return cudaGetLastError();
 }
 
@@ -331,7 +331,7 @@ __global__ void box_index_kernel(Geo<double> g, long long* out)
 
 cudaError_t launch_box_index(const Geo<double>& g, long long* out, cudaStream_t st)
 {
-    box_index_kernel<<<(g.n_nodes + 255) / 256, 256, 0, st>>>(g, out);
+    box_index_kernel<<<(g.n_nodes - 1) / 256 + 1, 256, 0, st>>>(g, out);
     return cudaGetLastError();
 }
 

@@ -322,10 +322,10 @@ gm_matvec_kernel(const __grid_constant__ Geo<G> g, VT* __restrict__ Q, long long
     const VT* x = Q + (size_t)k * ldq;
     VT* w = Q + (size_t)(k + 1) * ldq;
     const VT sk = (VT)gc->scale[k];
-    const int n = g.n_nodes;
-    const int stride = gridDim.x * kGmBlock;
+    // without a sign: a node and the stride after it may pass 2^31 together
+    const unsigned n = (unsigned)g.n_nodes, stride = gridDim.x * kGmBlock;
     if constexpr (std::is_same<G, float>::value) {
-        int j = blockIdx.x * kGmBlock + threadIdx.x;
+        unsigned j = blockIdx.x * kGmBlock + threadIdx.x;
         if (feet_hi) {
             // the word pair of the FP64-value phase
             FootWord next{0ull, 0u};
@@ -333,7 +333,7 @@ gm_matvec_kernel(const __grid_constant__ Geo<G> g, VT* __restrict__ Q, long long
             for (; j < n; j += stride) {
                 const FootWord fw = next;
                 if (j + stride < n) next = FootWord{__ldcs(&feet_lo[j + stride]), __ldcs(&feet_hi[j + stride])};
-                w[j] = sk * apply_a_feet<REDUCED, DYN>(g, x, j, fw, code);
+                w[j] = sk * apply_a_feet<REDUCED, DYN>(g, x, (int)j, fw, code);
             }
         } else {
             // 8-byte feet of the FP32-value phase
@@ -342,15 +342,15 @@ gm_matvec_kernel(const __grid_constant__ Geo<G> g, VT* __restrict__ Q, long long
             for (; j < n; j += stride) {
                 const unsigned long long fw = next;
                 if (j + stride < n) next = __ldcs(&feet_lo[j + stride]);
-                w[j] = sk * apply_a_feet<REDUCED, DYN>(g, x, j, fw, code);
+                w[j] = sk * apply_a_feet<REDUCED, DYN>(g, x, (int)j, fw, code);
             }
         }
     } else if (f64.w) {
-        for (int j = blockIdx.x * kGmBlock + threadIdx.x; j < n; j += stride)
-            w[j] = sk * apply_a_feet64<REDUCED, DYN>(g, x, j, f64, code);
+        for (unsigned j = blockIdx.x * kGmBlock + threadIdx.x; j < n; j += stride)
+            w[j] = sk * apply_a_feet64<REDUCED, DYN>(g, x, (int)j, f64, code);
     } else {
-        for (int j = blockIdx.x * kGmBlock + threadIdx.x; j < n; j += stride)
-            w[j] = sk * apply_a_node<REDUCED, DYN>(g, x, j, code);
+        for (unsigned j = blockIdx.x * kGmBlock + threadIdx.x; j < n; j += stride)
+            w[j] = sk * apply_a_node<REDUCED, DYN>(g, x, (int)j, code);
     }
 }
 
@@ -616,7 +616,8 @@ __global__ void __launch_bounds__(kGmBlock)
 feet_kernel(const __grid_constant__ Geo<float> g, const uint16_t* __restrict__ code,
             unsigned long long* __restrict__ feet_lo, unsigned* __restrict__ feet_hi)
 {
-    for (int j = blockIdx.x * kGmBlock + threadIdx.x; j < g.n_nodes; j += gridDim.x * kGmBlock) {
+    for (unsigned ju = blockIdx.x * kGmBlock + threadIdx.x; ju < (unsigned)g.n_nodes; ju += gridDim.x * kGmBlock) {
+        const int j = (int)ju;
         CachedEval<float, float, REDUCED, DYN, float, false> ev;
         decode_node(g, j, ev.i);
         const bool target = in_target(g, ev.i);

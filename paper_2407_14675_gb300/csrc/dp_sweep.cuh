@@ -283,7 +283,9 @@ __device__ __forceinline__ int cell_reach(const Geo<float>& g, int j, const int 
 // every sweep mode.  Folds max |V_out - V_in| into resid and non-finite
 // results into bad.  The modes kEvalFeet64* also deal out the last round by
 // block and thread indices: they are for the whole launch of sweep_kernel only
-// (j0 the thread's index in the grid, stride the grid's threads).
+// (j0 the thread's index in the grid, stride the grid's threads).  The others
+// step without a sign: a node and the stride after it are below 2^31 each, their
+// sum is not, on grids of more than 2^30 nodes whose launch has a thread a node.
 template <typename G, typename S, int MODE, bool REDUCED, int DYN, bool PREFETCH = true, bool SMALL = false>
 __device__ __forceinline__ void sweep_nodes(const Geo<G>& g, const Table<G>& T, const S* __restrict__ Vin,
                                             S* __restrict__ Vout, uint16_t* __restrict__ code,
@@ -398,15 +400,16 @@ __device__ __forceinline__ void sweep_nodes(const Geo<G>& g, const Table<G>& T, 
             w_next = load_foot(j);
             v_next = *at_node<SMALL>(Vin, j);
         }
-        for (; j < end; j += stride) {
+        for (unsigned jn; (unsigned)j < (unsigned)end; j = (int)jn) {
             FW w;
             S vj;
+            jn = (unsigned)j + (unsigned)stride;
             if constexpr (kPrefetch) {
                 w = w_next;
                 vj = v_next;
-                if (j + stride < end) {
-                    w_next = load_foot(j + stride);
-                    v_next = *at_node<SMALL>(Vin, j + stride);
+                if (jn < (unsigned)end) {
+                    w_next = load_foot((int)jn);
+                    v_next = *at_node<SMALL>(Vin, (int)jn);
                 }
             } else {
                 w = load_foot(j);
@@ -467,7 +470,8 @@ __device__ __forceinline__ void sweep_nodes(const Geo<G>& g, const Table<G>& T, 
         typedef typename std::conditional<kPolish, float, typename BlendType<G, S>::type>::type SearchR;
         typedef typename std::conditional<kSearch, CachedEval<G, S, REDUCED, DYN, SearchR, false, MODE == kVIDiag>,
                                           NodeEval<G, S, REDUCED, DYN>>::type Eval;
-        for (int j = j0; j < end; j += stride) {
+        for (unsigned ju = (unsigned)j0; ju < (unsigned)end; ju += (unsigned)stride) {
+            const int j = (int)ju;
             const S vj = Vin[j];
             S vnew = (S)0;
             double vnew64 = 0.0;
@@ -808,7 +812,7 @@ sweep_kernel(const __grid_constant__ Geo<G> g, const S* __restrict__ Vin, S* __r
     S resid = (S)0;
     bool bad = false;
     constexpr int B = sweep_block<G, S, MODE, REDUCED, BIG>();
-    const int j0 = blockIdx.x * B + threadIdx.x, end = g.n_nodes, stride = gridDim.x * B;
+    const int j0 = blockIdx.x * B + threadIdx.x, end = g.n_nodes, stride = (int)(gridDim.x * B);
     constexpr bool kReach = std::is_same<G, float>::value && (MODE == kImproveFull || MODE == kImproveWalk);
     int reach = 0;
     sweep_nodes<G, S, MODE, REDUCED, DYN, eval_prefetch<MODE, REDUCED>(), SMALL>(

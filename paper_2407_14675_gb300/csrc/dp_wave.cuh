@@ -63,7 +63,7 @@ struct WaveSched {
 __device__ __forceinline__ WaveSched wave_sched(int n_nodes, int levels, int reach, int blocks)
 {
     WaveSched S;
-    S.nC = (n_nodes + kWaveChunk - 1) / kWaveChunk;
+    S.nC = (n_nodes - 1) / kWaveChunk + 1;
     S.levels = levels;
     const long long R = reach > 0 ? reach : n_nodes;
     S.Dr = (int)min((R + kWaveChunk - 1) / kWaveChunk, (long long)S.nC);
@@ -235,11 +235,12 @@ __global__ void __launch_bounds__(kWaveBlock, 3) wave_kernel(const __grid_consta
         float* Vout = a.V[(a.in0 + lev + 1) & 1];
         const int e = a.e0 + lev;
         const bool first = kInc && e == 0, last = kInc && e == a.ne - 1;
-        const int j_end = min((c + 1) * kWaveChunk, g.n_nodes);
+        const unsigned j_end = min((unsigned)(c + 1) * kWaveChunk, (unsigned)g.n_nodes);
         float resid = 0.0f;
         bool bad = false;
 #pragma unroll 1
-        for (int j = c * kWaveChunk + threadIdx.x; j < j_end; j += kWaveBlock) {
+        for (unsigned ju = (unsigned)c * kWaveChunk + threadIdx.x; ju < j_end; ju += kWaveBlock) {
+            const int j = (int)ju;
             // plain evaluation: 8-byte feet; diagonal-solved evaluation and
             // increments: the word pair
             constexpr bool kF8 = MODE == kEvalFeet8;
@@ -320,7 +321,7 @@ cudaError_t launch_wave_mode(const WaveArgs& a, cudaStream_t st, int sm_count)
         if (e != cudaSuccess) return e;
         if (per_sm < 1) per_sm = 1;
     }
-    const long long chunks = (long long)a.levels * ((a.g.n_nodes + kWaveChunk - 1) / kWaveChunk);
+    const long long chunks = (long long)a.levels * ((a.g.n_nodes - 1) / kWaveChunk + 1);
     const long long blocks = std::min<long long>((long long)per_sm * sm_count, chunks);
     cudaError_t e = cudaMemsetAsync(a.sync, 0, wave_sync_ints(a.levels, a.g.n_nodes) * sizeof(int), st);
     if (e != cudaSuccess) return e;
