@@ -59,10 +59,10 @@
 // series, 0.15 of the noise.
 //
 // Measured (GB300, with one-round blocks of 64): a value-iteration sweep of
-// 17^4, 16 angles, 50 us, evaluating every angle 166; a walk sweep of a
-// 31x41x25x17 box 0.34 against 1.17 ms, of the paper's 110x30^3 2.3 against 9.9
-// ms.  Before the one-step map's shared parts came from tables
-// (node_dyn_table()) 78 us, 0.48 and 6.1 ms.
+// 17^4, 16 angles, 56 us (60 in a call of 50 sweeps, with its start and end),
+// evaluating every angle 166; a walk sweep of a 31x41x25x17 box 0.33 against
+// 1.17 ms, of the paper's 110x30^3 1.9 against 9.9 ms.  Before the one-step map's
+// shared parts came from tables (node_dyn_table()) 78 us, 0.48 and 6.1 ms.
 #pragma once
 
 #include "dp_device.cuh"
