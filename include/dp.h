@@ -23,7 +23,9 @@
  *   - Host pointers are owned by the caller and only read or written during
  *     the call; the library copies in and out and keeps no reference.
  *   - The library owns all device memory of a grid (allocated by
- *     dp_grid_create and by the first FP64 polish, freed by dp_grid_destroy).
+ *     dp_grid_create, by the first FP64 polish and GMRES evaluation, and on
+ *     FP64 grids by the first diagonal-solved evaluation, which does without
+ *     where there is none; freed by dp_grid_destroy).
  *   - All GPU work of a grid is issued on desc.stream (NULL: the legacy
  *     default stream) on the device that was current at dp_grid_create; calls
  *     that return host data synchronise that stream.
